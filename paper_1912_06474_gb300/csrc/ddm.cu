@@ -19,7 +19,7 @@
 // The closest hit found this way is the global closest hit (up to eps), so
 // the estimator is the same one the megakernel computes (Sec. 4 algorithm,
 // Eq. 2-3); shading is split into a per-bounce kernel over path slots whose
-// spectral throughput lives in HBM as [L][paths].
+// spectral throughput lives in HBM as one row of bins per path.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -77,7 +77,7 @@ struct KArgs {
     int64_t q_cap;
     int *pend_query;      // [np]
     int *cross_query;     // [kMaxCross][np]
-    const float2 *glass_res;
+    const float *glass_res;   // [query][2][Lp]: R, then T
     int *block_cnt;       // [gridDim] glass queries per block of path slots (count pass)
     PhotonGridView pm;    // photon map: gather at the first diffuse vertex, no continuation there
     PhotonGridView pmc;   // caustic map gathered with it (pmc.on)
@@ -232,7 +232,6 @@ __device__ __forceinline__ void block_bins_flush(const Queues &Q, const int *bin
 // --------------------------------------------------------- camera rays
 __global__ void __launch_bounds__(256) k_camera(KArgs a) {
     const int64_t np = a.ps.np;
-    const int L = a.sc.L;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     unsigned long long n_ext = 0;
     __shared__ PushSmem psm;
@@ -253,7 +252,6 @@ __global__ void __launch_bounds__(256) k_camera(KArgs a) {
             uint4 x = philox4x32_10(make_uint4(p, j, 0u, kSlotCamera), ri.seed, ri.render_id);
             V3 o, d;
             camera_ray(ri, (float)px + u01(x.x), (float)py + u01(x.y), o, d);
-            for (int i = 0; i < L; ++i) a.ps.T[(size_t)i * np + q] = 1.0f;
 #pragma unroll
             for (int k = 0; k < 6; ++k) a.ps.acc[k * np + q] = 0.0f;
             a.ps.flags[q] = kFlExt | kFlPrevSpec;
@@ -505,159 +503,287 @@ __global__ void __launch_bounds__(256) k_glass_gather(KArgs a) {
 
 // Spectral half of shading: resolve the previous vertex's shadow ray, apply its
 // weight, add this vertex's emission, per bin, with compensated sums.
-#ifndef SDDM_SHS_MINB
-#define SDDM_SHS_MINB 6      // resident 256-thread blocks per SM the spectral pass is compiled for (40
-                             // registers with some spills: 48 warps hide the per-bin load latency; +1.7%
-                             // on the hotel bench against 4 blocks, 8 blocks -1.6%)
-#endif
-#ifndef SDDM_SHS_UNROLL
-#define SDDM_SHS_UNROLL 2    // bins in flight per thread (8: -6%)
-#endif
-constexpr int kShsUnroll = SDDM_SHS_UNROLL;
+//
+// A warp takes 32 consecutive path slots in three phases. (1) A lane per path
+// reads the path's state and packs what its bins need into a 64-byte record in
+// shared memory; paths with nothing to do leave none. (2) The records' rows, cut
+// into chunks of four bins, are dealt out to the lanes one chunk at a time, so
+// every lane has work whatever L and however few paths live, the row moves in
+// 16-byte accesses of neighbouring lanes, and lanes side by side mostly share a
+// record's branch; the rows of a pass are all fetched at once (cp.async) before
+// the first is used, and a chunk's XYZ takes its row chunk's place in shared
+// memory. (3) A lane per path adds its chunks in bin order with compensation and
+// updates the path's accumulator.
+// The bound is the row traffic (2 x 176 B per live path at L = 41). A row is not
+// read before a weight has been applied to it (up to the second vertex the
+// throughput is 1) nor written once the path has ended.
+// All bounces of the hotel room (512 x 512 x 16 spp, 41 bins): 1.9 ms, against
+// 4.5 ms with a thread walking its path's bins down a column of an [L][paths]
+// array; of a facade room (960 x 540 x 4 spp, 81 bins) 4.3 ms against 9.7. It is
+// now bound by issue (60 % of the slots) and by the L1 it shares with the table rows.
+struct SpecRec {
+    int q, flags;         // path slot; kSr* bits
+    float G;              // geometry factor of the shadow ray
+    int r_rho, r_le;      // table rows: reflectance at its vertex, radiance of its light
+    int r_w, r_w2;        // table rows of the pending weight (n, k of a conductor)
+    float pcos, pw;       // pending |cos|, branch weight
+    int pq;               // glass query of the pending weight (-1: none)
+    int r_emit;           // table row of the emitter hit
+    int ncr;              // slabs the shadow ray crossed
+    int cq[kMaxCross];    // their glass queries (-1: none)
+};
+static_assert(sizeof(SpecRec) == 64, "four 16-byte loads");
+constexpr int kSrResolve = 1, kSrEmit = 2, kSrLoad = 4, kSrStore = 8, kSrRow = 16, kSrConductor = 32, kSrGlass = 64,
+              kSrDirect = 128;   // a glass evaluation the query list had no room for
+constexpr int kSpecThreads = 128;
+constexpr int kSpecItems = 192;  // chunks a warp works through between two sums (at least 3 records at L = 256)
+
+struct Float4 {
+    float v[4];
+};
+__device__ __forceinline__ Float4 ld4(const float4 *p) {
+    const float4 x = __ldg(p);
+    return Float4{{x.x, x.y, x.z, x.w}};
+}
+
+// One chunk of a record: the XYZ it adds (bins past L have a zero colour
+// matching function), the row's four bins updated. DIRECT also evaluates the
+// glass that has no query; that variant stays out of line: with it in the loop
+// every warp runs, instruction cache misses cost three times the pass (518
+// against 163 us, hotel room 256 x 256 x 16 spp, bounce 3).
+template <bool FILMS, bool DIRECT>
+__device__ __forceinline__ float3 spec_chunk(const KArgs &a, const SpecRec &rec, int ch, const float4 &tin) {
+    const DevScene &sc = a.sc;
+    const PathState &ps = a.ps;
+    const int L = sc.L, n_chunk = sc.Lp >> 2, xf = rec.flags, q = rec.q;
+    const float4 *const tab = reinterpret_cast<const float4 *>(sc.tab) + ch;
+    const float4 *const res = reinterpret_cast<const float4 *>(a.glass_res) + ch;
+    Float4 t{{1.f, 1.f, 1.f, 1.f}}, e{{0.f, 0.f, 0.f, 0.f}};
+    if (xf & kSrLoad) t = Float4{{tin.x, tin.y, tin.z, tin.w}};
+    auto direct = [&](int m, float c, int u, bool want_r) {
+        float R_, T_;
+        glass_rt<FILMS>(sc, m, min(4 * ch + u, L - 1), c, st_of(a.rb, find_render(a.rb, a.path_begin + q), m, sc.n_mat),
+                        __ldg(sc.mat_thick + m), R_, T_);
+        return want_r ? R_ : T_;
+    };
+    if (xf & kSrResolve) {
+        const Float4 rho = ld4(tab + rec.r_rho * n_chunk), le = ld4(tab + rec.r_le * n_chunk);
+        const float G = rec.G;
+        Float4 tr{{1.f, 1.f, 1.f, 1.f}};
+        for (int k = 0; k < rec.ncr; ++k) {
+            const int cq = rec.cq[k];
+            if (!DIRECT || cq >= 0) {
+                const Float4 v = ld4(res + ((size_t)cq * 2 + 1) * n_chunk);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) tr.v[u] *= v.v[u];
+            } else if (DIRECT) {
+                const int cm = ps.cross_mat[k * ps.np + q];
+                const float cc = ps.cross_cos[k * ps.np + q];
+#pragma unroll 1
+                for (int u = 0; u < 4; ++u) tr.v[u] *= direct(cm, cc, u, false);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) e.v[u] = t.v[u] * rho.v[u] * le.v[u] * G * tr.v[u];
+    }
+    if (xf & kSrRow) {
+        const Float4 w = ld4(tab + rec.r_w * n_chunk);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) t.v[u] *= w.v[u];
+    } else if (xf & kSrConductor) {
+        const Float4 n = ld4(tab + rec.r_w * n_chunk), k = ld4(tab + rec.r_w2 * n_chunk);
+        const float c = rec.pcos;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) t.v[u] *= conductor_F(c, n.v[u], k.v[u]);
+    } else if (xf & kSrGlass) {
+        const float pwabs = fabsf(rec.pw);
+        const bool refl = rec.pw < 0.0f;
+        if (!DIRECT || rec.pq >= 0) {
+            const Float4 v = ld4(res + ((size_t)rec.pq * 2 + (refl ? 0 : 1)) * n_chunk);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) t.v[u] *= v.v[u] * pwabs;
+        } else if (DIRECT) {
+#pragma unroll 1
+            for (int u = 0; u < 4; ++u) t.v[u] *= direct(rec.r_w, rec.pcos, u, refl) * pwabs;
+        }
+    }
+    // A resolved shadow ray and emission exclude each other: the first follows a
+    // diffuse vertex under next-event estimation, after which the second does not count.
+    if (xf & kSrEmit) {
+        const Float4 le = ld4(tab + rec.r_emit * n_chunk);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) e.v[u] = t.v[u] * le.v[u];
+    }
+    float3 s = make_float3(0.f, 0.f, 0.f);
+    if (xf & (kSrResolve | kSrEmit)) {
+        const float4 *const w = tab + 2 * sc.n_mat * n_chunk;
+        const Float4 wx = ld4(w), wy = ld4(w + n_chunk), wz = ld4(w + 2 * n_chunk);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            s.x = fmaf(e.v[u], wx.v[u], s.x);
+            s.y = fmaf(e.v[u], wy.v[u], s.y);
+            s.z = fmaf(e.v[u], wz.v[u], s.z);
+        }
+    }
+    if (xf & kSrStore)
+        reinterpret_cast<float4 *>(ps.T)[(size_t)q * n_chunk + ch] = make_float4(t.v[0], t.v[1], t.v[2], t.v[3]);
+    return s;
+}
+
+// The chunks of a warp's records, dealt to its lanes.
+template <bool FILMS, bool DIRECT>
+__device__ __forceinline__ void spec_items(const KArgs &a, const SpecRec *rec, float4 *part, int n_item, int n_chunk,
+                                           unsigned inv_chunk) {
+    const int lane = threadIdx.x & 31;
+    for (int i = lane; i < n_item; i += 32) {
+        const int j = (int)((unsigned)i * inv_chunk >> 16);
+        if (rec[j].flags & kSrLoad)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(part + i)),
+                         "l"(reinterpret_cast<const float4 *>(a.ps.T) + (size_t)rec[j].q * n_chunk + i - j * n_chunk)
+                         : "memory");
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");   // a lane reads only what it fetched itself
+    for (int i = lane; i < n_item; i += 32) {
+        const int j = (int)((unsigned)i * inv_chunk >> 16);
+        const float3 s = spec_chunk<FILMS, DIRECT>(a, rec[j], i - j * n_chunk, part[i]);
+        part[i] = make_float4(s.x, s.y, s.z, 0.0f);
+    }
+}
 template <bool FILMS>
-__global__ void __launch_bounds__(256, SDDM_SHS_MINB) k_shade_spectral(KArgs a) {
+static __device__ __noinline__ void spec_items_direct(const KArgs &a, const SpecRec *rec, float4 *part, int n_item,
+                                                      int n_chunk, unsigned inv_chunk) {
+    spec_items<FILMS, true>(a, rec, part, n_item, n_chunk, inv_chunk);
+}
+
+#ifndef SDDM_SHS_MINB
+#define SDDM_SHS_MINB 8      // resident 128-thread blocks per SM the spectral pass is compiled for
+#endif
+template <bool FILMS>
+__global__ void __launch_bounds__(kSpecThreads, SDDM_SHS_MINB) k_shade_spectral(const __grid_constant__ KArgs a) {
+    __shared__ __align__(16) SpecRec s_rec[kSpecThreads];
+    __shared__ __align__(16) float4 s_part[kSpecThreads / 32][kSpecItems];
     const int64_t np = a.ps.np;
     const DevScene &sc = a.sc;
-    const int L = sc.L;
+    const int n_chunk = sc.Lp >> 2, M = sc.n_mat;
     const int b = a.b;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    SpecRec *const rec = s_rec + (threadIdx.x & ~31);
+    float4 *const part = s_part[threadIdx.x >> 5];
+    const int per_pass = min(32, kSpecItems / n_chunk);        // records summed at a time
+    const unsigned inv_chunk = 65536u / (unsigned)n_chunk + 1u;   // i / n_chunk = i inv >> 16 for i < kSpecItems
     unsigned long long n_glass = 0;
     const PathState &ps = a.ps;
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < np; base += stride) {   // block-uniform trips
         const int64_t q = base + threadIdx.x;
-        int fl = q < np ? ps.flags[q] : 0;
+        const int fl = q < np ? ps.flags[q] : 0;
+        SpecRec me;
+        me.flags = 0;
         if (fl & (kFlExt | kFlShadow)) {
-            const int64_t gp = a.path_begin + q;
-            const int r = find_render(a.rb, gp);
-            const RenderInfo &ri = a.rb.info[r];
-
-            // (1) shadow ray of the previous vertex
-            bool resolve = false;
-            float G = 0.f;
-            const float *rho_prev = nullptr, *Le_l = nullptr;
-            int ncr = 0;
-            int cmat[kMaxCross];
-            float ccos[kMaxCross];
+            me.q = (int)q;
+            me.ncr = 0;
+            me.pq = -1;
+            me.G = me.pcos = me.pw = 0.f;
+            me.r_rho = me.r_le = me.r_w = me.r_w2 = me.r_emit = 0;
+            int pm = 0, pkind = 0;
+            if (fl & (kFlPend | kFlShadow)) {
+                pm = ps.pend_mat[q];
+                pkind = __ldg(sc.mat_kind + pm);
+            }
+            // shadow ray of the previous vertex
             if (fl & kFlShadow) {
                 const int stt = ps.sh_status[q];
                 if ((stt & 3) == kShadowClear) {
-                    resolve = true;
-                    ncr = stt >> 4;
-                    G = ps.nee_G[q];
-                    Le_l = sc.mat_a + (size_t)ps.nee_lmat[q] * L;
-                    const int pm = ps.pend_mat[q];
-                    rho_prev = (__ldg(sc.mat_kind + pm) == kLambert ? sc.mat_a : sc.mat_b) + (size_t)pm * L;
-                    for (int k = 0; k < ncr; ++k) {
-                        cmat[k] = ps.cross_mat[k * np + q];
-                        ccos[k] = ps.cross_cos[k * np + q];
-                    }
-                    n_glass += ncr;
-                }
-            }
-            // (2) weight of the previous vertex
-            const bool pend = (fl & kFlPend) != 0;
-            int pm = -1, pkind = 0;
-            float pcos = 0.f, pw = 0.f;
-            if (pend) {
-                pm = ps.pend_mat[q];
-                pkind = __ldg(sc.mat_kind + pm);
-                pcos = ps.pend_cos[q];
-                pw = ps.pend_w[q];
-            }
-            // (3) the hit of this vertex
-            bool emit = false;
-            int prim = -1, mat = 0, kind = 0;
-            V3 d = v3(0, 0, 0), ng = d;
-            float cd = 0.f;
-            if ((fl & kFlExt) && b <= ri.max_depth) {
-                const float4 h0 = ps.hit0[q], h1 = ps.hit1[q];
-                prim = __float_as_int(h0.w);
-                if (prim >= 0) {
-                    d = xyz(h1);
-                    const float4 tn = __ldg(sc.tri_n + prim);
-                    ng = xyz(tn);
-                    mat = __float_as_int(tn.w);
-                    kind = __ldg(sc.mat_kind + mat);
-                    cd = dot(d, ng);
-                    emit = (kind == kEmitter || kind == kDiffuseEmitter) && cd < 0.0f &&
-                           (!ri.nee || b == 1 || (fl & kFlPrevSpec));
-                }
-            }
-            // spectral pass over the bins: resolve, weight, emit
-            const float *Le_b = sc.mat_a + (size_t)mat * L;
-            const float *pA = sc.mat_a + (size_t)(pm < 0 ? 0 : pm) * L;
-            const float *pB = sc.mat_b + (size_t)(pm < 0 ? 0 : pm) * L;
-            const float ps_state = (pend && pkind == kGlass) ? st_of(a.rb, r, pm, sc.n_mat) : 0.f;
-            const float pthick = (pend && pkind == kGlass) ? __ldg(sc.mat_thick + pm) : 0.f;
-            const float pwabs = fabsf(pw);
-            const bool preflect = pw < 0.0f;
-            float cst[kMaxCross], cth[kMaxCross];
-            int cq[kMaxCross];
-            for (int k = 0; k < ncr; ++k) {
-                cst[k] = st_of(a.rb, r, cmat[k], sc.n_mat);
-                cth[k] = __ldg(sc.mat_thick + cmat[k]);
-                cq[k] = a.use_queries ? a.cross_query[k * np + q] : -1;
-            }
-            const int pq = (a.use_queries && pend && pkind == kGlass) ? a.pend_query[q] : -1;
-            const bool need_T = resolve || pend || emit;
-            if (need_T) {
-                Kahan NX, NY, NZ, EX, EY, EZ;
-#pragma unroll kShsUnroll
-                for (int i = 0; i < L; ++i) {
-                    float t = ps.T[(size_t)i * np + q];
-                    const float4 w4 = __ldg(sc.wcmf + i);
-                    const float wx = w4.x, wy = w4.y, wz = w4.z;
-                    if (resolve) {
-                        float tr = 1.0f;
-                        for (int k = 0; k < ncr; ++k) {
-                            if (cq[k] >= 0) {
-                                tr *= a.glass_res[(size_t)cq[k] * L + i].y;
-                                continue;
-                            }
-                            float R_, T_;
-                            glass_rt<FILMS>(sc, cmat[k], i, ccos[k], cst[k], cth[k], R_, T_);
-                            tr *= T_;
+                    me.flags |= kSrResolve;
+                    me.ncr = stt >> 4;
+                    me.G = ps.nee_G[q];
+                    me.r_le = ps.nee_lmat[q];
+                    me.r_rho = pkind == kLambert ? pm : M + pm;
+#pragma unroll
+                    for (int k = 0; k < kMaxCross; ++k)
+                        if (k < me.ncr) {
+                            me.cq[k] = a.use_queries ? a.cross_query[k * np + q] : -1;
+                            if (me.cq[k] < 0) me.flags |= kSrDirect;
                         }
-                        const float c = t * __ldg(rho_prev + i) * __ldg(Le_l + i) * G * tr;
-                        NX.add(c * wx);
-                        NY.add(c * wy);
-                        NZ.add(c * wz);
-                    }
-                    if (pend) {
-                        float w;
-                        if (pkind == kLambert) {
-                            w = __ldg(pA + i);
-                        } else if (pkind == kDiffuseEmitter) {
-                            w = __ldg(pB + i);
-                        } else if (pkind == kConductor) {
-                            w = conductor_F(pcos, __ldg(pA + i), __ldg(pB + i));
-                        } else if (pq >= 0) {
-                            const float2 rt = a.glass_res[(size_t)pq * L + i];
-                            w = (preflect ? rt.x : rt.y) * pwabs;
-                        } else {
-                            float R_, T_;
-                            glass_rt<FILMS>(sc, pm, i, pcos, ps_state, pthick, R_, T_);
-                            w = (preflect ? R_ : T_) * pwabs;
-                        }
-                        t *= w;
-                    }
-                    if (emit) {
-                        const float e = t * __ldg(Le_b + i);
-                        EX.add(e * wx);
-                        EY.add(e * wy);
-                        EZ.add(e * wz);
-                    }
-                    ps.T[(size_t)i * np + q] = t;
+                    n_glass += me.ncr;
                 }
-                Kahan3 acc;
+            }
+            // weight of the previous vertex
+            if (fl & kFlPend) {
+                if (pkind == kLambert || pkind == kDiffuseEmitter) {
+                    me.flags |= kSrRow;
+                    me.r_w = pkind == kLambert ? pm : M + pm;
+                } else {
+                    me.pcos = ps.pend_cos[q];
+                    me.r_w = pm;
+                    me.r_w2 = M + pm;
+                    if (pkind == kConductor) {
+                        me.flags |= kSrConductor;
+                    } else {
+                        me.flags |= kSrGlass;
+                        me.pw = ps.pend_w[q];
+                        me.pq = a.use_queries ? a.pend_query[q] : -1;
+                        if (me.pq < 0) me.flags |= kSrDirect;
+                    }
+                }
+            }
+            // the hit of this vertex: emission, and whether the path goes on from here
+            bool on = false;
+            if (fl & kFlExt) {
+                const RenderInfo &ri = a.rb.info[find_render(a.rb, a.path_begin + q)];
+                if (b <= ri.max_depth) {
+                    const int prim = __float_as_int(ps.hit0[q].w);
+                    if (prim >= 0) {
+                        const float4 tn = __ldg(sc.tri_n + prim);
+                        const int mat = __float_as_int(tn.w);
+                        const int kind = __ldg(sc.mat_kind + mat);
+                        if ((kind == kEmitter || kind == kDiffuseEmitter) &&
+                            (!ri.nee || b == 1 || (fl & kFlPrevSpec)) && dot(xyz(ps.hit1[q]), xyz(tn)) < 0.0f) {
+                            me.flags |= kSrEmit;
+                            me.r_emit = mat;
+                        }
+                        on = kind != kEmitter && (b < ri.max_depth || kind == kLambert || kind == kDiffuseEmitter);
+                    }
+                }
+            }
+            constexpr int kWeight = kSrRow | kSrConductor | kSrGlass;
+            if (on && (me.flags & kWeight)) me.flags |= kSrStore;
+            // an ended path's weight reaches nothing but its own emission
+            if (!on && !(me.flags & kSrEmit)) me.flags &= ~kWeight;
+            if (!(me.flags & (kSrResolve | kSrEmit | kSrStore))) me.flags = 0;
+            if (me.flags && b >= 3) me.flags |= kSrLoad;
+        }
+        const unsigned work = __ballot_sync(full, me.flags != 0);
+        const int n_rec = __popc(work), mine = __popc(work & ((1u << lane) - 1u));
+        const bool any_direct = __any_sync(full, me.flags & kSrDirect);
+        if (me.flags) rec[mine] = me;
+        __syncwarp();
+        for (int r0 = 0; r0 < n_rec; r0 += per_pass) {
+            const int nr = min(per_pass, n_rec - r0), n_item = nr * n_chunk;
+            if (!any_direct)
+                spec_items<FILMS, false>(a, rec + r0, part, n_item, n_chunk, inv_chunk);
+            else
+                spec_items_direct<FILMS>(a, rec + r0, part, n_item, n_chunk, inv_chunk);
+            __syncwarp();
+            const int j = mine - r0;
+            if ((me.flags & (kSrResolve | kSrEmit)) && j >= 0 && j < nr) {
+                Kahan3 sum, acc;
+                const float4 *p = part + j * n_chunk;
+                for (int c = 0; c < n_chunk; ++c) {
+                    const float4 v = p[c];
+                    sum.add(v.x, v.y, v.z);
+                }
                 acc.x.s = ps.acc[0 * np + q];
                 acc.y.s = ps.acc[1 * np + q];
                 acc.z.s = ps.acc[2 * np + q];
                 acc.x.c = ps.acc[3 * np + q];
                 acc.y.c = ps.acc[4 * np + q];
                 acc.z.c = ps.acc[5 * np + q];
-                if (resolve) acc.add(NX.s, NY.s, NZ.s);
-                if (emit) acc.add(EX.s, EY.s, EZ.s);
+                acc.x.c += sum.x.c;   // what the chunk sums lost goes on to the path's sum
+                acc.y.c += sum.y.c;
+                acc.z.c += sum.z.c;
+                acc.add(sum.x.s, sum.y.s, sum.z.s);
                 ps.acc[0 * np + q] = acc.x.s;
                 ps.acc[1 * np + q] = acc.y.s;
                 ps.acc[2 * np + q] = acc.z.s;
@@ -665,6 +791,7 @@ __global__ void __launch_bounds__(256, SDDM_SHS_MINB) k_shade_spectral(KArgs a) 
                 ps.acc[4 * np + q] = acc.y.c;
                 ps.acc[5 * np + q] = acc.z.c;
             }
+            __syncwarp();   // the next pass rewrites the partial sums, the next trip the records
         }
     }
     // counted per warp (no block barrier at the end: warps whose paths had less
@@ -891,7 +1018,6 @@ int ddm_trace_chunk_pm(const DDMRun &run, const PhotonGridView &pm, const Photon
 static int trace_chunk(const DDMRun &run, const PhotonGridView &pmv, const PhotonGridView &pmcv, DDMBuffers &buf,
                        cudaStream_t s) {
     const int64_t np = run.path_count;
-    const int L = run.sc.L;
     const int nc = run.g.n_cells, nb = run.g.n_bins;
     if (nc > kMaxCells || nb > kMaxBins) {
         set_error("sddm_render: the DDM method supports at most 2048 subdomains");
@@ -905,7 +1031,7 @@ static int trace_chunk(const DDMRun &run, const PhotonGridView &pmv, const Photo
         off = align_up(off + bytes);
         return o;
     };
-    const size_t oT = take(sizeof(float) * (size_t)L * np), oAcc = take(sizeof(float) * 6 * np),
+    const size_t oT = take(sizeof(float) * (size_t)run.sc.Lp * np), oAcc = take(sizeof(float) * 6 * np),
                  oFl = take(4 * np), oPm = take(4 * np), oPc = take(4 * np), oPw = take(4 * np), oG = take(4 * np),
                  oLm = take(4 * np), oSh = take(4 * np), oCo = take(4 * kMaxCross * np), oCm = take(4 * kMaxCross * np),
                  oCc = take(4 * kMaxCross * np), oH0 = take(16 * np), oH1 = take(16 * np), oIn = take(48 * cap),
@@ -919,7 +1045,7 @@ static int trace_chunk(const DDMRun &run, const PhotonGridView &pmv, const Photo
     const int sm = std::max(1, run.sm_count);
     const unsigned path_blocks = (unsigned)std::min<int64_t>((np + 255) / 256, (int64_t)sm * 16);
     const size_t oQ = take(16 * (size_t)q_cap + 16), oNq = take(16), oPq = take(use_queries ? 4 * np : 4),
-                 oCq = take(use_queries ? 4 * kMaxCross * np : 4), oRes = take(8 * (size_t)q_cap * L + 16),
+                 oCq = take(use_queries ? 4 * kMaxCross * np : 4), oRes = take(8 * (size_t)q_cap * run.sc.Lp + 16),
                  oBc = take(4 * (size_t)path_blocks + 16);
     if (off > buf.bytes) {
         if (buf.mem) cudaFree(buf.mem);
@@ -973,7 +1099,7 @@ static int trace_chunk(const DDMRun &run, const PhotonGridView &pmv, const Photo
     a.q_cap = q_cap;
     a.pend_query = (int *)(m + oPq);
     a.cross_query = (int *)(m + oCq);
-    a.glass_res = (const float2 *)(m + oRes);
+    a.glass_res = (const float *)(m + oRes);
     a.block_cnt = (int *)(m + oBc);
     a.pm = pmv;
     a.cell_perm = nullptr;
@@ -990,7 +1116,7 @@ static int trace_chunk(const DDMRun &run, const PhotonGridView &pmv, const Photo
         mr.queries = a.queries;
         mr.n_queries = a.n_queries;
         mr.q_cap = q_cap;
-        mr.results = (float2 *)(m + oRes);
+        mr.results = (float *)(m + oRes);
         mr.mode = 1;
         mr.raw = 0;
         mr.fallbacks = run.counters + 4;
@@ -1004,6 +1130,7 @@ static int trace_chunk(const DDMRun &run, const PhotonGridView &pmv, const Photo
     const int waves = ddm_waves(run.g);
     const size_t ctl_bytes = 32 + 4 * (size_t)nb;
     const unsigned cont_blocks = whole_waves(k_shade_continue, 256, sizeof(int) * (size_t)nb, sm, path_blocks);
+    const unsigned spec_blocks = (unsigned)std::min<int64_t>((np + kSpecThreads - 1) / kSpecThreads, (int64_t)sm * 32);
     // the glass count and gather passes share one partition of the path slots
     const unsigned glass_blocks = whole_waves(k_glass_gather, 256, 0, sm, path_blocks);
     cudaError_t e;
@@ -1104,9 +1231,9 @@ static int trace_chunk(const DDMRun &run, const PhotonGridView &pmv, const Photo
             *run.launches += 2;
         }
         if (run.sc.mat_nfilm)
-            k_shade_spectral<true><<<path_blocks, 256, 0, s>>>(a);
+            k_shade_spectral<true><<<spec_blocks, kSpecThreads, 0, s>>>(a);
         else
-            k_shade_spectral<false><<<path_blocks, 256, 0, s>>>(a);
+            k_shade_spectral<false><<<spec_blocks, kSpecThreads, 0, s>>>(a);
         DDM_CHECK(cudaGetLastError());
         if (a.pm.on) {
             // one path slot per thread: the gather is latency-bound and gains from the most blocks in flight

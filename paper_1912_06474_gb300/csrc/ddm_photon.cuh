@@ -259,7 +259,8 @@ __global__ void __launch_bounds__(256) k_ddm_gather(KArgs a) {
         const float *rho = (kind == kLambert ? sc.mat_a : sc.mat_b) + (size_t)mat * L;
         Kahan X, Y, Z;
         for (int i = 0; i < L; ++i) {
-            const float e = ps.T[(size_t)i * np + q] * __ldg(rho + i) * S[i] * norm;
+            const float t = b >= 2 ? ps.T[(size_t)q * sc.Lp + i] : 1.0f;   // no weight yet at the first vertex
+            const float e = t * __ldg(rho + i) * S[i] * norm;
             const float4 w4 = __ldg(sc.wcmf + i);
             X.add(e * w4.x);
             Y.add(e * w4.y);

@@ -321,6 +321,7 @@ __device__ __forceinline__ void tc_put_hidden(TcSmem &s, int row, const float v[
 struct RowIn {
     float c, lam, s, d;
     int mat, bin;
+    int64_t q;   // mode 1: the row's query
 };
 
 // Normal-incidence absorbance of a row's glass: alpha(lambda, s) d of the
@@ -364,6 +365,7 @@ __device__ __forceinline__ bool row_input(const MlpRows &a, int64_t r, int64_t t
         in.d = 0.5f * (a.thick_min + a.thick_max);
         in.mat = 0;
         in.bin = 0;
+        in.q = 0;
         return false;
     }
     const int L = a.sc.L;
@@ -383,6 +385,7 @@ __device__ __forceinline__ bool row_input(const MlpRows &a, int64_t r, int64_t t
         in.d = qq.z;
         in.mat = __float_as_int(qq.w);
         in.bin = (int)(r - q * L);
+        in.q = q;
     } else {
         int64_t q = r;
         const int ic = (int)(q % kGridCos);
@@ -413,12 +416,23 @@ __device__ __forceinline__ bool row_in_box(const MlpRows &a, const RowIn &in) {
            in.d >= a.thick_min && in.d <= a.thick_max;
 }
 
-__device__ __forceinline__ void store_row(const MlpRows &a, int64_t r, float2 y) {
+// Renderer results: R and T of a query in two rows of Lp bins, so that a
+// reader takes four bins of the one it needs per 16-byte load; the last bin's
+// thread fills the padding.
+__device__ __forceinline__ float *result_at(const MlpRows &a, const RowIn &in) {
+    return a.results + (size_t)in.q * 2 * a.sc.Lp + in.bin;
+}
+__device__ __forceinline__ void store_row(const MlpRows &a, int64_t r, const RowIn &in, float2 y) {
     if (a.mode == 0) {
         a.R[r] = y.x;
         a.T[r] = y.y;
     } else {
-        a.results[r] = y;
+        float *at = result_at(a, in);
+        const int Lp = a.sc.Lp, n = in.bin == a.sc.L - 1 ? Lp - in.bin : 1;
+        for (int k = 0; k < n; ++k) {
+            at[k] = y.x;
+            at[Lp + k] = y.y;
+        }
     }
 }
 
@@ -530,7 +544,7 @@ __global__ void __launch_bounds__(kTcRows, SDDM_MLP_MINB) k_mlp_net(MlpRows a) {
                 atomicMax(a.grid_err + 0, __float_as_uint(fabsf(e.x - y.x)));
                 atomicMax(a.grid_err + 1, __float_as_uint(fabsf(e.y - y.y)));
             } else {
-                store_row(a, r, y);
+                store_row(a, r, in, y);
             }
         }
     }
@@ -604,7 +618,8 @@ __global__ void __launch_bounds__(256) k_mlp_probe(MlpRows a) {
             const int64_t r = r0 + (int)(pr.x % (uint32_t)nvalid);
             row_input(a, r, total, in);
             const float2 e = exact_row<FILMS>(a, in);
-            const float2 y = a.mode == 0 ? make_float2(a.R[r], a.T[r]) : a.results[r];
+            const float2 y = a.mode == 0 ? make_float2(a.R[r], a.T[r])
+                                         : make_float2(*result_at(a, in), result_at(a, in)[a.sc.Lp]);
             bad |= fabsf(e.x - y.x) > kMlpProbeTol || fabsf(e.y - y.y) > kMlpProbeTol;
         }
         unsigned fall = __ballot_sync(kFull, bad);
@@ -615,7 +630,8 @@ __global__ void __launch_bounds__(256) k_mlp_probe(MlpRows a) {
             int nvalid;
             batch_rows(b_first + (k0 + k) * nwarps, r0, nvalid);
             RowIn in;
-            if (lane < nvalid && row_input(a, r0 + lane, total, in)) store_row(a, r0 + lane, exact_row<FILMS>(a, in));
+            if (lane < nvalid && row_input(a, r0 + lane, total, in))
+                store_row(a, r0 + lane, in, exact_row<FILMS>(a, in));
             if (lane == 0) ++n_fb;
         }
     }
@@ -632,13 +648,7 @@ __global__ void __launch_bounds__(256) k_slab_rows(MlpRows a) {
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < total; r += stride) {
         RowIn in;
         row_input(a, r, total, in);
-        const float2 y = exact_row<FILMS>(a, in);
-        if (a.mode == 0) {
-            a.R[r] = y.x;
-            a.T[r] = y.y;
-        } else {
-            a.results[r] = y;
-        }
+        store_row(a, r, in, exact_row<FILMS>(a, in));
     }
 }
 

@@ -126,7 +126,7 @@ struct sddm_ctx {
     bool built = false;
     sddm_build_opts opts{};
     // device scene
-    DevBuf d_wcmf, d_lam, d_kind, d_a, d_b, d_c, d_thick, d_tri_n, d_tri_obj, d_light_v, d_light_cdf;
+    DevBuf d_wcmf, d_tab, d_lam, d_kind, d_a, d_b, d_c, d_thick, d_tri_n, d_tri_obj, d_light_v, d_light_cdf;
     DevBuf d_nfilm, d_film_n, d_film_k, d_film_dk, d_film_t;
     DevBuf d_gnodes, d_gtris;
     float light_area = 0.f;
@@ -446,7 +446,8 @@ int sddm_build(sddm_ctx *ctx, const sddm_build_opts *opts) {
     for (size_t i = 0; i < light_cum.size(); ++i) light_cdf[i] = (float)(light_cum[i] / light_total);
 
     // --- materials, spectral weights
-    std::vector<float> wcmf(4 * (size_t)L, 0.f), A((size_t)M * L, 0.f), B((size_t)M * L, 0.f), Cc((size_t)M * L, 0.f),
+    const int Lp = (L + 3) & ~3;
+    std::vector<float> wcmf(4 * (size_t)L, 0.f), tab((2 * (size_t)M + 3) * Lp, 0.f), A((size_t)M * L, 0.f), B((size_t)M * L, 0.f), Cc((size_t)M * L, 0.f),
         thick(M, 0.f);
     std::vector<int> kinds(M);
     for (int i = 0; i < L; ++i)
@@ -461,6 +462,13 @@ int sddm_build(sddm_ctx *ctx, const sddm_build_opts *opts) {
         }
         thick[m] = mt.thick;
     }
+    for (int m = 0; m < M; ++m)
+        for (int i = 0; i < Lp; ++i) {
+            tab[(size_t)m * Lp + i] = A[(size_t)m * L + std::min(i, L - 1)];
+            tab[(size_t)(M + m) * Lp + i] = B[(size_t)m * L + std::min(i, L - 1)];
+        }
+    for (int c = 0; c < 3; ++c)
+        for (int i = 0; i < L; ++i) tab[(2 * (size_t)M + c) * Lp + i] = wcmf[4 * i + c];
     // coating films of glass materials, [m][SDDM_MAX_FILMS][L] (+ thickness [m][SDDM_MAX_FILMS])
     bool any_film = false;
     for (int m = 0; m < M; ++m) any_film |= ctx->mats[m].n_film > 0;
@@ -544,7 +552,7 @@ int sddm_build(sddm_ctx *ctx, const sddm_build_opts *opts) {
 
     // --- upload
     cudaStream_t s = ctx->stream;
-    if ((e = ctx->d_wcmf.upload(wcmf, s)) || (e = ctx->d_lam.upload(ctx->lam, s)) ||
+    if ((e = ctx->d_wcmf.upload(wcmf, s)) || (e = ctx->d_tab.upload(tab, s)) || (e = ctx->d_lam.upload(ctx->lam, s)) ||
         (e = ctx->d_kind.upload(kinds, s)) || (e = ctx->d_a.upload(A, s)) || (e = ctx->d_b.upload(B, s)) ||
         (e = ctx->d_c.upload(Cc, s)) || (e = ctx->d_thick.upload(thick, s)) || (e = ctx->d_tri_n.upload(tri_n, s)) ||
         (e = ctx->d_tri_obj.upload(tri_obj, s)) || (e = ctx->d_light_v.upload(light_v, s)) ||
@@ -564,7 +572,9 @@ int sddm_build(sddm_ctx *ctx, const sddm_build_opts *opts) {
     DevScene &d = ctx->dev;
     d.L = L;
     d.n_mat = M;
+    d.Lp = Lp;
     d.wcmf = ctx->d_wcmf.as<float4>();
+    d.tab = ctx->d_tab.as<float>();
     d.lam = ctx->d_lam.as<float>();
     d.mat_kind = ctx->d_kind.as<int>();
     d.mat_a = ctx->d_a.as<float>();

@@ -47,7 +47,7 @@ struct DDMScene {
 // Path state of one chunk of np path slots (structure of arrays).
 struct PathState {
     int64_t np;
-    float *T;             // [L][np] spectral throughput
+    float *T;             // spectral throughput: camera paths [np][Lp], photons' power [L][np]
     float *acc;           // [6][np] XYZ compensated sums (s, c) x 3
     int *flags;           // [np] kFl* bits
     int *pend_mat;        // [np] material of the last vertex (weight still to apply)

@@ -44,7 +44,10 @@ constexpr uint32_t kTriGlass = 1u;
 struct DevScene {
     int L;
     int n_mat;
+    int Lp;                   // L rounded up to a multiple of 4: bins of a padded row
     const float4 *wcmf;       // [L] (quad_w * cmf_x, quad_w * cmf_y, quad_w * cmf_z, 0)
+    const float *tab;         // [2 n_mat + 3][Lp] padded rows: mat_a, mat_b (the last bin repeated), then
+                              // quad_w * cmf_x, _y, _z (zero past L)
     const float *lam;         // [L]
     const int *mat_kind;      // [n_mat]
     const float *mat_a;       // [n_mat][L] rho | n | n(glass) | Le

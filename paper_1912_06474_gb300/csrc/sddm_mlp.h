@@ -30,7 +30,7 @@ struct MlpRows {
     const float4 *queries;
     const unsigned long long *n_queries;
     int64_t q_cap;                    // queries beyond it were not stored
-    float2 *results;                  // [query][L] (R, T)
+    float *results;                   // [query][2][Lp]: R, then T, of its bins
     int mode;
     int raw;                          // 1: network output only, no probe or fallback
     unsigned long long *fallbacks;    // 32-row batches that fell back to the exact slab
