@@ -79,6 +79,7 @@ struct KArgs {
     int *cross_query;     // [kMaxCross][np]
     const float *glass_res;   // [query][2][Lp]: R, then T
     int *block_cnt;       // [gridDim] glass queries per block of path slots (count pass)
+    uint32_t *list_cnt;   // [4] surrogate batch lists, emptied by the gather pass
     PhotonGridView pm;    // photon map: gather at the first diffuse vertex, no continuation there
     PhotonGridView pmc;   // caustic map gathered with it (pmc.on)
     // subdomain cache: the wave's queue is sorted with the cells in this order
@@ -465,6 +466,7 @@ __global__ void __launch_bounds__(256) k_glass_gather(KArgs a) {
     int before_all;
     block_scan256(part, s_w, &before_all);
     int64_t base = before_all;
+    if (blockIdx.x == 0 && threadIdx.x < 4) a.list_cnt[threadIdx.x] = 0;
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0)
         *a.n_queries = (unsigned long long)(base + a.block_cnt[blockIdx.x]);
     for (int64_t t0 = lo; t0 < hi; t0 += 256) {
@@ -1047,6 +1049,13 @@ static int trace_chunk(const DDMRun &run, const PhotonGridView &pmv, const Photo
     const size_t oQ = take(16 * (size_t)q_cap + 16), oNq = take(16), oPq = take(use_queries ? 4 * np : 4),
                  oCq = take(use_queries ? 4 * kMaxCross * np : 4), oRes = take(8 * (size_t)q_cap * run.sc.Lp + 16),
                  oBc = take(4 * (size_t)path_blocks + 16);
+    // surrogate batches sorted by their probes
+    const int64_t n_batch = use_mlp ? q_cap * ((run.sc.L + 31) / 32) : 0;
+    if (n_batch > UINT32_MAX) {
+        set_error("sddm_render: too many surrogate batches in one chunk (reduce paths_in_flight)");
+        return SDDM_ERR_OOM;
+    }
+    const size_t oLp = take(4 * (size_t)n_batch), oLf = take(4 * (size_t)n_batch), oLc = take(16);
     if (off > buf.bytes) {
         if (buf.mem) cudaFree(buf.mem);
         buf.mem = nullptr;
@@ -1101,6 +1110,7 @@ static int trace_chunk(const DDMRun &run, const PhotonGridView &pmv, const Photo
     a.cross_query = (int *)(m + oCq);
     a.glass_res = (const float *)(m + oRes);
     a.block_cnt = (int *)(m + oBc);
+    a.list_cnt = (uint32_t *)(m + oLc);
     a.pm = pmv;
     a.cell_perm = nullptr;
     a.q_begin = 0;
@@ -1123,6 +1133,10 @@ static int trace_chunk(const DDMRun &run, const PhotonGridView &pmv, const Photo
         mr.batches = run.counters + 8;
         mr.rows = run.counters + 9;
         mr.err = run.error_flag;
+        mr.list_pass = (uint32_t *)(m + oLp);
+        mr.list_fail = (uint32_t *)(m + oLf);
+        mr.list_cnt = a.list_cnt;
+        mr.list_cap = (uint32_t)n_batch;
     }
 
     const int trace_blocks = sm * (run.blocks_per_sm > 0 ? run.blocks_per_sm : 8);
@@ -1225,7 +1239,7 @@ static int trace_chunk(const DDMRun &run, const PhotonGridView &pmv, const Photo
                 if (run.time_trace && (e = buf.mlp_event_pair(m0, m1)) != cudaSuccess)
                     return cuda_fail(e, "sddm_render: events");
                 DDM_CHECK(launch_mlp_rows(mr, run.sm_count, s, m0, m1));
-                *run.launches += mr.raw ? 0 : 1;   // the probe pass
+                *run.launches += 2;   // probes, passed batches, exact fallback
             } else
                 DDM_CHECK(launch_slab_rows(mr, run.sm_count, s));
             *run.launches += 2;

@@ -107,6 +107,9 @@ struct DevBuf {
     T *as() const { return reinterpret_cast<T *>(p); }
 };
 
+// Device error word [4] and, behind it, the surrogate's batch counts [4].
+constexpr size_t kErrBytes = 32;
+
 }  // namespace sddm
 
 using namespace sddm;
@@ -156,7 +159,7 @@ struct sddm_ctx {
     };
     std::vector<std::unique_ptr<MlpNet>> nets;
     std::vector<int> net_of_mat;     // per material, -1 = none
-    DevBuf mlp_grad_cta, mlp_loss_cta, mlp_scalar, mlp_X, mlp_Y;
+    DevBuf mlp_grad_cta, mlp_loss_cta, mlp_scalar, mlp_X, mlp_Y, mlp_lists;
     // CUDA graphs of the render launch sequence, keyed by everything that is
     // baked into kernel parameters (sizes, buffer addresses, build)
     int64_t build_id = 0;
@@ -825,7 +828,7 @@ int sddm_render(sddm_ctx *ctx, const sddm_render_desc *d, int n, sddm_stats *st)
     cudaStream_t s = ctx->stream;
     if ((e = ctx->d_info.upload(info, s)) || (e = ctx->d_state.upload(state, s)) || (e = ctx->d_out_tab.upload(outs, s)) ||
         (e = ctx->d_aov_xyz_tab.upload(aov_x, s)) || (e = ctx->d_aov_prim_tab.upload(aov_p, s)) ||
-        (e = ctx->d_counters.ensure(kNumCounters * sizeof(unsigned long long))) || (e = ctx->d_err.ensure(16)))
+        (e = ctx->d_counters.ensure(kNumCounters * sizeof(unsigned long long))) || (e = ctx->d_err.ensure(kErrBytes)))
         return cuda_fail(e, "sddm_render: upload of the render table");
     if ((e = cudaMemsetAsync(ctx->d_counters.p, 0, kNumCounters * sizeof(unsigned long long), s)) ||
         (e = cudaMemsetAsync(ctx->d_err.p, 0, 16, s)))
@@ -1507,7 +1510,7 @@ int sddm_mlp_train(sddm_ctx *ctx, uint32_t mat, const sddm_mlp_train_opts *opts,
     }
     if ((e = cudaEventRecord(ctx->ev1, s))) return cuda_fail(e, "sddm_mlp_train: event");
     unsigned int *errs = reinterpret_cast<unsigned int *>(ctx->mlp_scalar.as<char>() + 16);
-    if ((e = launch_mlp_pack(net->params.as<float>(), s)) || (e = ctx->d_err.ensure(16)) ||
+    if ((e = launch_mlp_pack(net->params.as<float>(), s)) || (e = ctx->d_err.ensure(kErrBytes)) ||
         (e = cudaMemsetAsync(ctx->d_err.p, 0, 16, s)) || (e = cudaMemsetAsync(errs, 0, 8, s)) ||
         (e = launch_mlp_grid_error(net->params.as<float>(), ctx->dev, mat, o.thick_min, o.thick_max, errs,
                                    ctx->d_err.as<int>(), ctx->sm_count, s)))
@@ -1695,9 +1698,16 @@ int sddm_glass_eval(sddm_ctx *ctx, uint32_t mat, int n, const float *cos_theta, 
         a.test_timeout = (ctx->profile & SDDM_PROFILE_TEST_MLP_TIMEOUT) != 0;
         int derr[4] = {0, 0, 0, 0};
         cudaError_t e = cudaSetDevice(ctx->device);
-        if (e == cudaSuccess) e = ctx->d_err.ensure(16);
-        if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_err.p, 0, 16, ctx->stream);
+        // the batch counts lie behind the error word, the two lists in scratch kept for the next call
+        const size_t n_batch = ((size_t)n + 31) / 32;
+        if (e == cudaSuccess) e = ctx->d_err.ensure(kErrBytes);
+        if (e == cudaSuccess && !a.raw) e = ctx->mlp_lists.ensure(8 * n_batch);
+        if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_err.p, 0, kErrBytes, ctx->stream);
         a.err = ctx->d_err.as<int>();
+        a.list_cnt = ctx->d_err.as<uint32_t>() + 4;
+        a.list_pass = ctx->mlp_lists.as<uint32_t>();
+        a.list_fail = a.list_pass + n_batch;
+        a.list_cap = (uint32_t)n_batch;
         if (e == cudaSuccess) e = launch_mlp_rows(a, ctx->sm_count, ctx->stream);
         if (e == cudaSuccess) e = cudaMemcpyAsync(derr, ctx->d_err.p, sizeof derr, cudaMemcpyDeviceToHost, ctx->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);

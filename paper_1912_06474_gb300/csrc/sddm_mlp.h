@@ -38,11 +38,17 @@ struct MlpRows {
     int *err;                         // device error word [4] (NULL: not reported); 2 = a wait ran out
     unsigned int *grid_err;           // mode 2: largest |dR|, |dT| as float bits [2]
     unsigned long long *rows;         // rows the network evaluated (NULL: not counted)
+    // unless raw: batches sorted by their probes, full ones from the front of
+    // a list, short ones from its back; list_cnt[4] zero before the call
+    uint32_t *list_pass, *list_fail;  // [list_cap]
+    uint32_t *list_cnt;               // passed full, passed short, failed full, failed short
+    uint32_t list_cap;                // at least the call's batches
     int test_timeout;                 // 1: CTA 0 issues no layer-1 MMA and waits 2^10 tries (failure-path test)
 };
-// The network over every row (tensor cores), then, unless raw, the probes
-// and the exact fallback of failing batches: two kernels on `stream`. With
-// ev0 / ev1 given, they are recorded around the network kernel.
+// raw: the network over every row (tensor cores). Otherwise the network over
+// one probe row per batch, then over the batches that passed, and the exact slab
+// over the others: three kernels on `stream`. With ev0 / ev1 given, they are
+// recorded around the network kernels.
 cudaError_t launch_mlp_rows(const MlpRows &a, int sm_count, cudaStream_t stream, cudaEvent_t ev0 = nullptr,
                             cudaEvent_t ev1 = nullptr);
 // The exact slab over the same rows (no network).
