@@ -146,7 +146,8 @@ struct Hit {
     int prim;   // original triangle id, -1 = none
 };
 
-// Closest hit with t in (tmin, tmax]; ties on t go to the lower triangle id.
+// Closest hit with t in (tmin, tmax); ties on t go to the lower triangle id. A
+// triangle the ray misses has t = +inf, which is no hit for tmax = +inf either.
 // excl_prim: triangle skipped; excl_obj >= 0: every triangle of that object skipped.
 // The hierarchy starts at node `root` (0 for the global one).
 // With COUNT, interior nodes visited and triangles tested are added to *cnt.
@@ -192,7 +193,7 @@ __device__ __forceinline__ Hit trace_closest(const float4 *__restrict__ nodes, c
                 if (id == excl_prim || (excl_obj >= 0 && __float_as_int(b.w) == excl_obj)) continue;
                 if (COUNT) ++cnt->tris;
                 float t = wt_intersect(r, xyz(a), xyz(b), xyz(c));
-                if (t > tmin && (t < h.t || (t == h.t && (h.prim < 0 || id < h.prim)))) {
+                if (t > tmin && (t < h.t || (t == h.t && id < h.prim))) {
                     h.t = t;
                     h.prim = id;
                 }
