@@ -1139,7 +1139,7 @@ static int trace_chunk(const DDMRun &run, const PhotonGridView &pmv, const Photo
         mr.list_cap = (uint32_t)n_batch;
     }
 
-    const int trace_blocks = sm * (run.blocks_per_sm > 0 ? run.blocks_per_sm : 8);
+    const int trace_blocks = sm * (run.blocks_per_sm > 0 ? run.blocks_per_sm : SDDM_TRACE_MIN_BLOCKS);
     const unsigned scatter_blocks = whole_waves(k_scatter, 256, 0, sm, (unsigned)sm * 4);
     const int waves = ddm_waves(run.g);
     const size_t ctl_bytes = 32 + 4 * (size_t)nb;

@@ -347,7 +347,7 @@ int ddm_photon_pass(const DDMPhotonRun &run, DDMBuffers &buf, cudaStream_t s) {
 
     const int sm = std::max(1, run.sm_count);
     const unsigned path_blocks = (unsigned)std::min<int64_t>((np + 255) / 256, (int64_t)sm * 16);
-    const int trace_blocks = sm * (run.blocks_per_sm > 0 ? run.blocks_per_sm : 8);
+    const int trace_blocks = sm * (run.blocks_per_sm > 0 ? run.blocks_per_sm : SDDM_TRACE_MIN_BLOCKS);
     const int scatter_blocks = sm * 4;
     const int waves = ddm_waves(run.g);
     const size_t ctl_bytes = 32 + 4 * (size_t)nb;

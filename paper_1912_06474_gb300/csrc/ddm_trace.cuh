@@ -9,30 +9,30 @@
 // (-1 when it leaves the grid). Ties between faces go x, then y, then z. The
 // cell's planes and neighbours come from the per-cell table; distances use
 // the ray's reciprocal direction.
-__device__ __forceinline__ float cell_exit(const DDMScene &g, int cell, const Ray &r, int &next) {
+__device__ __forceinline__ float cell_exit(const DDMScene &g, int cell, V3 o, V3 d, V3 inv, int &next) {
     const float4 p0 = __ldg(g.cell_planes + 2 * cell), p1 = __ldg(g.cell_planes + 2 * cell + 1);
     const int4 n0 = __ldg(g.cell_next + 2 * cell), n1 = __ldg(g.cell_next + 2 * cell + 1);
     float t = __int_as_float(0x7f800000);
     next = -1;
-    if (r.d.x != 0.0f) {
-        const bool pos = r.d.x > 0.0f;
-        const float ta = ((pos ? p0.y : p0.x) - r.o.x) * r.inv.x;
+    if (d.x != 0.0f) {
+        const bool pos = d.x > 0.0f;
+        const float ta = ((pos ? p0.y : p0.x) - o.x) * inv.x;
         if (ta < t) {
             t = ta;
             next = pos ? n0.y : n0.x;
         }
     }
-    if (r.d.y != 0.0f) {
-        const bool pos = r.d.y > 0.0f;
-        const float ta = ((pos ? p0.w : p0.z) - r.o.y) * r.inv.y;
+    if (d.y != 0.0f) {
+        const bool pos = d.y > 0.0f;
+        const float ta = ((pos ? p0.w : p0.z) - o.y) * inv.y;
         if (ta < t) {
             t = ta;
             next = pos ? n0.w : n0.z;
         }
     }
-    if (r.d.z != 0.0f) {
-        const bool pos = r.d.z > 0.0f;
-        const float ta = ((pos ? p1.y : p1.x) - r.o.z) * r.inv.z;
+    if (d.z != 0.0f) {
+        const bool pos = d.z > 0.0f;
+        const float ta = ((pos ? p1.y : p1.x) - o.z) * inv.z;
         if (ta < t) {
             t = ta;
             next = pos ? n1.y : n1.x;
@@ -72,16 +72,37 @@ __device__ __forceinline__ void block_count3(unsigned long long *c0, unsigned lo
 }
 
 // ------------------------------------------------------ trace one wave
-// Persistent warps whose lanes are refilled one by one: a lane that finishes
-// its ray (hit, occlusion, or exit from the cell) takes the next ray of the
-// cell-sorted queue while the other lanes carry on, so a warp is not held by
-// its slowest ray. Traversal is a resumable state machine; each round runs the
-// warp through interior nodes until every lane stands at a leaf (at most
-// kTraceSteps steps), then through the leaves, then refills.
+// Persistent warps whose lanes are refilled from the cell-sorted queue while the
+// others carry on, so a warp is not held by its slowest ray. Traversal is a
+// resumable state machine; a round takes the warp through interior nodes, then
+// through leaves. What bounds it is latency and issue together (DRAM 5 %, L1
+// wavefronts half of peak, 59 % of the slots issued at 13.5 of 32 lanes when a
+// round ran until the last lane stood at a leaf and stopped for every single
+// finished lane). So
+//  * results, hand-offs and refills wait until kTraceBatch lanes need one: their
+//    some 300 instructions ran for two or three lanes at a time. Hotel room, 12
+//    launches (512 x 512 x 16 spp), lanes 1 / 4 / 8 / 12 / 16: 13.5 / 13.1 / 13.0
+//    / 12.7 / 12.7 ms (20: no better);
+//  * the interior phase ends once at most 1 / kTraceQuorum of the busy lanes still
+//    descend (64 i.e. the last lane / 6 / 4 / 3: 13.6 / 12.9 / 13.0 / 13.3 ms);
+//  * a lane carries only what the traversal itself uses, and triangle records are
+//    read in the ray's axis order (make_ray, load_tri) instead of permuted by
+//    selects: 12.7 -> 12.1 ms;
+//  * 7 resident blocks of 128 threads (72 registers, few spills): 11.4 ms, against
+//    12.1 with 8 (64 registers) and 12.1 with 6 (80).
+// 13.2 ms before all of it; facade room (480 x 270 x 4 spp, 81 bins) 7.4 -> 6.7 ms.
 #ifndef SDDM_TRACE_STEPS
 #define SDDM_TRACE_STEPS 64   // interior steps per round at most
 #endif
 constexpr int kTraceSteps = SDDM_TRACE_STEPS;
+#ifndef SDDM_TRACE_BATCH
+#define SDDM_TRACE_BATCH 16
+#endif
+constexpr int kTraceBatch = SDDM_TRACE_BATCH;
+#ifndef SDDM_TRACE_QUORUM
+#define SDDM_TRACE_QUORUM 6
+#endif
+constexpr int kTraceQuorum = SDDM_TRACE_QUORUM;
 // Queue slots a warp reserves per refill atomic (>= 32, so one run always covers a refill).
 constexpr int kRefillChunk = 32;
 // Rays a warp buffers in shared memory before appending them to the staging area.
@@ -102,9 +123,10 @@ __device__ __forceinline__ void flush_push_buf(const Queues &Q, const float4 *bu
     for (int k = lane; k < 3 * n; k += 32) dst[k] = buf[k];
     __syncwarp();
 }
-// Resident 128-thread blocks per SM the trace kernel is compiled for (register budget).
+// Resident 128-thread blocks per SM the trace kernel is compiled for (register
+// budget), and launched with unless the build options say otherwise.
 #ifndef SDDM_TRACE_MIN_BLOCKS
-#define SDDM_TRACE_MIN_BLOCKS 8
+#define SDDM_TRACE_MIN_BLOCKS 7
 #endif
 
 // First device check to fail records its code and two details in the error word.
@@ -131,7 +153,7 @@ __global__ void __launch_bounds__(128, SDDM_TRACE_MIN_BLOCKS) k_trace_wave(KArgs
     const int lane = threadIdx.x & 31;
     const unsigned lt_mask = (1u << lane) - 1u;
     const int64_t np = a.ps.np;
-    unsigned long long n_cross = 0, n_vis = 0, n_cont = 0;   // n_cont: crossings carried on by the lane
+    unsigned n_cross = 0, n_vis = 0, n_cont = 0;   // n_cont: crossings carried on by the lane
     TravCount tc;
 
     __shared__ float4 s_push[128 / 32][3 * kPushBuf];   // per-warp hand-off buffers
@@ -144,95 +166,198 @@ __global__ void __launch_bounds__(128, SDDM_TRACE_MIN_BLOCKS) k_trace_wave(KArgs
     if (lane == 0) run[0] = run[1] = 0;
     __syncwarp();
     Ray ray;
-    float t_cur = 0.f, t_max = 0.f, t_exit = 0.f, tmin = 0.f, tw = 0.f;
-    int q = 0, excl = -1, rfl = 0, next = -1, node = 0, sp = 0, best = -1, ep = -1, eo = -1, n_prev = 0;
-    bool occ = false;
+    // what a lane carries through the traversal; the rest of its ray (direction,
+    // range, path slot, exclusion) is read again from the queue when it finishes
+    float t_cur = 0.f, t_exit = 0.f, tmin = 0.f, tw = 0.f;
+    int rfl = 0, next = -1, node = 0, sp = 0, best = -1, ep = -1, eo = -1;
+    bool occ = false, fin = false;
     Crossings cr;
     cr.n = 0;
     int stack[kStackSize];
 
     for (;;) {
-        // 1. idle lanes take the next rays of the queue, from a run of
-        //    kRefillChunk queue slots the warp reserves at a time (one atomic
-        //    per run instead of one per refill)
-        const bool need = idx < 0 && !exhausted;
-        const unsigned m = __ballot_sync(full, need);
-        if (m) {
-            const unsigned want = __popc(m);
-            const unsigned long long cbeg = run[0], cend = run[1];
-            const unsigned long long avail = cend - cbeg;
-            unsigned long long nb = 0;
-            if (avail < want) {
-                if (lane == 0) nb = atomicAdd(Q.ctl + 1, (unsigned long long)kRefillChunk);
-                nb = __shfl_sync(full, nb, 0);
-            }
-            const unsigned rank = __popc(m & lt_mask);
-            const unsigned long long mine = rank < avail ? cbeg + rank : nb + (rank - avail);
-            __syncwarp();
-            if (lane == 0) {
-                if (avail >= want) {
-                    run[0] = cbeg + want;
-                } else {
-                    run[0] = nb + (want - avail);
-                    run[1] = nb + kRefillChunk;
-                }
-            }
-            __syncwarp();
-            if (need) {
-                const unsigned long long my = mine;
-                if (my < (unsigned long long)total) {
-                    idx = q0 + (int)my;
-                    const float4 *src = Q.in + 3 * (size_t)idx;
-                    const float4 r0 = src[0], r1 = src[1], r2f = src[2];
-                    q = __float_as_int(r2f.x);
-                    excl = __float_as_int(r2f.y);
-                    rfl = __float_as_int(r2f.z);
-                    int cell = __float_as_int(r2f.w);
-                    if (CHECKED && (q < 0 || q >= np || cell < 0 || cell >= g.n_cells)) {
-                        trace_check_fail(a.err, 12, q, cell);
-                        q = 0;
-                        cell = 0;
+        // 1. results, hand-offs and refills, once enough lanes wait for them
+        const unsigned m_fin = __ballot_sync(full, fin);
+        const unsigned m_need = __ballot_sync(full, idx < 0 && !exhausted);
+        const unsigned m_busy = __ballot_sync(full, idx >= 0 && !fin);
+        if (m_busy == 0 || __popc(m_fin | m_need) >= kTraceBatch) {
+            if ((m_fin | m_need) == 0) break;
+            // 1a. finished lanes: final result, or hand-off to the neighbouring cell
+            bool want = false;
+            float4 o0 = make_float4(0, 0, 0, 0), o1 = o0;
+            int4 o2 = make_int4(0, 0, 0, 0);
+            if (fin) {
+                const float4 *src = Q.in + 3 * (size_t)idx;
+                const float4 r0 = src[0], r1 = src[1];
+                const float2 r2f = *reinterpret_cast<const float2 *>(src + 2);
+                const V3 ro = xyz(r0), rd = xyz(r1);
+                const float t_max = r1.w;
+                int q = __float_as_int(r2f.x);
+                if (CHECKED && (q < 0 || q >= np)) q = 0;   // recorded when the ray was taken
+                const int excl = __float_as_int(r2f.y);
+                bool done = false;
+                int rfl_next = rfl;
+                if (rfl & kRayShadow) {
+                    for (int k = (rfl >> 1) & 7; k < cr.n; ++k) {
+                        const float4 cn = __ldg(a.sc.tri_n + cr.tri[k]);
+                        a.ps.cross_obj[k * np + q] = cr.obj[k];
+                        a.ps.cross_mat[k * np + q] = __float_as_int(cn.w);
+                        a.ps.cross_cos[k * np + q] = -dot(rd, xyz(cn));
                     }
-                    ray = make_ray(xyz(r0), xyz(r1));
-                    t_cur = r0.w;
-                    t_max = r1.w;
-                    t_exit = cell_exit(g, cell, ray, next);
+                    if (occ) {
+                        a.ps.sh_status[q] = kShadowOccluded;
+                        done = true;
+                    } else if (t_exit + g.eps >= t_max || next < 0) {
+                        a.ps.sh_status[q] = kShadowClear | (cr.n << 4);
+                        done = true;
+                    }
+                    rfl_next = (rfl & 1) | (cr.n << 1);
+                } else {
+                    if (best >= 0) {
+                        const V3 x = ro + tw * rd;
+                        a.ps.hit0[q] = make_float4(x.x, x.y, x.z, __int_as_float(best));
+                        a.ps.hit1[q] = make_float4(rd.x, rd.y, rd.z, tw);
+                        done = true;
+                    } else if (next < 0) {
+                        a.ps.hit0[q] = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
+                        a.ps.hit1[q] = make_float4(rd.x, rd.y, rd.z, 0.f);
+                        done = true;
+                    }
+                }
+                fin = false;
+                if (!done && a.g.continue_cells) {
+                    // the lane carries the ray on into the neighbouring cell's
+                    // BVH, with the same record it would have handed over
+                    const int cell = next;
+                    t_cur = fmaxf(t_cur, t_exit);
+                    t_exit = cell_exit(g, cell, ro, rd, ray.inv, next);
                     tmin = fmaxf(0.0f, t_cur - g.eps);
                     node = __ldg(g.root + cell);
-                    if (CHECKED && (node < 0 || node >= g.node_cap)) {
-                        trace_check_fail(a.err, 8, cell, node);
-                        node = ~0;   // an empty leaf: the ray ends here
-                    }
                     sp = 0;
                     best = -1;
                     occ = false;
-                    ++n_vis;
-                    if (rfl & kRayShadow) {
-                        tw = fminf(t_exit + g.eps, t_max);
-                        cr.n = (rfl >> 1) & 7;
-                        for (int k = 0; k < cr.n; ++k) cr.obj[k] = a.ps.cross_obj[k * np + q];
-                        n_prev = cr.n;
-                    } else {
-                        tw = t_exit + g.eps;
-                        ep = excl >= 0 ? excl : -1;
-                        eo = excl <= -2 ? -excl - 2 : -1;
-                    }
+                    rfl = rfl_next;
+                    tw = (rfl & kRayShadow) ? fminf(t_exit + g.eps, t_max) : t_exit + g.eps;
+                    ++n_cross;
+                    if (COUNT) ++n_vis;
+                    if (COUNT) ++n_cont;
                 } else {
-                    exhausted = true;
+                    if (!done) {
+                        want = true;
+                        o0 = make_float4(ro.x, ro.y, ro.z, fmaxf(t_cur, t_exit));
+                        o1 = r1;
+                        o2 = make_int4(q, excl, rfl_next, next);
+                        ++n_cross;
+                    }
+                    idx = -1;
+                }
+            }
+            if (want && a.last_wave) {   // cannot happen: each wave moves a ray forward along one axis
+                atomicCAS(a.err, 0, 4);
+                want = false;
+            }
+            // hand-off: append to the warp's buffer, flushing it to the staging
+            // area (one atomic, coalesced stores) when the new rays do not fit
+            const unsigned mw = __ballot_sync(full, want);
+            if (mw) {
+                const int n = __popc(mw);
+                if (nbuf + n > kPushBuf) {
+                    flush_push_buf(Q, pbuf, nbuf, lane, a.err);
+                    nbuf = 0;
+                }
+                if (want) {
+                    float4 *slot = pbuf + 3 * (nbuf + __popc(mw & lt_mask));
+                    slot[0] = o0;
+                    slot[1] = o1;
+                    slot[2] = make_float4(__int_as_float(o2.x), __int_as_float(o2.y), __int_as_float(o2.z),
+                                          __int_as_float(o2.w));
+                    const int bin = ray_bin(g, next, o2.z, o0, o1);
+                    const unsigned peers = __match_any_sync(mw, bin);
+                    if (lane == __ffs(peers) - 1) atomicAdd(Q.cnt + bin, __popc(peers));
+                }
+                nbuf += n;
+                __syncwarp();
+            }
+            // 1b. idle lanes take the next rays of the queue, from a run of
+            //     kRefillChunk queue slots the warp reserves at a time (one
+            //     atomic per run instead of one per refill)
+            const bool need = idx < 0 && !exhausted;
+            const unsigned m = __ballot_sync(full, need);
+            if (m) {
+                const unsigned want_n = __popc(m);
+                const unsigned long long cbeg = run[0], cend = run[1];
+                const unsigned long long avail = cend - cbeg;
+                unsigned long long nb = 0;
+                if (avail < want_n) {
+                    if (lane == 0) nb = atomicAdd(Q.ctl + 1, (unsigned long long)kRefillChunk);
+                    nb = __shfl_sync(full, nb, 0);
+                }
+                const unsigned rank = __popc(m & lt_mask);
+                const unsigned long long mine = rank < avail ? cbeg + rank : nb + (rank - avail);
+                __syncwarp();
+                if (lane == 0) {
+                    if (avail >= want_n) {
+                        run[0] = cbeg + want_n;
+                    } else {
+                        run[0] = nb + (want_n - avail);
+                        run[1] = nb + kRefillChunk;
+                    }
+                }
+                __syncwarp();
+                if (need) {
+                    const unsigned long long my = mine;
+                    if (my < (unsigned long long)total) {
+                        idx = q0 + (int)my;
+                        const float4 *src = Q.in + 3 * (size_t)idx;
+                        const float4 r0 = src[0], r1 = src[1], r2f = src[2];
+                        int q = __float_as_int(r2f.x);
+                        const int excl = __float_as_int(r2f.y);
+                        rfl = __float_as_int(r2f.z);
+                        int cell = __float_as_int(r2f.w);
+                        if (CHECKED && (q < 0 || q >= np || cell < 0 || cell >= g.n_cells)) {
+                            trace_check_fail(a.err, 12, q, cell);
+                            q = 0;
+                            cell = 0;
+                        }
+                        ray = make_ray(xyz(r0), xyz(r1));
+                        t_cur = r0.w;
+                        t_exit = cell_exit(g, cell, xyz(r0), xyz(r1), ray.inv, next);
+                        tmin = fmaxf(0.0f, t_cur - g.eps);
+                        node = __ldg(g.root + cell);
+                        if (CHECKED && (node < 0 || node >= g.node_cap)) {
+                            trace_check_fail(a.err, 8, cell, node);
+                            node = ~0;   // an empty leaf: the ray ends here
+                        }
+                        sp = 0;
+                        best = -1;
+                        occ = false;
+                        if (COUNT) ++n_vis;
+                        ep = excl >= 0 ? excl : -1;
+                        if (rfl & kRayShadow) {
+                            tw = fminf(t_exit + g.eps, r1.w);
+                            cr.n = (rfl >> 1) & 7;
+                            for (int k = 0; k < cr.n; ++k) cr.obj[k] = a.ps.cross_obj[k * np + q];
+                        } else {
+                            tw = t_exit + g.eps;
+                            eo = excl <= -2 ? -excl - 2 : -1;
+                        }
+                    } else {
+                        exhausted = true;
+                    }
                 }
             }
         }
-        if (__ballot_sync(full, idx >= 0) == 0) break;
 
-        // 2. one traversal round, while-while: an interior phase in which every
-        //    lane descends until it stands at a leaf (or its stack runs out),
-        //    then a leaf phase in which the lanes at a leaf test its triangles.
-        bool fin = false;
-        const bool live = idx >= 0;
+        // 2. one traversal round, while-while: an interior phase in which the
+        //    lanes descend until most of them stand at a leaf (or their stacks
+        //    run out), then a leaf phase in which the lanes at a leaf test its
+        //    triangles.
+        const bool live = idx >= 0 && !fin;
+        const int n_live = __popc(__ballot_sync(full, live));
         const bool shadow = (rfl & kRayShadow) != 0;
         for (int it = 0; it < kTraceSteps; ++it) {
             const bool act = live && !fin && node >= 0;
-            if (!__any_sync(full, act)) break;
+            if (__popc(__ballot_sync(full, act)) * kTraceQuorum <= n_live) break;
             if (act) {
                 if (COUNT) ++tc.nodes;
                 const float4 n0 = __ldg(g.nodes + 4 * node + 0), n1 = __ldg(g.nodes + 4 * node + 1),
@@ -278,21 +403,20 @@ __global__ void __launch_bounds__(128, SDDM_TRACE_MIN_BLOCKS) k_trace_wave(KArgs
                 trace_check_fail(a.err, 10, first, count);
                 count = 0;
             }
-            for (int i = 0; i < count; ++i) {
-                const float4 *tp = g.tris + 3 * (first + i);
-                const float4 ta4 = __ldg(tp), tb4 = __ldg(tp + 1), tc4 = __ldg(tp + 2);
-                const int id = __float_as_int(ta4.w);
+            for (int i = first; i < first + count; ++i) {
+                const TriRows tri = load_tri(g.tris, i, ray);
+                const int id = tri.key() & kTriIdMask;
+                if (id == ep) continue;
                 if (shadow) {
-                    if (id == excl) continue;
                     if (COUNT) ++tc.tris;
-                    const float t = wt_intersect(ray, xyz(ta4), xyz(tb4), xyz(tc4));
+                    const float t = wt_intersect(ray, tri);
                     if (!(t > tmin && t <= tw)) continue;
-                    if (!(__float_as_uint(tc4.w) & kTriGlass)) {
+                    if (!(tri.key() & kTriGlassBit)) {
                         occ = true;
                         break;
                     }
-                    if (dot(ray.d, cross(xyz(tb4) - xyz(ta4), xyz(tc4) - xyz(ta4))) >= 0.0f) continue;   // leaving face
-                    const int ob = __float_as_int(tb4.w);
+                    if (tri_leaving(g.tris, i, xyz(Q.in[3 * (size_t)idx + 1]))) continue;
+                    const int ob = __ldg(a.sc.tri_obj + id);
                     bool seen = false;
                     for (int k = 0; k < cr.n; ++k) seen |= cr.obj[k] == ob;
                     if (seen) continue;
@@ -304,9 +428,9 @@ __global__ void __launch_bounds__(128, SDDM_TRACE_MIN_BLOCKS) k_trace_wave(KArgs
                     cr.tri[cr.n] = id;
                     ++cr.n;
                 } else {
-                    if (id == ep || (eo >= 0 && __float_as_int(tb4.w) == eo)) continue;
+                    if (eo >= 0 && __ldg(a.sc.tri_obj + id) == eo) continue;
                     if (COUNT) ++tc.tris;
-                    const float t = wt_intersect(ray, xyz(ta4), xyz(tb4), xyz(tc4));
+                    const float t = wt_intersect(ray, tri);
                     if (t > tmin && (t < tw || (t == tw && (best < 0 || id < best)))) {
                         tw = t;
                         best = id;
@@ -318,97 +442,6 @@ __global__ void __launch_bounds__(128, SDDM_TRACE_MIN_BLOCKS) k_trace_wave(KArgs
             } else {
                 node = stack[--sp];
             }
-        }
-
-        // 3. finished lanes: final result, or hand-off to the neighbouring cell
-        bool want = false;
-        float4 o0 = make_float4(0, 0, 0, 0), o1 = o0;
-        int4 o2 = make_int4(0, 0, 0, 0);
-        if (fin) {
-            bool done = false;
-            int rfl_next = rfl;
-            if (rfl & kRayShadow) {
-                for (int k = n_prev; k < cr.n; ++k) {
-                    const float4 cn = __ldg(a.sc.tri_n + cr.tri[k]);
-                    a.ps.cross_obj[k * np + q] = cr.obj[k];
-                    a.ps.cross_mat[k * np + q] = __float_as_int(cn.w);
-                    a.ps.cross_cos[k * np + q] = -dot(ray.d, xyz(cn));
-                }
-                if (occ) {
-                    a.ps.sh_status[q] = kShadowOccluded;
-                    done = true;
-                } else if (t_exit + g.eps >= t_max || next < 0) {
-                    a.ps.sh_status[q] = kShadowClear | (cr.n << 4);
-                    done = true;
-                }
-                rfl_next = (rfl & 1) | (cr.n << 1);
-            } else {
-                if (best >= 0) {
-                    const V3 x = ray.o + tw * ray.d;
-                    a.ps.hit0[q] = make_float4(x.x, x.y, x.z, __int_as_float(best));
-                    a.ps.hit1[q] = make_float4(ray.d.x, ray.d.y, ray.d.z, tw);
-                    done = true;
-                } else if (next < 0) {
-                    a.ps.hit0[q] = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
-                    a.ps.hit1[q] = make_float4(ray.d.x, ray.d.y, ray.d.z, 0.f);
-                    done = true;
-                }
-            }
-            if (!done && a.g.continue_cells) {
-                // the lane carries the ray on into the neighbouring cell's
-                // BVH, with the same record it would have handed over
-                const int cell = next;
-                t_cur = fmaxf(t_cur, t_exit);
-                t_exit = cell_exit(g, cell, ray, next);
-                tmin = fmaxf(0.0f, t_cur - g.eps);
-                node = __ldg(g.root + cell);
-                sp = 0;
-                best = -1;
-                occ = false;
-                rfl = rfl_next;
-                n_prev = cr.n;
-                tw = (rfl & kRayShadow) ? fminf(t_exit + g.eps, t_max) : t_exit + g.eps;
-                ++n_cross;
-                ++n_vis;
-                if (COUNT) ++n_cont;
-                done = true;
-                fin = false;
-            } else {
-                if (!done) {
-                    want = true;
-                    o0 = make_float4(ray.o.x, ray.o.y, ray.o.z, fmaxf(t_cur, t_exit));
-                    o1 = make_float4(ray.d.x, ray.d.y, ray.d.z, t_max);
-                    o2 = make_int4(q, excl, rfl_next, next);
-                    ++n_cross;
-                }
-                idx = -1;
-            }
-        }
-        if (want && a.last_wave) {   // cannot happen: each wave moves a ray forward along one axis
-            atomicCAS(a.err, 0, 4);
-            want = false;
-        }
-        // hand-off: append to the warp's buffer, flushing it to the staging
-        // area (one atomic, coalesced stores) when the new rays do not fit
-        const unsigned mw = __ballot_sync(full, want);
-        if (mw) {
-            const int n = __popc(mw);
-            if (nbuf + n > kPushBuf) {
-                flush_push_buf(Q, pbuf, nbuf, lane, a.err);
-                nbuf = 0;
-            }
-            if (want) {
-                float4 *slot = pbuf + 3 * (nbuf + __popc(mw & lt_mask));
-                slot[0] = o0;
-                slot[1] = o1;
-                slot[2] = make_float4(__int_as_float(o2.x), __int_as_float(o2.y), __int_as_float(o2.z),
-                                      __int_as_float(o2.w));
-                const int bin = ray_bin(g, next, o2.z, o0, o1);
-                const unsigned peers = __match_any_sync(mw, bin);
-                if (lane == __ffs(peers) - 1) atomicAdd(Q.cnt + bin, __popc(peers));
-            }
-            nbuf += n;
-            __syncwarp();
         }
     }
     if (nbuf > 0) flush_push_buf(Q, pbuf, nbuf, lane, a.err);

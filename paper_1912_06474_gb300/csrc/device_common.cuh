@@ -51,19 +51,31 @@ __device__ __forceinline__ float u01(uint32_t x) { return (float)(x >> 8) * (1.0
 // Node = 4 float4: (c0.lo.x, c0.hi.x, c0.lo.y, c0.hi.y) (c1 same) (c0.lo.z, c0.hi.z,
 // c1.lo.z, c1.hi.z) (child0, child1 as int bits). child >= 0: node index;
 // child < 0: leaf, ~child = (first triangle << 4) | count.
-// Triangle = 3 float4: (v0, id) (v1, obj) (v2, flags): the vertices
-// themselves, so that triangles sharing an edge see bit-identical endpoints.
+// Triangle = 3 float4, one per axis: (v0, v1, v2 along x, key) (along y, key)
+// (along z, key), key = id, with bit 30 set on glass: the vertices themselves,
+// so that triangles sharing an edge see bit-identical endpoints. A ray reads
+// the rows in the order of its own axes (below).
+constexpr int kTriIdMask = (1 << 30) - 1;
+constexpr int kTriGlassBit = 1 << 30;
+struct TriRows {
+    float4 x, y, z;   // along the ray's kx, ky, kz
+    __device__ __forceinline__ int key() const { return __float_as_int(x.w); }
+};
 
 // A ray with what its box and triangle tests need: reciprocal direction and
 // origin times it (boxes), and the set-up of the watertight triangle test of
 // Woop, Benthin and Wald (JCGT 2013): the axis kz along which the direction is
-// largest, the other two kx, ky (swapped when d[kz] < 0, which keeps the
-// winding), and the shear (sx, sy) = (d[kx], d[ky]) / d[kz] that maps the
-// ray onto the +z axis of a frame centred on its origin; the scale 1 / d[kz]
-// is inv[kz] (|d[kz]| >= 1/sqrt(3) for a unit direction, never clamped).
+// largest, the next two kx, ky in cyclic order, the shear (sx, sy) = (d[kx],
+// d[ky]) / d[kz] that maps the ray onto the z axis of a frame centred on its
+// origin, the scale sz = 1 / d[kz] (|d[kz]| >= 1/sqrt(3) for a unit direction,
+// never clamped) and the origin in that axis order. For d[kz] < 0 the method
+// swaps kx and ky to keep the winding; exchanging them only negates U, V, W,
+// their sum and the scaled distance, each exactly, and the test looks at neither
+// sign, so the swap is left out.
 struct Ray {
-    V3 o, d, inv, oi;   // oi = o * inv
-    float sx, sy;
+    V3 inv, oi;         // oi = o * inv
+    float sx, sy, sz;
+    V3 po;              // o along kx, ky, kz
     int k;              // kx | ky << 2 | kz << 4
 };
 __device__ __forceinline__ float safe_inv(float d) {
@@ -72,40 +84,46 @@ __device__ __forceinline__ float safe_inv(float d) {
 __device__ __forceinline__ float comp(V3 v, int k) { return k == 0 ? v.x : (k == 1 ? v.y : v.z); }
 __device__ __forceinline__ Ray make_ray(V3 o, V3 d) {
     Ray r;
-    r.o = o;
-    r.d = d;
     r.inv = v3(safe_inv(d.x), safe_inv(d.y), safe_inv(d.z));
     r.oi = v3(o.x * r.inv.x, o.y * r.inv.y, o.z * r.inv.z);
     const float ax = fabsf(d.x), ay = fabsf(d.y), az = fabsf(d.z);
     const int kz = ax >= ay ? (ax >= az ? 0 : 2) : (ay >= az ? 1 : 2);
-    int kx = kz == 2 ? 0 : kz + 1, ky = kx == 2 ? 0 : kx + 1;
+    const int kx = kz == 2 ? 0 : kz + 1, ky = kx == 2 ? 0 : kx + 1;
     const float dz = comp(d, kz);
-    if (dz < 0.0f) {
-        const int t = kx;
-        kx = ky;
-        ky = t;
-    }
     r.sx = comp(d, kx) / dz;
     r.sy = comp(d, ky) / dz;
+    r.sz = comp(r.inv, kz);
+    r.po = v3(comp(o, kx), comp(o, ky), comp(o, kz));
     r.k = kx | (ky << 2) | (kz << 4);
     return r;
+}
+// Triangle record i in the ray's axis order: the permutation is in the
+// addresses, not in selects of the nine coordinates.
+__device__ __forceinline__ TriRows load_tri(const float4 *__restrict__ tris, int i, const Ray &r) {
+    const float4 *tp = tris + 3 * i;
+    return TriRows{__ldg(tp + (r.k & 3)), __ldg(tp + ((r.k >> 2) & 3)), __ldg(tp + (r.k >> 4))};
+}
+// Whether a ray of direction d leaves the (glass) triangle's front side.
+__device__ __forceinline__ bool tri_leaving(const float4 *__restrict__ tris, int i, V3 d) {
+    const float4 *tp = tris + 3 * i;
+    const float4 x = __ldg(tp), y = __ldg(tp + 1), z = __ldg(tp + 2);
+    const V3 a = v3(x.x, y.x, z.x);
+    return dot(d, cross(v3(x.y, y.y, z.y) - a, v3(x.z, y.z, z.z) - a)) >= 0.0f;
 }
 
 // Watertight ray/triangle test (Woop, Benthin, Wald 2013), double sided:
 // the vertices are taken relative to the ray origin and sheared so that the
-// ray runs along +z; the signed edge functions U, V, W of the projected
+// ray runs along z; the signed edge functions U, V, W of the projected
 // triangle decide inside/outside. Each is a difference of two correctly
 // rounded products, so a shared edge gives its two triangles edge functions
 // of exactly opposite sign and a ray through it cannot slip between them;
 // an exact zero is re-evaluated in double precision. Returns the hit
 // distance, or +inf.
-__device__ __forceinline__ float wt_intersect(const Ray &r, V3 p0, V3 p1, V3 p2) {
-    const int kx = r.k & 3, ky = (r.k >> 2) & 3, kz = r.k >> 4;
-    const V3 A = p0 - r.o, B = p1 - r.o, C = p2 - r.o;
-    const float Az = comp(A, kz), Bz = comp(B, kz), Cz = comp(C, kz);
-    const float Ax = fmaf(-r.sx, Az, comp(A, kx)), Ay = fmaf(-r.sy, Az, comp(A, ky));
-    const float Bx = fmaf(-r.sx, Bz, comp(B, kx)), By = fmaf(-r.sy, Bz, comp(B, ky));
-    const float Cx = fmaf(-r.sx, Cz, comp(C, kx)), Cy = fmaf(-r.sy, Cz, comp(C, ky));
+__device__ __forceinline__ float wt_intersect(const Ray &r, const TriRows &p) {
+    const float Az = p.z.x - r.po.z, Bz = p.z.y - r.po.z, Cz = p.z.z - r.po.z;
+    const float Ax = fmaf(-r.sx, Az, p.x.x - r.po.x), Ay = fmaf(-r.sy, Az, p.y.x - r.po.y);
+    const float Bx = fmaf(-r.sx, Bz, p.x.y - r.po.x), By = fmaf(-r.sy, Bz, p.y.y - r.po.y);
+    const float Cx = fmaf(-r.sx, Cz, p.x.z - r.po.x), Cy = fmaf(-r.sy, Cz, p.y.z - r.po.y);
     float U = __fsub_rn(__fmul_rn(Cx, By), __fmul_rn(Cy, Bx));
     float V = __fsub_rn(__fmul_rn(Ax, Cy), __fmul_rn(Ay, Cx));
     float W = __fsub_rn(__fmul_rn(Bx, Ay), __fmul_rn(By, Ax));
@@ -117,9 +135,21 @@ __device__ __forceinline__ float wt_intersect(const Ray &r, V3 p0, V3 p1, V3 p2)
     if (fminf(U, fminf(V, W)) < 0.0f && fmaxf(U, fmaxf(V, W)) > 0.0f) return __int_as_float(0x7f800000);
     const float det = U + V + W;
     if (det == 0.0f) return __int_as_float(0x7f800000);
-    const float sz = comp(r.inv, kz);
-    const float T = fmaf(U, sz * Az, fmaf(V, sz * Bz, W * (sz * Cz)));
+    const float T = fmaf(U, r.sz * Az, fmaf(V, r.sz * Bz, W * (r.sz * Cz)));
     return T / det;
+}
+
+// Three-operand minimum and maximum (one instruction on sm_100 and later, at the
+// rate of the two-operand form; a NaN operand is ignored as by fminf / fmaxf).
+__device__ __forceinline__ float fmin3(float a, float b, float c) {
+    float d;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+__device__ __forceinline__ float fmax3(float a, float b, float c) {
+    float d;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
 }
 
 // Slab test of both children of a node against [tmin, tmax]: hit flags and entry distances.
@@ -131,10 +161,10 @@ __device__ __forceinline__ void child_boxes(const Ray &r, float4 n0, float4 n1, 
     float bx0 = fmaf(n1.x, r.inv.x, -r.oi.x), bx1 = fmaf(n1.y, r.inv.x, -r.oi.x);
     float by0 = fmaf(n1.z, r.inv.y, -r.oi.y), by1 = fmaf(n1.w, r.inv.y, -r.oi.y);
     float bz0 = fmaf(n2.z, r.inv.z, -r.oi.z), bz1 = fmaf(n2.w, r.inv.z, -r.oi.z);
-    float alo = fmaxf(fmaxf(fminf(ax0, ax1), fminf(ay0, ay1)), fmaxf(fminf(az0, az1), tmin));
-    float ahi = fminf(fminf(fmaxf(ax0, ax1), fmaxf(ay0, ay1)), fminf(fmaxf(az0, az1), tmax));
-    float blo = fmaxf(fmaxf(fminf(bx0, bx1), fminf(by0, by1)), fmaxf(fminf(bz0, bz1), tmin));
-    float bhi = fminf(fminf(fmaxf(bx0, bx1), fmaxf(by0, by1)), fminf(fmaxf(bz0, bz1), tmax));
+    const float alo = fmax3(fminf(ax0, ax1), fminf(ay0, ay1), fmaxf(fminf(az0, az1), tmin));
+    const float ahi = fmin3(fmaxf(ax0, ax1), fmaxf(ay0, ay1), fminf(fmaxf(az0, az1), tmax));
+    const float blo = fmax3(fminf(bx0, bx1), fminf(by0, by1), fmaxf(fminf(bz0, bz1), tmin));
+    const float bhi = fmin3(fmaxf(bx0, bx1), fmaxf(by0, by1), fminf(fmaxf(bz0, bz1), tmax));
     h0 = alo <= ahi;
     h1 = blo <= bhi;
     t0 = alo;
@@ -156,8 +186,8 @@ struct TravCount {
 };
 template <bool COUNT = false>
 __device__ __forceinline__ Hit trace_closest(const float4 *__restrict__ nodes, const float4 *__restrict__ tris,
-                                             int root, const Ray &r, float tmin, float tmax, int excl_prim,
-                                             int excl_obj, TravCount *cnt = nullptr) {
+                                             const int *__restrict__ tri_obj, int root, const Ray &r, float tmin,
+                                             float tmax, int excl_prim, int excl_obj, TravCount *cnt = nullptr) {
     Hit h;
     h.t = tmax;
     h.prim = -1;
@@ -187,12 +217,11 @@ __device__ __forceinline__ Hit trace_closest(const float4 *__restrict__ nodes, c
             int v = ~node;
             int first = v >> kLeafBits, count = v & ((1 << kLeafBits) - 1);
             for (int i = 0; i < count; ++i) {
-                const float4 *tp = tris + 3 * (first + i);
-                float4 a = __ldg(tp), b = __ldg(tp + 1), c = __ldg(tp + 2);
-                int id = __float_as_int(a.w);
-                if (id == excl_prim || (excl_obj >= 0 && __float_as_int(b.w) == excl_obj)) continue;
+                const TriRows tr = load_tri(tris, first + i, r);
+                const int id = tr.key() & kTriIdMask;
+                if (id == excl_prim || (excl_obj >= 0 && __ldg(tri_obj + id) == excl_obj)) continue;
                 if (COUNT) ++cnt->tris;
-                float t = wt_intersect(r, xyz(a), xyz(b), xyz(c));
+                const float t = wt_intersect(r, tr);
                 if (t > tmin && (t < h.t || (t == h.t && id < h.prim))) {
                     h.t = t;
                     h.prim = id;
@@ -216,8 +245,8 @@ struct Crossings {
 };
 template <bool COUNT = false>
 __device__ __forceinline__ bool trace_shadow(const float4 *__restrict__ nodes, const float4 *__restrict__ tris,
-                                             int root, const Ray &r, float tmin, float tmax, int excl_prim,
-                                             Crossings &cr, TravCount *cnt = nullptr) {
+                                             const int *__restrict__ tri_obj, int root, const Ray &r, V3 d, float tmin,
+                                             float tmax, int excl_prim, Crossings &cr, TravCount *cnt = nullptr) {
     int stack[kStackSize];
     int sp = 0;
     int node = root;
@@ -243,16 +272,15 @@ __device__ __forceinline__ bool trace_shadow(const float4 *__restrict__ nodes, c
             int v = ~node;
             int first = v >> kLeafBits, count = v & ((1 << kLeafBits) - 1);
             for (int i = 0; i < count; ++i) {
-                const float4 *tp = tris + 3 * (first + i);
-                float4 a = __ldg(tp), b = __ldg(tp + 1), c = __ldg(tp + 2);
-                int id = __float_as_int(a.w);
+                const TriRows tr = load_tri(tris, first + i, r);
+                const int id = tr.key() & kTriIdMask;
                 if (id == excl_prim) continue;
                 if (COUNT) ++cnt->tris;
-                float t = wt_intersect(r, xyz(a), xyz(b), xyz(c));
+                const float t = wt_intersect(r, tr);
                 if (!(t > tmin && t <= tmax)) continue;
-                if (!(__float_as_uint(c.w) & kTriGlass)) return true;
-                if (dot(r.d, cross(xyz(b) - xyz(a), xyz(c) - xyz(a))) >= 0.0f) continue;   // leaving face
-                int ob = __float_as_int(b.w);
+                if (!(tr.key() & kTriGlassBit)) return true;
+                if (tri_leaving(tris, first + i, d)) continue;
+                const int ob = __ldg(tri_obj + id);
                 bool seen = false;
                 for (int q = 0; q < cr.n; ++q) seen |= cr.obj[q] == ob;
                 if (seen) continue;

@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(128) k_megakernel(MegaArgs a) {
     for (int b = 1; b <= ri.max_depth; ++b) {
         Ray ray = make_ray(o, d);
         ++n_ext;
-        Hit h = trace_closest<COUNT>(sc.g_nodes, sc.g_tris, 0, ray, 0.0f, __int_as_float(0x7f800000), excl_prim,
+        Hit h = trace_closest<COUNT>(sc.g_nodes, sc.g_tris, sc.tri_obj, 0, ray, 0.0f, __int_as_float(0x7f800000), excl_prim,
                                            excl_obj, &tc);
         if (b == 1) first = h.prim;
         if (h.prim < 0) break;
@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(128) k_megakernel(MegaArgs a) {
                     Crossings cr;
                     cr.n = 0;
                     Ray sray = make_ray(xo, w);
-                    bool occ = trace_shadow<COUNT>(sc.g_nodes, sc.g_tris, 0, sray, 0.0f,
+                    bool occ = trace_shadow<COUNT>(sc.g_nodes, sc.g_tris, sc.tri_obj, 0, sray, w, 0.0f,
                                                    (1.0f - kShadowShorten) * dist, h.prim, cr, &tc);
                     if (!occ) {
                         const float G = cx * cy / (dist * dist) * sc.light_area * (1.0f / 3.14159265358979f);

@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(128) k_photon_trace(DevScene sc, PhotonTraceAr
     for (int b = 1; b <= D - 1; ++b) {
         const Ray ray = make_ray(o, d);
         ++segs;
-        const Hit h = trace_closest(sc.g_nodes, sc.g_tris, 0, ray, 0.0f, __int_as_float(0x7f800000), excl_prim,
+        const Hit h = trace_closest(sc.g_nodes, sc.g_tris, sc.tri_obj, 0, ray, 0.0f, __int_as_float(0x7f800000), excl_prim,
                                     excl_obj);
         if (h.prim < 0) break;
         const float4 tn = __ldg(sc.tri_n + h.prim);

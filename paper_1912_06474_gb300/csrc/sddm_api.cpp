@@ -553,6 +553,25 @@ int sddm_build(sddm_ctx *ctx, const sddm_build_opts *opts) {
     if (tri_base_check >= (1LL << (31 - kLeafBits)) || (int64_t)global.tris.size() / 3 >= (1LL << (31 - kLeafBits)))
         return fail(SDDM_ERR_INVALID_ARG, "sddm_build: too many triangle references for the leaf encoding");
 
+    // the kernels' triangle records: a row per axis with the three vertices'
+    // coordinates and the key (id, bit 30 set on glass)
+    auto rows_by_axis = [](std::vector<float4> &v) {
+        for (size_t k = 0; k + 2 < v.size(); k += 3) {
+            const float4 p = v[k], q = v[k + 1], r = v[k + 2];
+            uint32_t key, flags;
+            std::memcpy(&key, &p.w, 4);
+            std::memcpy(&flags, &r.w, 4);
+            if (flags & kTriGlass) key |= 1u << 30;
+            float w;
+            std::memcpy(&w, &key, 4);
+            v[k] = make_float4(p.x, q.x, r.x, w);
+            v[k + 1] = make_float4(p.y, q.y, r.y, w);
+            v[k + 2] = make_float4(p.z, q.z, r.z, w);
+        }
+    };
+    rows_by_axis(global.tris);
+    rows_by_axis(cell_tris);
+
     // --- upload
     cudaStream_t s = ctx->stream;
     if ((e = ctx->d_wcmf.upload(wcmf, s)) || (e = ctx->d_tab.upload(tab, s)) || (e = ctx->d_lam.upload(ctx->lam, s)) ||

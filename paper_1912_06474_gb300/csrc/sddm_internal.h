@@ -37,7 +37,7 @@ constexpr uint32_t kSlotProbe = 0x10004u;
 constexpr float kRayOffset = 1e-4f;       // metres along the geometric normal
 constexpr float kShadowShorten = 1e-4f;   // shadow rays end at (1 - 1e-4) * distance
 
-// Triangle flag bits stored in the .w of the third float4 of a packed triangle.
+// Triangle flag bits of the builder's records.
 constexpr uint32_t kTriGlass = 1u;
 
 // Device view of the scene: plain pointers into context-owned device memory.
@@ -68,7 +68,7 @@ struct DevScene {
     float light_area;
     // global BVH (single domain)
     const float4 *g_nodes;    // [n][4]
-    const float4 *g_tris;     // [refs][3]
+    const float4 *g_tris;     // [refs][3], a row per axis
 };
 
 // Per-render constants (device copy in a table).
