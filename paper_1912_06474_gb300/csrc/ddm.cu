@@ -248,7 +248,8 @@ __global__ void __launch_bounds__(256) k_camera(KArgs a) {
             const int r = find_render(a.rb, gp);
             const RenderInfo &ri = a.rb.info[r];
             const int64_t local = gp - ri.path_begin;
-            const uint32_t p = (uint32_t)(local / ri.spp), j = (uint32_t)(local % ri.spp);
+            uint32_t p, j;
+            pixel_sample(local, ri.spp, p, j);
             const int px = (int)(p % (uint32_t)ri.width), py = (int)(p / (uint32_t)ri.width);
             uint4 x = philox4x32_10(make_uint4(p, j, 0u, kSlotCamera), ri.seed, ri.render_id);
             V3 o, d;
@@ -572,6 +573,7 @@ __device__ __forceinline__ float3 spec_chunk(const KArgs &a, const SpecRec &rec,
         const Float4 rho = ld4(tab + rec.r_rho * n_chunk), le = ld4(tab + rec.r_le * n_chunk);
         const float G = rec.G;
         Float4 tr{{1.f, 1.f, 1.f, 1.f}};
+#pragma unroll 1
         for (int k = 0; k < rec.ncr; ++k) {
             const int cq = rec.cq[k];
             if (!DIRECT || cq >= 0) {
@@ -645,6 +647,7 @@ __device__ __forceinline__ void spec_items(const KArgs &a, const SpecRec *rec, f
                          : "memory");
     }
     asm volatile("cp.async.wait_all;" ::: "memory");   // a lane reads only what it fetched itself
+#pragma unroll 1
     for (int i = lane; i < n_item; i += 32) {
         const int j = (int)((unsigned)i * inv_chunk >> 16);
         const float3 s = spec_chunk<FILMS, DIRECT>(a, rec[j], i - j * n_chunk, part[i]);
@@ -761,6 +764,7 @@ __global__ void __launch_bounds__(kSpecThreads, SDDM_SHS_MINB) k_shade_spectral(
         const bool any_direct = __any_sync(full, me.flags & kSrDirect);
         if (me.flags) rec[mine] = me;
         __syncwarp();
+#pragma unroll 1
         for (int r0 = 0; r0 < n_rec; r0 += per_pass) {
             const int nr = min(per_pass, n_rec - r0), n_item = nr * n_chunk;
             if (!any_direct)
@@ -817,6 +821,7 @@ __global__ void __launch_bounds__(256, SDDM_SHC_MINB) k_shade_continue(KArgs a) 
     unsigned long long n_ext = 0, n_sh = 0, n_glass = 0;
     const PathState &ps = a.ps;
     __shared__ PushSmem psm;
+    __shared__ float s_terms[8][kBranchTerms];
     int *bins = block_bins_init(a.g.n_bins);
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < np; base += stride) {   // block-uniform trips
         const int64_t q = base + threadIdx.x;
@@ -825,18 +830,21 @@ __global__ void __launch_bounds__(256, SDDM_SHC_MINB) k_shade_continue(KArgs a) 
         float4 e0 = make_float4(0, 0, 0, 0), e1 = e0, s0 = e0, s1 = e0;
         int4 e2 = make_int4(0, 0, 0, 0), s2 = e2;
         int fl = q < np ? ps.flags[q] : 0;
+        bool spec = false, glass = false;   // a mirror or glass vertex to continue from
+        int prim = -1, mat = 0;
+        V3 x = v3(0, 0, 0), d = x, ng = x, ns = x;
+        float cd = 0.f, u_glass = 0.f;
         if (fl & (kFlExt | kFlShadow)) {
             const int64_t gp = a.path_begin + q;
             const int r = find_render(a.rb, gp);
             const RenderInfo &ri = a.rb.info[r];
             const int64_t local = gp - ri.path_begin;
-            const uint32_t p = (uint32_t)(local / ri.spp), j = (uint32_t)(local % ri.spp);
+            uint32_t p, j;
+            pixel_sample(local, ri.spp, p, j);
 
             // (3) the hit of this vertex
             bool has_hit = false;
-            int prim = -1, mat = 0, kind = 0;
-            V3 x = v3(0, 0, 0), d = x, ng = x, ns = x;
-            float cd = 0.f;
+            int kind = 0;
             if ((fl & kFlExt) && b <= ri.max_depth) {
                 const float4 h0 = ps.hit0[q], h1 = ps.hit1[q];
                 prim = __float_as_int(h0.w);
@@ -863,6 +871,7 @@ __global__ void __launch_bounds__(256, SDDM_SHC_MINB) k_shade_continue(KArgs a) 
                         uint4 xl = philox4x32_10(make_uint4(p, j, (uint32_t)b, kSlotLight), k0, k1);
                         const float ua = u01(xl.x), su = sqrtf(u01(xl.y)), u2 = u01(xl.z);
                         int li = sc.n_light - 1;
+#pragma unroll 1
                         for (int k = 0; k < sc.n_light; ++k)
                             if (ua < __ldg(sc.light_cdf + k)) { li = k; break; }
                         const float4 lv0 = __ldg(sc.light_v + 3 * li), lv1 = __ldg(sc.light_v + 3 * li + 1),
@@ -913,44 +922,49 @@ __global__ void __launch_bounds__(256, SDDM_SHC_MINB) k_shade_continue(KArgs a) 
                         }
                     }
                 } else if (b < ri.max_depth) {
-                    const float c = fabsf(cd);
-                    V3 dn = d, on;
-                    int excl = prim;
-                    ps.pend_mat[q] = mat;
-                    ps.pend_cos[q] = c;
-                    if (kind == kConductor) {
-                        dn = d - (2.0f * cd) * ng;
-                        on = x + kRayOffset * ns;
-                        ps.pend_w[q] = 1.0f;
-                    } else {
-                        const float pr = branch_proxy(c, L, sc.mat_a + (size_t)mat * L);
-                        uint4 xg = philox4x32_10(make_uint4(p, j, (uint32_t)b, kSlotGlass), k0, k1);
-                        const bool refl = u01(xg.x) < pr;
-                        ++n_glass;
-                        if (refl) {
-                            dn = d - (2.0f * cd) * ng;
-                            on = x + kRayOffset * ns;
-                            ps.pend_w[q] = -1.0f / pr;
-                        } else {
-                            on = x - kRayOffset * ns;
-                            excl = -__ldg(sc.tri_obj + prim) - 2;
-                            ps.pend_w[q] = 1.0f / (1.0f - pr);
-                        }
-                    }
+                    spec = true;
                     nfl |= kFlPend | kFlPrevSpec | kFlExt;
                     ++n_ext;
-                    float t0;
-                    if (grid_enter(a.g, on, dn, __int_as_float(0x7f800000), t0, cell_e)) {
-                        want_e = true;
-                        e0 = make_float4(on.x, on.y, on.z, t0);
-                        e1 = make_float4(dn.x, dn.y, dn.z, __int_as_float(0x7f800000));
-                        e2 = make_int4((int)q, excl, 0, cell_e);
+                    ps.pend_mat[q] = mat;
+                    ps.pend_cos[q] = fabsf(cd);
+                    if (kind == kConductor) {
+                        ps.pend_w[q] = 1.0f;
                     } else {
-                        ps.hit0[q] = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
+                        glass = true;
+                        ++n_glass;
+                        const uint4 xg = philox4x32_10(make_uint4(p, j, (uint32_t)b, kSlotGlass), k0, k1);
+                        u_glass = u01(xg.x);
                     }
                 }
             }
             ps.flags[q] = nfl;
+        }
+        // mirror or glass: the next direction, the glass branch by the whole warp
+        if (__any_sync(0xffffffffu, spec)) {
+            const float pr = warp_branch_proxy(glass, fabsf(cd), L, sc.mat_a + (size_t)mat * L, s_terms[threadIdx.x >> 5]);
+            if (spec) {
+                V3 dn = d - (2.0f * cd) * ng, on = x + kRayOffset * ns;
+                int excl = prim;
+                if (glass) {
+                    if (u_glass < pr) {
+                        ps.pend_w[q] = -1.0f / pr;
+                    } else {
+                        dn = d;
+                        on = x - kRayOffset * ns;
+                        excl = -__ldg(sc.tri_obj + prim) - 2;
+                        ps.pend_w[q] = 1.0f / (1.0f - pr);
+                    }
+                }
+                float t0;
+                if (grid_enter(a.g, on, dn, __int_as_float(0x7f800000), t0, cell_e)) {
+                    want_e = true;
+                    e0 = make_float4(on.x, on.y, on.z, t0);
+                    e1 = make_float4(dn.x, dn.y, dn.z, __int_as_float(0x7f800000));
+                    e2 = make_int4((int)q, excl, 0, cell_e);
+                } else {
+                    ps.hit0[q] = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
+                }
+            }
         }
         block_stage_push2(a.Q, a.g, psm, bins, want_e, cell_e, e0, e1, e2, want_s, cell_s, s0, s1, s2, a.err);
     }

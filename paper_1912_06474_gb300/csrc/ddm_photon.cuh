@@ -98,6 +98,7 @@ __global__ void __launch_bounds__(256) k_photon_shade(KArgs a, PhotonPass pp) {
     unsigned long long n_ext = 0;
     __shared__ PushSmem psm;
     int *bins = block_bins_init(a.g.n_bins);
+    __shared__ float s_terms[8][kBranchTerms];
     const bool staged = L <= kStageMaxL;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     float *stage = reinterpret_cast<float *>(bins + ((a.g.n_bins + 3) & ~3)) + (size_t)w * L * 33;
@@ -129,6 +130,23 @@ __global__ void __launch_bounds__(256) k_photon_shade(KArgs a, PhotonPass pp) {
                 }
                 __syncwarp();
             }
+        }
+        // the glass branch of the warp's photons that stand on glass
+        float pr = 0.f;
+        {
+            bool glass = false;
+            float c = 0.f;
+            int mat = 0;
+            if ((fl & kFlExt) && b < D - 1) {
+                const int prim = __float_as_int(a.ps.hit0[q].w);
+                if (prim >= 0) {
+                    const float4 tn = __ldg(sc.tri_n + prim);
+                    mat = __float_as_int(tn.w);
+                    glass = __ldg(sc.mat_kind + mat) == kGlass;
+                    if (glass) c = fabsf(dot(xyz(a.ps.hit1[q]), xyz(tn)));
+                }
+            }
+            pr = warp_branch_proxy(glass, c, L, sc.mat_a + (size_t)mat * L, s_terms[w]);
         }
         if (fl & kFlExt) {
             int nfl = 0;
@@ -177,7 +195,6 @@ __global__ void __launch_bounds__(256) k_photon_shade(KArgs a, PhotonPass pp) {
                 } else if (kind == kGlass) {
                     if (b < D - 1) {
                         const float c = fabsf(cd);
-                        const float pr = branch_proxy(c, L, mA);
                         uint4 xg = philox4x32_10(make_uint4(pi, pj, (uint32_t)b, kSlotGlass), pp.seed, pp.render_id);
                         const bool refl = u01(xg.x) < pr;
                         const float st = __ldg(pp.state_s + mat), th = __ldg(sc.mat_thick + mat);

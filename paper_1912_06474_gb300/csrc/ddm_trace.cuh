@@ -129,14 +129,6 @@ __device__ __forceinline__ void flush_push_buf(const Queues &Q, const float4 *bu
 #define SDDM_TRACE_MIN_BLOCKS 7
 #endif
 
-// First device check to fail records its code and two details in the error word.
-__device__ __forceinline__ void trace_check_fail(int *err, int code, int x, int y) {
-    if (atomicCAS(err, 0, code) == 0) {
-        err[1] = x;
-        err[2] = y;
-    }
-}
-
 // CHECKED (the subdomain cache, whose cells move between loads): every root,
 // child and leaf index is checked against the records the cache holds before
 // it is read; a bad one is recorded (codes 8-10) and the ray is dropped.
@@ -165,28 +157,31 @@ __global__ void __launch_bounds__(128, SDDM_TRACE_MIN_BLOCKS) k_trace_wave(KArgs
     unsigned long long *run = s_run[threadIdx.x >> 5];
     if (lane == 0) run[0] = run[1] = 0;
     __syncwarp();
-    Ray ray;
     // what a lane carries through the traversal; the rest of its ray (direction,
     // range, path slot, exclusion) is read again from the queue when it finishes
-    float t_cur = 0.f, t_exit = 0.f, tmin = 0.f, tw = 0.f;
-    int rfl = 0, next = -1, node = 0, sp = 0, best = -1, ep = -1, eo = -1;
-    bool occ = false, fin = false;
-    Crossings cr;
+    LaneTrav t;
+    t.tmin = t.tw = 0.f;
+    t.node = t.sp = 0;
+    t.best = t.ep = t.eo = -1;
+    t.occ = t.fin = false;
+    Crossings cr;   // slabs a shadow ray has crossed
     cr.n = 0;
+    float t_cur = 0.f, t_exit = 0.f;
+    int rfl = 0, next = -1;
     int stack[kStackSize];
 
     for (;;) {
         // 1. results, hand-offs and refills, once enough lanes wait for them
-        const unsigned m_fin = __ballot_sync(full, fin);
+        const unsigned m_fin = __ballot_sync(full, t.fin);
         const unsigned m_need = __ballot_sync(full, idx < 0 && !exhausted);
-        const unsigned m_busy = __ballot_sync(full, idx >= 0 && !fin);
+        const unsigned m_busy = __ballot_sync(full, idx >= 0 && !t.fin);
         if (m_busy == 0 || __popc(m_fin | m_need) >= kTraceBatch) {
             if ((m_fin | m_need) == 0) break;
             // 1a. finished lanes: final result, or hand-off to the neighbouring cell
             bool want = false;
             float4 o0 = make_float4(0, 0, 0, 0), o1 = o0;
             int4 o2 = make_int4(0, 0, 0, 0);
-            if (fin) {
+            if (t.fin) {
                 const float4 *src = Q.in + 3 * (size_t)idx;
                 const float4 r0 = src[0], r1 = src[1];
                 const float2 r2f = *reinterpret_cast<const float2 *>(src + 2);
@@ -204,7 +199,7 @@ __global__ void __launch_bounds__(128, SDDM_TRACE_MIN_BLOCKS) k_trace_wave(KArgs
                         a.ps.cross_mat[k * np + q] = __float_as_int(cn.w);
                         a.ps.cross_cos[k * np + q] = -dot(rd, xyz(cn));
                     }
-                    if (occ) {
+                    if (t.occ) {
                         a.ps.sh_status[q] = kShadowOccluded;
                         done = true;
                     } else if (t_exit + g.eps >= t_max || next < 0) {
@@ -213,10 +208,10 @@ __global__ void __launch_bounds__(128, SDDM_TRACE_MIN_BLOCKS) k_trace_wave(KArgs
                     }
                     rfl_next = (rfl & 1) | (cr.n << 1);
                 } else {
-                    if (best >= 0) {
-                        const V3 x = ro + tw * rd;
-                        a.ps.hit0[q] = make_float4(x.x, x.y, x.z, __int_as_float(best));
-                        a.ps.hit1[q] = make_float4(rd.x, rd.y, rd.z, tw);
+                    if (t.best >= 0) {
+                        const V3 x = ro + t.tw * rd;
+                        a.ps.hit0[q] = make_float4(x.x, x.y, x.z, __int_as_float(t.best));
+                        a.ps.hit1[q] = make_float4(rd.x, rd.y, rd.z, t.tw);
                         done = true;
                     } else if (next < 0) {
                         a.ps.hit0[q] = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
@@ -224,20 +219,20 @@ __global__ void __launch_bounds__(128, SDDM_TRACE_MIN_BLOCKS) k_trace_wave(KArgs
                         done = true;
                     }
                 }
-                fin = false;
+                t.fin = false;
                 if (!done && a.g.continue_cells) {
                     // the lane carries the ray on into the neighbouring cell's
                     // BVH, with the same record it would have handed over
                     const int cell = next;
                     t_cur = fmaxf(t_cur, t_exit);
-                    t_exit = cell_exit(g, cell, ro, rd, ray.inv, next);
-                    tmin = fmaxf(0.0f, t_cur - g.eps);
-                    node = __ldg(g.root + cell);
-                    sp = 0;
-                    best = -1;
-                    occ = false;
+                    t_exit = cell_exit(g, cell, ro, rd, t.ray.inv, next);
+                    t.tmin = fmaxf(0.0f, t_cur - g.eps);
+                    t.node = __ldg(g.root + cell);
+                    t.sp = 0;
+                    t.best = -1;
+                    t.occ = false;
                     rfl = rfl_next;
-                    tw = (rfl & kRayShadow) ? fminf(t_exit + g.eps, t_max) : t_exit + g.eps;
+                    t.tw = (rfl & kRayShadow) ? fminf(t_exit + g.eps, t_max) : t_exit + g.eps;
                     ++n_cross;
                     if (COUNT) ++n_vis;
                     if (COUNT) ++n_cont;
@@ -319,27 +314,27 @@ __global__ void __launch_bounds__(128, SDDM_TRACE_MIN_BLOCKS) k_trace_wave(KArgs
                             q = 0;
                             cell = 0;
                         }
-                        ray = make_ray(xyz(r0), xyz(r1));
+                        t.ray = make_ray(xyz(r0), xyz(r1));
                         t_cur = r0.w;
-                        t_exit = cell_exit(g, cell, xyz(r0), xyz(r1), ray.inv, next);
-                        tmin = fmaxf(0.0f, t_cur - g.eps);
-                        node = __ldg(g.root + cell);
-                        if (CHECKED && (node < 0 || node >= g.node_cap)) {
-                            trace_check_fail(a.err, 8, cell, node);
-                            node = ~0;   // an empty leaf: the ray ends here
+                        t_exit = cell_exit(g, cell, xyz(r0), xyz(r1), t.ray.inv, next);
+                        t.tmin = fmaxf(0.0f, t_cur - g.eps);
+                        t.node = __ldg(g.root + cell);
+                        if (CHECKED && (t.node < 0 || t.node >= g.node_cap)) {
+                            trace_check_fail(a.err, 8, cell, t.node);
+                            t.node = ~0;   // an empty leaf: the ray ends here
                         }
-                        sp = 0;
-                        best = -1;
-                        occ = false;
+                        t.sp = 0;
+                        t.best = -1;
+                        t.occ = false;
                         if (COUNT) ++n_vis;
-                        ep = excl >= 0 ? excl : -1;
+                        t.ep = excl >= 0 ? excl : -1;
                         if (rfl & kRayShadow) {
-                            tw = fminf(t_exit + g.eps, r1.w);
+                            t.tw = fminf(t_exit + g.eps, r1.w);
                             cr.n = (rfl >> 1) & 7;
                             for (int k = 0; k < cr.n; ++k) cr.obj[k] = a.ps.cross_obj[k * np + q];
                         } else {
-                            tw = t_exit + g.eps;
-                            eo = excl <= -2 ? -excl - 2 : -1;
+                            t.tw = t_exit + g.eps;
+                            t.eo = excl <= -2 ? -excl - 2 : -1;
                         }
                     } else {
                         exhausted = true;
@@ -348,101 +343,10 @@ __global__ void __launch_bounds__(128, SDDM_TRACE_MIN_BLOCKS) k_trace_wave(KArgs
             }
         }
 
-        // 2. one traversal round, while-while: an interior phase in which the
-        //    lanes descend until most of them stand at a leaf (or their stacks
-        //    run out), then a leaf phase in which the lanes at a leaf test its
-        //    triangles.
-        const bool live = idx >= 0 && !fin;
-        const int n_live = __popc(__ballot_sync(full, live));
-        const bool shadow = (rfl & kRayShadow) != 0;
-        for (int it = 0; it < kTraceSteps; ++it) {
-            const bool act = live && !fin && node >= 0;
-            if (__popc(__ballot_sync(full, act)) * kTraceQuorum <= n_live) break;
-            if (act) {
-                if (COUNT) ++tc.nodes;
-                const float4 n0 = __ldg(g.nodes + 4 * node + 0), n1 = __ldg(g.nodes + 4 * node + 1),
-                             n2 = __ldg(g.nodes + 4 * node + 2), n3 = __ldg(g.nodes + 4 * node + 3);
-                float ta, tb;
-                bool ha, hb;
-                child_boxes(ray, n0, n1, n2, tmin, tw, ta, tb, ha, hb);
-                int ca = __float_as_int(n3.x), cb = __float_as_int(n3.y);
-                if (CHECKED) {
-                    if (ca >= g.node_cap) {
-                        trace_check_fail(a.err, 9, node, ca);
-                        ca = ~0;
-                    }
-                    if (cb >= g.node_cap) {
-                        trace_check_fail(a.err, 9, node, cb);
-                        cb = ~0;
-                    }
-                }
-                if (ha && hb) {
-                    const bool a_first = shadow || ta <= tb;
-                    if (sp < kStackSize) {
-                        stack[sp++] = a_first ? cb : ca;
-                    } else {
-                        atomicCAS(a.err, 0, 5);   // deeper than the builder allows
-                    }
-                    node = a_first ? ca : cb;
-                } else if (ha) {
-                    node = ca;
-                } else if (hb) {
-                    node = cb;
-                } else if (sp == 0) {
-                    fin = true;
-                } else {
-                    node = stack[--sp];
-                }
-            }
-        }
-        if (live && !fin && node < 0) {
-            const int v = ~node;
-            const int first = v >> kLeafBits;
-            int count = v & ((1 << kLeafBits) - 1);
-            if (CHECKED && (int64_t)first + count > g.tri_cap) {
-                trace_check_fail(a.err, 10, first, count);
-                count = 0;
-            }
-            for (int i = first; i < first + count; ++i) {
-                const TriRows tri = load_tri(g.tris, i, ray);
-                const int id = tri.key() & kTriIdMask;
-                if (id == ep) continue;
-                if (shadow) {
-                    if (COUNT) ++tc.tris;
-                    const float t = wt_intersect(ray, tri);
-                    if (!(t > tmin && t <= tw)) continue;
-                    if (!(tri.key() & kTriGlassBit)) {
-                        occ = true;
-                        break;
-                    }
-                    if (tri_leaving(g.tris, i, xyz(Q.in[3 * (size_t)idx + 1]))) continue;
-                    const int ob = __ldg(a.sc.tri_obj + id);
-                    bool seen = false;
-                    for (int k = 0; k < cr.n; ++k) seen |= cr.obj[k] == ob;
-                    if (seen) continue;
-                    if (cr.n >= kMaxCross) {
-                        occ = true;
-                        break;
-                    }
-                    cr.obj[cr.n] = ob;
-                    cr.tri[cr.n] = id;
-                    ++cr.n;
-                } else {
-                    if (eo >= 0 && __ldg(a.sc.tri_obj + id) == eo) continue;
-                    if (COUNT) ++tc.tris;
-                    const float t = wt_intersect(ray, tri);
-                    if (t > tmin && (t < tw || (t == tw && (best < 0 || id < best)))) {
-                        tw = t;
-                        best = id;
-                    }
-                }
-            }
-            if (occ || sp == 0) {
-                fin = true;
-            } else {
-                node = stack[--sp];
-            }
-        }
+        // 2. one traversal round
+        trav_round<COUNT, CHECKED, kTraceSteps, kTraceQuorum>(
+            g.nodes, g.tris, a.sc.tri_obj, t, cr, stack, idx >= 0 && !t.fin, (rfl & kRayShadow) != 0,
+            [&]() { return xyz(Q.in[3 * (size_t)idx + 1]); }, tc, a.err, g.node_cap, g.tri_cap);
     }
     if (nbuf > 0) flush_push_buf(Q, pbuf, nbuf, lane, a.err);
     block_count3(a.counters + 3, n_cross, nullptr, 0, nullptr, 0);

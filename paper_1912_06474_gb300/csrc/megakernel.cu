@@ -58,8 +58,10 @@ __device__ __forceinline__ void add_xyz(const DevScene &sc, int L, Kahan3 &acc, 
     acc.add(X.s, Y.s, Z.s);
 }
 
-template <int LT, bool COUNT, bool FILMS, bool PM>
-__global__ void __launch_bounds__(128) k_megakernel(MegaArgs a) {
+// The photon-mapped camera pass: a thread per path, which ends at its first
+// diffuse vertex, where it gathers the map.
+template <int LT, bool FILMS>
+__global__ void __launch_bounds__(128) k_megakernel_pm(MegaArgs a) {
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= a.path_count) return;
     const DevScene &sc = a.sc;
@@ -68,7 +70,8 @@ __global__ void __launch_bounds__(128) k_megakernel(MegaArgs a) {
     const int r = find_render(a.rb, gp);
     const RenderInfo &ri = a.rb.info[r];
     const int64_t local = gp - ri.path_begin;
-    const uint32_t p = (uint32_t)(local / ri.spp), j = (uint32_t)(local % ri.spp);
+    uint32_t p, j;
+    pixel_sample(local, ri.spp, p, j);
     const int px = (int)(p % (uint32_t)ri.width), py = (int)(p / (uint32_t)ri.width);
     const uint32_t k0 = ri.seed, k1 = ri.render_id;
 
@@ -84,14 +87,13 @@ __global__ void __launch_bounds__(128) k_megakernel(MegaArgs a) {
     int excl_prim = -1, excl_obj = -1;
     bool prev_specular = true;
     unsigned long long n_ext = 0, n_sh = 0, n_glass = 0;
-    TravCount tc;
     int first = -1;
 
     for (int b = 1; b <= ri.max_depth; ++b) {
         Ray ray = make_ray(o, d);
         ++n_ext;
-        Hit h = trace_closest<COUNT>(sc.g_nodes, sc.g_tris, sc.tri_obj, 0, ray, 0.0f, __int_as_float(0x7f800000), excl_prim,
-                                           excl_obj, &tc);
+        Hit h = trace_closest<false>(sc.g_nodes, sc.g_tris, sc.tri_obj, 0, ray, 0.0f, __int_as_float(0x7f800000), excl_prim,
+                                    excl_obj);
         if (b == 1) first = h.prim;
         if (h.prim < 0) break;
         const float4 tn = __ldg(sc.tri_n + h.prim);
@@ -132,8 +134,8 @@ __global__ void __launch_bounds__(128) k_megakernel(MegaArgs a) {
                     Crossings cr;
                     cr.n = 0;
                     Ray sray = make_ray(xo, w);
-                    bool occ = trace_shadow<COUNT>(sc.g_nodes, sc.g_tris, sc.tri_obj, 0, sray, w, 0.0f,
-                                                   (1.0f - kShadowShorten) * dist, h.prim, cr, &tc);
+                    bool occ = trace_shadow<false>(sc.g_nodes, sc.g_tris, sc.tri_obj, 0, sray, w, 0.0f,
+                                                   (1.0f - kShadowShorten) * dist, h.prim, cr);
                     if (!occ) {
                         const float G = cx * cy / (dist * dist) * sc.light_area * (1.0f / 3.14159265358979f);
                         const float *Le = sc.mat_a + (size_t)__float_as_int(ln.w) * L;
@@ -159,20 +161,8 @@ __global__ void __launch_bounds__(128) k_megakernel(MegaArgs a) {
                     }
                 }
             }
-            if constexpr (PM) {
-                pm_radiance_xyz(a.pm, a.pmc, xh, ns, L, rho, sc.wcmf, [&](int i) { return T.v[i]; }, acc);
-                break;
-            }
-            if (b == ri.max_depth) break;
-            uint4 xb = philox4x32_10(make_uint4(p, j, (uint32_t)b, kSlotBsdf), k0, k1);
-            d = cosine_dir(ns, u01(xb.x), u01(xb.y));
-            for_bins<LT>(L, [&](int i) {
-                T.v[i] *= __ldg(rho + i);
-            });
-            o = xh + kRayOffset * ns;
-            excl_prim = h.prim;
-            excl_obj = -1;
-            prev_specular = false;
+            pm_radiance_xyz(a.pm, a.pmc, xh, ns, L, rho, sc.wcmf, [&](int i) { return T.v[i]; }, acc);
+            break;
         } else if (kind == kConductor) {
             if (b == ri.max_depth) break;
             const float c = fabsf(cd);
@@ -217,13 +207,455 @@ __global__ void __launch_bounds__(128) k_megakernel(MegaArgs a) {
     if (a.first_prim) a.first_prim[g] = first;
     // counters: warp-aggregated when the whole warp is here, per thread otherwise
     if (!a.counters) return;
-    unsigned long long v[6] = {n_ext, n_sh, n_glass, tc.nodes, tc.tris, n_ext + n_sh};
-    const int nv = COUNT ? 6 : 3;
+    unsigned long long v[3] = {n_ext, n_sh, n_glass};
     if (__activemask() == 0xffffffffu) {
-        for (int k = 0; k < nv; ++k)
+        for (int k = 0; k < 3; ++k)
             for (int off = 16; off > 0; off >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], off);
         if ((threadIdx.x & 31) != 0) return;
     }
+    atomicAdd(a.counters + 0, v[0]);
+    atomicAdd(a.counters + 1, v[1]);
+    atomicAdd(a.counters + 2, v[2]);
+}
+
+// ---------------------------------------------------------- plain renders
+// Persistent warps, a path per lane. A thread per path left most of its warp
+// idle: 4.8 of 32 lanes per instruction (hotel room), since paths differ in
+// length, vertex kind and traversal and each walked its own bins. Here
+//  * a lane is a state machine of queries (trav_round, as in the DDM trace): an
+//    extension or shadow query runs in rounds with the other lanes', and once
+//    kMegaBatch lanes wait the warp stops to shade them, start their next
+//    queries and give lanes without a path the next one;
+//  * the spectral part of shading is done by the whole warp: each waiting lane
+//    leaves a record (emission, resolved shadow ray, weight), the rows of bins
+//    are dealt out to the lanes in chunks of four, as in the DDM's spectral pass,
+//    with the throughput rows in shared memory, a row per lane.
+// Hotel room, 512 x 512 x 4 spp, 41 bins: 10.2 -> 6.1 ms; tiny room, 400 x 400 x 6
+// spp, depth 6: 4.4 -> 3.4 ms; with a coated pane, 200 x 200 x 3 spp: 2.1 -> 0.96.
+// The loop holds all that a path meets, some 4000 instructions, and the
+// instruction cache bounds it on small scenes (2.7 of 9 stall cycles per
+// instruction): not unrolling its loops took the tiny room from 4.4 to 3.5 ms,
+// 32-bit path indices and one triangle test for both query kinds from 5.0 to 4.4
+// (pixel_sample, trav_round), the glass branch by the whole warp from 6.8 to 5.0
+// (warp_branch_proxy). Waiting lanes that stop the warp, 12 / 16 / 20 / 24 (hotel):
+// 8.0 (early version) / 6.04 / 6.06 / 6.25 ms, tiny room - / 3.54 / 3.41 / 3.35;
+// resident blocks 8 / 9 / 10 / 12: 6.0 / 6.3 / 5.9 / 6.4, tiny room 3.5 / 3.9 /
+// 3.9 / 4.7.
+struct __align__(16) MegaRec {
+    float G, pcos, pw;             // shadow ray's geometry factor; |cos| and branch weight at this vertex
+    int flags;                     // kMr* bits, 0 = nothing to do
+    int r_le, r_rho;               // table rows: light of the shadow ray; reflectance here (its weight too)
+    int r_w, r_w2;                 // table rows of a specular weight (n, k of a conductor; the glass)
+    int r_emit, ncr, r, pad;       // table row of the emitter hit; slabs crossed; render
+    int cmat[kMaxCross];           // their materials and cosines
+    float ccos[kMaxCross];
+};
+constexpr int kMrEmit = 1, kMrResolve = 2, kMrDiffuse = 4, kMrConductor = 8, kMrGlass = 16, kMrFirst = 32;
+#ifndef SDDM_MEGA_BATCH
+#define SDDM_MEGA_BATCH 20
+#endif
+#ifndef SDDM_MEGA_MIN_BLOCKS
+#define SDDM_MEGA_MIN_BLOCKS 8
+#endif
+constexpr int kMegaBatch = SDDM_MEGA_BATCH;
+constexpr int kMegaWarps = 2;      // warps of a block: small images spread over more SMs
+constexpr int kMegaItems = 96;     // chunks worked through between two sums
+static_assert(4 * kMegaItems >= kBranchTerms, "the two share their place");
+// What a lane needs only when the warp shades: the path's sums, and the
+// continuation ray while its vertex's shadow ray is under way.
+struct MegaWarp {
+    float acc[6][32];
+    float on[3][32], dn[3][32];
+    int xprim[32], xobj[32];
+    MegaRec rec[32];
+    float4 part[kMegaItems];   // also the glass branch's terms
+    int order[32];
+};
+__host__ __device__ constexpr size_t mega_warp_bytes(int Lp) { return sizeof(MegaWarp) + sizeof(float) * 32 * (size_t)Lp; }
+
+struct Quad {
+    float v[4];
+};
+__device__ __forceinline__ Quad ld_quad(const float4 *p) {
+    const float4 x = __ldg(p);
+    return Quad{{x.x, x.y, x.z, x.w}};
+}
+
+// One chunk of a lane's record: the XYZ it adds; its four throughput bins updated.
+template <bool FILMS>
+__device__ __forceinline__ float3 mega_chunk(const MegaArgs &a, const MegaRec &m, float4 *row, int ch) {
+    const DevScene &sc = a.sc;
+    const int n_chunk = sc.Lp >> 2, xf = m.flags;
+    const float4 *const tab = reinterpret_cast<const float4 *>(sc.tab) + ch;
+    Quad t{{1.f, 1.f, 1.f, 1.f}}, e{{0.f, 0.f, 0.f, 0.f}};
+    if (!(xf & kMrFirst)) {
+        const float4 v = row[ch];
+        t = Quad{{v.x, v.y, v.z, v.w}};
+    }
+    if (xf & kMrEmit) {
+        const Quad le = ld_quad(tab + m.r_emit * n_chunk);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) e.v[u] = t.v[u] * le.v[u];
+    }
+    if (xf & (kMrResolve | kMrDiffuse)) {
+        const Quad rho = ld_quad(tab + m.r_rho * n_chunk);
+        if (xf & kMrResolve) {
+            const Quad le = ld_quad(tab + m.r_le * n_chunk);
+            Quad tr{{1.f, 1.f, 1.f, 1.f}};
+#pragma unroll 1
+            for (int k = 0; k < m.ncr; ++k) {
+                const int cm = m.cmat[k];
+                const float st = __ldg(a.rb.state_s + (size_t)m.r * sc.n_mat + cm), th = __ldg(sc.mat_thick + cm);
+#pragma unroll 1
+                for (int u = 0; u < 4; ++u) {
+                    float R_, T_;
+                    glass_rt<FILMS>(sc, cm, min(4 * ch + u, sc.L - 1), m.ccos[k], st, th, R_, T_);
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) tr.v[x] *= x == u ? T_ : 1.0f;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) e.v[u] += t.v[u] * rho.v[u] * le.v[u] * m.G * tr.v[u];
+        }
+        if (xf & kMrDiffuse) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) t.v[u] *= rho.v[u];
+        }
+    }
+    if (xf & kMrConductor) {
+        const Quad n = ld_quad(tab + m.r_w * n_chunk), k = ld_quad(tab + m.r_w2 * n_chunk);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) t.v[u] *= conductor_F(m.pcos, n.v[u], k.v[u]);
+    } else if (xf & kMrGlass) {
+        const float st = __ldg(a.rb.state_s + (size_t)m.r * sc.n_mat + m.r_w), th = __ldg(sc.mat_thick + m.r_w);
+        const bool refl = m.pw < 0.0f;
+#pragma unroll 1
+        for (int u = 0; u < 4; ++u) {
+            float R_, T_;
+            glass_rt<FILMS>(sc, m.r_w, min(4 * ch + u, sc.L - 1), m.pcos, st, th, R_, T_);
+            const float w = (refl ? R_ : T_) * fabsf(m.pw);
+#pragma unroll
+            for (int x = 0; x < 4; ++x) t.v[x] *= x == u ? w : 1.0f;
+        }
+    }
+    if (xf & (kMrDiffuse | kMrConductor | kMrGlass)) row[ch] = make_float4(t.v[0], t.v[1], t.v[2], t.v[3]);
+    float3 s = make_float3(0.f, 0.f, 0.f);
+    if (xf & (kMrEmit | kMrResolve)) {
+        const float4 *const w = tab + 2 * sc.n_mat * n_chunk;
+        const Quad wx = ld_quad(w), wy = ld_quad(w + n_chunk), wz = ld_quad(w + 2 * n_chunk);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            s.x = fmaf(e.v[u], wx.v[u], s.x);
+            s.y = fmaf(e.v[u], wy.v[u], s.y);
+            s.z = fmaf(e.v[u], wz.v[u], s.z);
+        }
+    }
+    return s;
+}
+
+template <bool COUNT, bool FILMS>
+__global__ void __launch_bounds__(32 * kMegaWarps, SDDM_MEGA_MIN_BLOCKS) k_megakernel(const __grid_constant__ MegaArgs a) {
+    extern __shared__ __align__(16) unsigned char s_mega[];
+    const DevScene &sc = a.sc;
+    const int L = sc.L, Lp = sc.Lp, n_chunk = Lp >> 2, M = sc.n_mat;
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const unsigned lt_mask = (1u << lane) - 1u;
+    unsigned char *const mem = s_mega + mega_warp_bytes(Lp) * (threadIdx.x >> 5);
+    float4 *const rows = reinterpret_cast<float4 *>(mem);
+    MegaWarp &w = *reinterpret_cast<MegaWarp *>(mem + sizeof(float) * 32 * (size_t)Lp);
+    const int per_pass = kMegaItems / n_chunk;                    // records summed at a time (n_chunk <= 64)
+    const unsigned inv_chunk = 65536u / (unsigned)n_chunk + 1u;   // i / n_chunk = i inv >> 16 for i < kMegaItems
+
+    enum { kIdle, kExt, kShadow };
+    int mode = kIdle, b = 0;
+    int64_t g = 0;                // the lane's path
+    bool dry = false;             // no path left for this lane
+    bool prev_specular = true, t_set = false;   // t_set: the lane's row holds the throughput (1 until a weight)
+    V3 rd = v3(0.f, 0.f, 0.f);    // direction of the query under way
+    V3 ro = rd;
+    LaneTrav t;
+    t.tmin = t.tw = 0.f;
+    t.node = t.sp = 0;
+    t.best = t.ep = t.eo = -1;
+    t.occ = t.fin = false;
+    Crossings cr;
+    cr.n = 0;
+    int stack[kStackSize];
+    unsigned n_ext = 0, n_sh = 0, n_glass = 0;
+    TravCount tc;
+
+    for (;;) {
+        const unsigned m_wait = __ballot_sync(full, t.fin || (mode == kIdle && !dry));
+        const unsigned m_busy = __ballot_sync(full, mode != kIdle && !t.fin);
+        if (m_busy == 0 || __popc(m_wait) >= kMegaBatch) {
+            if (m_wait == 0) break;
+            int next_mode = kIdle;        // the lane's next query, where it has one
+            V3 no = ro, nd = rd;
+            float n_tmax = 3.402823466e38f;   // below +inf: a missed triangle's distance is no hit
+            int n_ep = -1, n_eo = -1;
+            bool ended = false;
+            int flags = 0;
+            float u_glass = 0.0f;
+            V3 thru = ro;
+            MegaRec &me = w.rec[lane];
+            if (t.fin && mode == kShadow) {
+                flags = me.flags;         // the diffuse weight, where the path goes on
+                if (!t.occ) {
+                    flags |= kMrResolve;
+                    me.ncr = cr.n;
+#pragma unroll 1
+                    for (int k = 0; k < cr.n; ++k) {
+                        const float4 cn = __ldg(sc.tri_n + cr.tri[k]);
+                        me.ccos[k] = -dot(rd, xyz(cn));
+                        me.cmat[k] = __float_as_int(cn.w);
+                    }
+                    n_glass += cr.n;
+                }
+                if (flags & kMrDiffuse) {
+                    next_mode = kExt;
+                    no = v3(w.on[0][lane], w.on[1][lane], w.on[2][lane]);
+                    nd = v3(w.dn[0][lane], w.dn[1][lane], w.dn[2][lane]);
+                    n_ep = w.xprim[lane];
+                    n_eo = -1;
+                } else {
+                    ended = true;
+                }
+            } else if (t.fin) {
+                const int prim = t.best;
+                if (b == 1 && a.first_prim) a.first_prim[g] = prim;
+                if (prim < 0) {
+                    ended = true;
+                } else {
+                    const int64_t gp = a.path_begin + g;
+                    const int r = find_render(a.rb, gp);
+                    const RenderInfo &ri = a.rb.info[r];
+                    const int64_t local = gp - ri.path_begin;
+                    uint32_t p, j;
+                    pixel_sample(local, ri.spp, p, j);
+                    const uint32_t k0 = ri.seed, k1 = ri.render_id;
+                    const float4 tn = __ldg(sc.tri_n + prim);
+                    const V3 ng = xyz(tn);
+                    const int mat = __float_as_int(tn.w);
+                    const int kind = __ldg(sc.mat_kind + mat);
+                    const V3 xh = ro + t.tw * rd;
+                    const float cd = dot(rd, ng);
+                    const V3 ns = cd < 0.0f ? ng : (-1.0f) * ng;
+                    const bool last = b == ri.max_depth;
+                    me.r = r;
+                    if ((kind == kEmitter || kind == kDiffuseEmitter) && cd < 0.0f &&
+                        (!ri.nee || b == 1 || prev_specular)) {
+                        flags |= kMrEmit;
+                        me.r_emit = mat;
+                    }
+                    if (kind == kLambert || kind == kDiffuseEmitter) {
+                        me.r_rho = kind == kLambert ? mat : M + mat;
+                        if (!last) {
+                            uint4 xb = philox4x32_10(make_uint4(p, j, (uint32_t)b, kSlotBsdf), k0, k1);
+                            nd = cosine_dir(ns, u01(xb.x), u01(xb.y));
+                            no = xh + kRayOffset * ns;
+                            n_ep = prim;
+                            next_mode = kExt;
+                        }
+                        bool shadow = false;
+                        if (ri.nee && sc.n_light > 0) {
+                            uint4 xl = philox4x32_10(make_uint4(p, j, (uint32_t)b, kSlotLight), k0, k1);
+                            float ua = u01(xl.x), su = sqrtf(u01(xl.y)), u2 = u01(xl.z);
+                            int li = sc.n_light - 1;
+#pragma unroll 1
+                            for (int q = 0; q < sc.n_light; ++q)
+                                if (ua < __ldg(sc.light_cdf + q)) { li = q; break; }
+                            const float4 lv0 = __ldg(sc.light_v + 3 * li), lv1 = __ldg(sc.light_v + 3 * li + 1),
+                                         lv2 = __ldg(sc.light_v + 3 * li + 2);
+                            const float b0 = 1.0f - su, b1 = u2 * su, b2 = 1.0f - b0 - b1;
+                            const V3 y = b0 * xyz(lv0) + b1 * xyz(lv1) + b2 * xyz(lv2);
+                            const V3 xo = xh + kRayOffset * ns;
+                            V3 wl = y - xo;
+                            const float dist = sqrtf(dot(wl, wl));
+                            wl = (1.0f / dist) * wl;
+                            const int lt = __float_as_int(lv0.w);
+                            const float4 ln = __ldg(sc.tri_n + lt);
+                            const float cx = dot(ns, wl), cy = -dot(xyz(ln), wl);
+                            if (cx > 0.0f && cy > 0.0f) {
+                                ++n_sh;
+                                shadow = true;
+                                me.G = cx * cy / (dist * dist) * sc.light_area * (1.0f / 3.14159265358979f);
+                                me.r_le = __float_as_int(ln.w);
+                                w.on[0][lane] = no.x;
+                                w.on[1][lane] = no.y;
+                                w.on[2][lane] = no.z;
+                                w.dn[0][lane] = nd.x;
+                                w.dn[1][lane] = nd.y;
+                                w.dn[2][lane] = nd.z;
+                                w.xprim[lane] = prim;
+                                no = xo;
+                                nd = wl;
+                                n_tmax = (1.0f - kShadowShorten) * dist;
+                                n_ep = prim;
+                            }
+                        }
+                        prev_specular = false;
+                        if (shadow) {
+                            me.flags = last ? 0 : kMrDiffuse;   // taken up when the shadow ray is answered
+                            next_mode = kShadow;
+                        } else if (last) {
+                            ended = true;
+                        } else {
+                            flags |= kMrDiffuse;
+                        }
+                    } else if (kind == kEmitter || last) {
+                        ended = true;
+                    } else {
+                        const float c = fabsf(cd);
+                        me.pcos = c;
+                        me.r_w = mat;
+                        me.r_w2 = M + mat;
+                        nd = rd - (2.0f * cd) * ng;
+                        no = xh + kRayOffset * ns;
+                        n_ep = prim;
+                        if (kind == kConductor) {
+                            flags |= kMrConductor;
+                        } else {
+                            flags |= kMrGlass;
+                            ++n_glass;
+                            n_eo = __ldg(sc.tri_obj + prim);   // for the branch that transmits
+                            const uint4 xg = philox4x32_10(make_uint4(p, j, (uint32_t)b, kSlotGlass), k0, k1);
+                            u_glass = u01(xg.x);
+                            thru = xh - kRayOffset * ns;
+                        }
+                        next_mode = kExt;
+                        prev_specular = true;
+                    }
+                }
+            }
+            if (__any_sync(full, flags & kMrGlass)) {
+                const float pr = warp_branch_proxy((flags & kMrGlass) != 0, me.pcos, L,
+                                                   sc.mat_a + (size_t)((flags & kMrGlass) ? me.r_w : 0) * L,
+                                                   reinterpret_cast<float *>(w.part));
+                if (flags & kMrGlass) {
+                    if (u_glass < pr) {
+                        me.pw = -1.0f / pr;
+                        n_eo = -1;
+                    } else {
+                        me.pw = 1.0f / (1.0f - pr);
+                        nd = rd;
+                        no = thru;
+                    }
+                }
+            }
+            // the warp works through the records' bins
+            if (flags && !t_set) flags |= kMrFirst;
+            const int held = me.flags;     // a shadow ray now under way keeps its flags
+            const unsigned work = __ballot_sync(full, flags != 0);
+            const int n_rec = __popc(work), mine = __popc(work & lt_mask);
+            if (flags) {
+                me.flags = flags;
+                w.order[mine] = lane;
+            }
+            __syncwarp();
+#pragma unroll 1
+            for (int r0 = 0; r0 < n_rec; r0 += per_pass) {
+                const int nr = min(per_pass, n_rec - r0), n_item = nr * n_chunk;
+#pragma unroll 1
+                for (int i = lane; i < n_item; i += 32) {
+                    const int jr = (int)((unsigned)i * inv_chunk >> 16), from = w.order[r0 + jr];
+                    const float3 s = mega_chunk<FILMS>(a, w.rec[from], rows + from * n_chunk, i - jr * n_chunk);
+                    w.part[i] = make_float4(s.x, s.y, s.z, 0.0f);
+                }
+                __syncwarp();
+                const int jr = mine - r0;
+                if ((flags & (kMrEmit | kMrResolve)) && jr >= 0 && jr < nr) {
+                    Kahan3 sum, acc;
+                    const float4 *pp = w.part + jr * n_chunk;
+#pragma unroll 1
+                    for (int c = 0; c < n_chunk; ++c) {
+                        const float4 v = pp[c];
+                        sum.add(v.x, v.y, v.z);
+                    }
+                    acc.x.s = w.acc[0][lane];
+                    acc.y.s = w.acc[1][lane];
+                    acc.z.s = w.acc[2][lane];
+                    acc.x.c = w.acc[3][lane] + sum.x.c;   // what the chunk sums lost goes on to the path's sum
+                    acc.y.c = w.acc[4][lane] + sum.y.c;
+                    acc.z.c = w.acc[5][lane] + sum.z.c;
+                    acc.add(sum.x.s, sum.y.s, sum.z.s);
+                    w.acc[0][lane] = acc.x.s;
+                    w.acc[1][lane] = acc.y.s;
+                    w.acc[2][lane] = acc.z.s;
+                    w.acc[3][lane] = acc.x.c;
+                    w.acc[4][lane] = acc.y.c;
+                    w.acc[5][lane] = acc.z.c;
+                }
+                __syncwarp();
+            }
+            if (flags & (kMrDiffuse | kMrConductor | kMrGlass)) t_set = true;
+            if (next_mode == kShadow) me.flags = held;
+            if (ended) {
+                a.sample_xyz[3 * g + 0] = w.acc[0][lane];
+                a.sample_xyz[3 * g + 1] = w.acc[1][lane];
+                a.sample_xyz[3 * g + 2] = w.acc[2][lane];
+                mode = kIdle;
+                t.fin = false;
+            }
+            // lanes without a path take the next ones
+            const bool need = mode == kIdle && !dry;
+            const unsigned m = __ballot_sync(full, need);
+            if (m) {
+                unsigned long long c0 = 0;
+                if (lane == 0) c0 = atomicAdd(a.cursor, (unsigned long long)__popc(m));
+                c0 = __shfl_sync(full, c0, 0);
+                if (need) {
+                    g = (int64_t)(c0 + (unsigned long long)__popc(m & lt_mask));
+                    dry = g >= a.path_count;
+                    if (!dry) {
+                        const int64_t gp = a.path_begin + g;
+                        const RenderInfo &ri = a.rb.info[find_render(a.rb, gp)];
+                        const int64_t local = gp - ri.path_begin;
+                        uint32_t p, j;
+                        pixel_sample(local, ri.spp, p, j);
+                        const int px = (int)(p % (uint32_t)ri.width), py = (int)(p / (uint32_t)ri.width);
+                        uint4 x = philox4x32_10(make_uint4(p, j, 0u, kSlotCamera), ri.seed, ri.render_id);
+                        camera_ray(ri, (float)px + u01(x.x), (float)py + u01(x.y), no, nd);
+                        next_mode = kExt;
+                        n_ep = n_eo = -1;
+                        n_tmax = 3.402823466e38f;
+                        b = 0;
+                        prev_specular = true;
+                        t_set = false;
+                        mode = kExt;
+#pragma unroll
+                        for (int k = 0; k < 6; ++k) w.acc[k][lane] = 0.0f;
+                    }
+                }
+            }
+            if (next_mode != kIdle) {
+                if (next_mode == kExt) {
+                    ++b;
+                    ++n_ext;
+                }
+                mode = next_mode;
+                ro = no;
+                rd = nd;
+                t.ray = make_ray(ro, rd);
+                t.tmin = 0.0f;
+                t.tw = n_tmax;
+                t.node = t.sp = 0;
+                t.best = -1;
+                t.ep = n_ep;
+                t.eo = n_eo;
+                t.occ = t.fin = false;
+                cr.n = 0;
+            }
+        }
+        trav_round<COUNT, false, 64, 6>(sc.g_nodes, sc.g_tris, sc.tri_obj, t, cr, stack, mode != kIdle && !t.fin,
+                                        mode == kShadow, [&]() { return rd; }, tc, a.error_flag, 0, 0);
+    }
+    if (!a.counters) return;
+    unsigned long long v[6] = {n_ext, n_sh, n_glass, tc.nodes, tc.tris, (unsigned long long)n_ext + n_sh};
+    const int nv = COUNT ? 6 : 3;
+    for (int k = 0; k < nv; ++k)
+        for (int off = 16; off > 0; off >>= 1) v[k] += __shfl_down_sync(full, v[k], off);
+    if (lane != 0) return;
     atomicAdd(a.counters + 0, v[0]);
     atomicAdd(a.counters + 1, v[1]);
     atomicAdd(a.counters + 2, v[2]);
@@ -234,28 +666,45 @@ __global__ void __launch_bounds__(128) k_megakernel(MegaArgs a) {
     }
 }
 
-template <bool COUNT, bool FILMS, bool PM = false>
-static void launch_mk(const MegaArgs &a, unsigned nb, int threads, cudaStream_t stream) {
+template <bool FILMS>
+static void launch_pm(const MegaArgs &a, cudaStream_t stream) {
+    const unsigned nb = (unsigned)((a.path_count + 127) / 128);
     switch (a.sc.L) {
-        case 8: k_megakernel<8, COUNT, FILMS, PM><<<nb, threads, 0, stream>>>(a); break;
-        case 16: k_megakernel<16, COUNT, FILMS, PM><<<nb, threads, 0, stream>>>(a); break;
-        default: k_megakernel<0, COUNT, FILMS, PM><<<nb, threads, 0, stream>>>(a); break;
+        case 8: k_megakernel_pm<8, FILMS><<<nb, 128, 0, stream>>>(a); break;
+        case 16: k_megakernel_pm<16, FILMS><<<nb, 128, 0, stream>>>(a); break;
+        default: k_megakernel_pm<0, FILMS><<<nb, 128, 0, stream>>>(a); break;
     }
+}
+
+template <bool COUNT, bool FILMS>
+static cudaError_t launch_plain(const MegaArgs &a, cudaStream_t stream) {
+    const size_t smem = mega_warp_bytes(a.sc.Lp) * kMegaWarps;
+    cudaError_t e = cudaSuccess;
+    if (smem > 48 * 1024)   // more than a block has without asking: over 104 bins
+        e = cudaFuncSetAttribute(k_megakernel<COUNT, FILMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) e = cudaMemsetAsync(a.cursor, 0, sizeof(unsigned long long), stream);
+    if (e != cudaSuccess) return e;
+    // one wave of resident blocks, fewer when there are not the paths for them
+    const int64_t want = (a.path_count + 32 * kMegaWarps - 1) / (32 * kMegaWarps);
+    int per_sm = 1;
+    if (want > a.sm_count) {
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_megakernel<COUNT, FILMS>, 32 * kMegaWarps, smem);
+        if (e != cudaSuccess) return e;
+    }
+    const int64_t most = (int64_t)a.sm_count * (per_sm > 0 ? per_sm : 1);
+    k_megakernel<COUNT, FILMS><<<(unsigned)(want < most ? want : most), 32 * kMegaWarps, smem, stream>>>(a);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_megakernel(const MegaArgs &a, cudaStream_t stream) {
     if (a.path_count <= 0) return cudaSuccess;
-    const int threads = 128;
-    const int64_t blocks = (a.path_count + threads - 1) / threads;
-    const unsigned nb = (unsigned)blocks;
     const bool films = a.sc.mat_nfilm != nullptr;
-    if (a.pm.on)
-        films ? launch_mk<false, true, true>(a, nb, threads, stream) : launch_mk<false, false, true>(a, nb, threads, stream);
-    else if (a.count_traversal)
-        films ? launch_mk<true, true>(a, nb, threads, stream) : launch_mk<true, false>(a, nb, threads, stream);
-    else
-        films ? launch_mk<false, true>(a, nb, threads, stream) : launch_mk<false, false>(a, nb, threads, stream);
-    return cudaGetLastError();
+    if (a.pm.on) {
+        films ? launch_pm<true>(a, stream) : launch_pm<false>(a, stream);
+        return cudaGetLastError();
+    }
+    if (a.count_traversal) return films ? launch_plain<true, true>(a, stream) : launch_plain<true, false>(a, stream);
+    return films ? launch_plain<false, true>(a, stream) : launch_plain<false, false>(a, stream);
 }
 
 }  // namespace sddm

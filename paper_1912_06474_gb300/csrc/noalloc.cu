@@ -39,7 +39,7 @@ namespace {
 
 constexpr size_t kNoAllocBytes = 16u << 20;
 constexpr size_t kNoAllocHeader = 8192;
-constexpr size_t kOffCounters = 0, kOffErr = 64, kOffInfo = 128, kOffOut = 384, kOffAovX = 392, kOffAovP = 400,
+constexpr size_t kOffCounters = 0, kOffErr = 64, kOffCursor = 80, kOffInfo = 128, kOffOut = 384, kOffAovX = 392, kOffAovP = 400,
                  kOffState = 512;
 constexpr int kNoAllocMaxMat = (int)((kNoAllocHeader - kOffState) / sizeof(float));
 constexpr int64_t kNoAllocMaxPaths = (int64_t)((kNoAllocBytes - kNoAllocHeader) / (3 * sizeof(float)));
@@ -145,6 +145,8 @@ extern "C" int sddm_render_noalloc(sddm_ctx *ctx, const sddm_render_desc *d, sdd
     a.first_prim = nullptr;
     a.counters = reinterpret_cast<unsigned long long *>(scratch + kOffCounters);
     a.error_flag = reinterpret_cast<int *>(scratch + kOffErr);
+    a.cursor = reinterpret_cast<unsigned long long *>(scratch + kOffCursor);
+    a.sm_count = v.sm_count;
     a.count_traversal = 0;
     if ((e = launch_megakernel(a, s)) != cudaSuccess) return cuda_fail(e, "sddm_render_noalloc: megakernel");
     ReduceArgs ra;

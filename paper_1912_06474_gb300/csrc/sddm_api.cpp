@@ -766,6 +766,7 @@ int ctx_view(sddm_ctx *ctx, CtxView *v) {
     v->n_mat = (int)ctx->mats.size();
     v->ev0 = ctx->ev0;
     v->ev1 = ctx->ev1;
+    v->sm_count = ctx->sm_count;
     return SDDM_OK;
 }
 int check_render_desc(const sddm_ctx *ctx, const sddm_render_desc *d, int n) { return validate_desc(ctx, d, n); }
@@ -903,6 +904,8 @@ int sddm_render(sddm_ctx *ctx, const sddm_render_desc *d, int n, sddm_stats *st)
                 a.first_prim = any_aov ? ctx->d_first.as<int32_t>() : nullptr;
                 a.counters = ctx->d_counters.as<unsigned long long>();
                 a.error_flag = ctx->d_err.as<int>();
+                a.cursor = a.counters + kNumCounters - 1;
+                a.sm_count = ctx->sm_count;
                 a.count_traversal = count_trav;
                 a.pm = ctx->pm_view;
                 a.pmc = ctx->pmc_view;

@@ -14,7 +14,7 @@ namespace sddm {
 // Statistics counters of a render call, u64 each (layout at DevScene users'
 // `counters` fields): ext, shadow, glass, crossings, fallbacks, nodes, tris,
 // visits, surrogate batches, surrogate rows, crossings carried on by the
-// tracing thread; the rest spare.
+// tracing thread; the last one the megakernel's path cursor; the rest spare.
 constexpr int kNumCounters = 16;
 
 constexpr int kMaxL = 256;
@@ -137,6 +137,7 @@ struct CtxView {
     DevScene dev;
     int n_mat;
     cudaEvent_t ev0, ev1;
+    int sm_count;
 };
 int ctx_view(sddm_ctx *ctx, CtxView *v);
 int check_render_desc(const sddm_ctx *ctx, const sddm_render_desc *d, int n);
@@ -170,6 +171,8 @@ struct MegaArgs {
     unsigned long long *counters;      // [16]: ext, shadow, glass, crossings, fallbacks, nodes, tris, visits,
                                        // surrogate batches, spare
     int *error_flag;
+    unsigned long long *cursor;        // next path to hand to a lane (set to 0 by the launch)
+    int sm_count;
     int count_traversal;
     PhotonGridView pm = {};            // photon map gathered at the first diffuse vertex (pm.on)
     PhotonGridView pmc = {};           // caustic map gathered there too (pmc.on)
