@@ -654,6 +654,14 @@ __device__ __forceinline__ void spec_items(const KArgs &a, const SpecRec *rec, f
         part[i] = make_float4(s.x, s.y, s.z, 0.0f);
     }
 }
+// k + (s2 - c2), the rounding error of the addition kept in k.c (true sum k.s - k.c).
+__device__ __forceinline__ void two_sum(Kahan &k, float s2, float c2) {
+    const float t = k.s + s2, b = t - k.s;
+    const float e = (k.s - (t - b)) + (s2 - b);
+    k.c = (k.c + c2) - e;
+    k.s = t;
+}
+
 template <bool FILMS>
 static __device__ __noinline__ void spec_items_direct(const KArgs &a, const SpecRec *rec, float4 *part, int n_item,
                                                       int n_chunk, unsigned inv_chunk) {
@@ -1070,6 +1078,8 @@ static int trace_chunk(const DDMRun &run, const PhotonGridView &pmv, const Photo
         return SDDM_ERR_OOM;
     }
     const size_t oLp = take(4 * (size_t)n_batch), oLf = take(4 * (size_t)n_batch), oLc = take(16);
+    // photon map: the paths that gather at a bounce
+    const size_t oGl = take(pmv.on ? 4 * np : 4), oGh = take(pmv.on ? 4 * np : 4), oGc = take(16);
     if (off > buf.bytes) {
         if (buf.mem) cudaFree(buf.mem);
         buf.mem = nullptr;
@@ -1125,6 +1135,7 @@ static int trace_chunk(const DDMRun &run, const PhotonGridView &pmv, const Photo
     a.glass_res = (const float *)(m + oRes);
     a.block_cnt = (int *)(m + oBc);
     a.list_cnt = (uint32_t *)(m + oLc);
+    const GatherLists gl{(int *)(m + oGl), (int *)(m + oGh), (unsigned *)(m + oGc)};
     a.pm = pmv;
     a.cell_perm = nullptr;
     a.q_begin = 0;
@@ -1264,10 +1275,8 @@ static int trace_chunk(const DDMRun &run, const PhotonGridView &pmv, const Photo
             k_shade_spectral<false><<<spec_blocks, kSpecThreads, 0, s>>>(a);
         DDM_CHECK(cudaGetLastError());
         if (a.pm.on) {
-            // one path slot per thread: the gather is latency-bound and gains from the most blocks in flight
-            k_ddm_gather<<<(unsigned)((np + 255) / 256), 256, 0, s>>>(a);
-            DDM_CHECK(cudaGetLastError());
-            *run.launches += 1;
+            DDM_CHECK(launch_gather(a, gl, sm, s));
+            *run.launches += 2;
         }
         k_shade_continue<<<cont_blocks, 256, bins_smem, s>>>(a);
         DDM_CHECK(cudaGetLastError());
