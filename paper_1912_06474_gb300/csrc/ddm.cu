@@ -327,6 +327,10 @@ __global__ void __launch_bounds__(256, SDDM_SCATTER_MINB) k_scatter(KArgs a) {
     const bool bad = (unsigned long long)total != Q.ctl[0] || (int64_t)total > Q.cap;
     if (bad) total = 0;
     if (blockIdx.x == 0) {
+        if (Q.ctl_next) {
+            for (int i = threadIdx.x; i < n_cells; i += blockDim.x) Q.cnt_next[i] = 0;
+            if (threadIdx.x < 4) Q.ctl_next[threadIdx.x] = 0;
+        }
         for (int i = threadIdx.x; i < n_cells; i += blockDim.x) Q.off[i] = bad ? 0 : s_off[i];
         if (threadIdx.x == 0) {
             Q.off[n_cells] = total;
@@ -1059,7 +1063,7 @@ static int trace_chunk(const DDMRun &run, const PhotonGridView &pmv, const Photo
                  oFl = take(4 * np), oPm = take(4 * np), oPc = take(4 * np), oPw = take(4 * np), oG = take(4 * np),
                  oLm = take(4 * np), oSh = take(4 * np), oCo = take(4 * kMaxCross * np), oCm = take(4 * kMaxCross * np),
                  oCc = take(4 * kMaxCross * np), oH0 = take(16 * np), oH1 = take(16 * np), oIn = take(48 * cap),
-                 oSt = take(48 * cap), oCtl = take(32 + 4 * (size_t)nb), oFill = take(4 * (size_t)nb),
+                 oSt = take(48 * cap), oCtl = take(queue_counter_bytes(nb)),
                  oOff = take(4 * ((size_t)nb + 1));
     // glass evaluations of each bounce go through a query list, evaluated by the
     // exact slab or the learned model in a dense pass before shading
@@ -1122,9 +1126,7 @@ static int trace_chunk(const DDMRun &run, const PhotonGridView &pmv, const Photo
     Q.cap = cap;
     Q.in = (float4 *)(m + oIn);
     Q.stage = (float4 *)(m + oSt);
-    Q.ctl = (unsigned long long *)(m + oCtl);
-    Q.cnt = (int *)(m + oCtl + 32);
-    Q.fill = (int *)(m + oFill);
+    queue_counters(Q, m + oCtl, nb);
     Q.off = (int *)(m + oOff);
     a.use_queries = use_queries;
     a.queries = (float4 *)(m + oQ);
@@ -1177,7 +1179,11 @@ static int trace_chunk(const DDMRun &run, const PhotonGridView &pmv, const Photo
     do {                                                                 \
         if ((e = (x)) != cudaSuccess) return cuda_fail(e, "sddm_render: " #x); \
     } while (0)
-    DDM_CHECK(cudaMemsetAsync(Q.ctl, 0, ctl_bytes, s));
+    DDM_CHECK(cudaMemsetAsync(Q.ctl, 0, queue_counter_bytes(nb), s));
+    if (run.cache) {   // the cache's waves are sorted and traced in groups: one set, emptied between them
+        Q.ctl_next = nullptr;
+        Q.cnt_next = nullptr;
+    }
     a.b = 0;
     a.last_wave = 0;
     const size_t bins_smem = sizeof(int) * (size_t)nb;
@@ -1206,16 +1212,16 @@ static int trace_chunk(const DDMRun &run, const PhotonGridView &pmv, const Photo
         for (int w = 0; w < waves; ++w) {
             a.last_wave = w == waves - 1;
             a.g.continue_cells = ddm_wave_continues(run.g, w, waves);
-            DDM_CHECK(cudaMemsetAsync(Q.fill, 0, 4 * (size_t)nb, s));
             if (!cache) {
                 k_scatter<<<scatter_blocks, 256, 0, s>>>(a);
                 DDM_CHECK(cudaGetLastError());
-                DDM_CHECK(cudaMemsetAsync(Q.ctl, 0, ctl_bytes, s));
+                Q.flip();
                 const int rc = trace_launch();
                 if (rc != SDDM_OK) return rc;
                 *run.launches += 1;
                 continue;
             }
+            DDM_CHECK(cudaMemsetAsync(Q.fill, 0, 4 * (size_t)nb, s));
             // subdomain cache (Sec. 5's loading and unloading of subdomains):
             // the rays waiting per cell decide which cells are loaded, in
             // which groups the wave is traced, and the order of its queue

@@ -417,8 +417,8 @@ int ddm_photon_pass(const DDMPhotonRun &run, DDMBuffers &buf, cudaStream_t s) {
         return o;
     };
     const size_t oT = take(sizeof(float) * (size_t)L * np), oFl = take(4 * np), oH0 = take(16 * np),
-                 oH1 = take(16 * np), oIn = take(48 * cap), oSt = take(48 * cap), oCtl = take(32 + 4 * (size_t)nb),
-                 oFill = take(4 * (size_t)nb), oOff = take(4 * ((size_t)nb + 1));
+                 oH1 = take(16 * np), oIn = take(48 * cap), oSt = take(48 * cap), oCtl = take(queue_counter_bytes(nb)),
+                 oOff = take(4 * ((size_t)nb + 1));
     if (off > buf.bytes) {
         if (buf.mem) cudaFree(buf.mem);
         buf.mem = nullptr;
@@ -446,9 +446,7 @@ int ddm_photon_pass(const DDMPhotonRun &run, DDMBuffers &buf, cudaStream_t s) {
     Q.cap = cap;
     Q.in = (float4 *)(m + oIn);
     Q.stage = (float4 *)(m + oSt);
-    Q.ctl = (unsigned long long *)(m + oCtl);
-    Q.cnt = (int *)(m + oCtl + 32);
-    Q.fill = (int *)(m + oFill);
+    queue_counters(Q, m + oCtl, nb);
     Q.off = (int *)(m + oOff);
     PhotonPass pp;
     pp.begin = run.begin;
@@ -467,23 +465,21 @@ int ddm_photon_pass(const DDMPhotonRun &run, DDMBuffers &buf, cudaStream_t s) {
     const int trace_blocks = sm * (run.blocks_per_sm > 0 ? run.blocks_per_sm : SDDM_TRACE_MIN_BLOCKS);
     const int scatter_blocks = sm * 4;
     const int waves = ddm_waves(run.g);
-    const size_t ctl_bytes = 32 + 4 * (size_t)nb;
     const size_t bins_smem = sizeof(int) * (size_t)nb;
     cudaError_t e;
 #define PM_CHECK(x)                                                                \
     do {                                                                           \
         if ((e = (x)) != cudaSuccess) return cuda_fail(e, "sddm_render_photon_map: " #x); \
     } while (0)
-    PM_CHECK(cudaMemsetAsync(Q.ctl, 0, ctl_bytes, s));
+    PM_CHECK(cudaMemsetAsync(Q.ctl, 0, queue_counter_bytes(nb), s));
     k_photon_emit<<<path_blocks, 256, bins_smem, s>>>(a, pp);
     PM_CHECK(cudaGetLastError());
     *run.launches += 1;
     for (int b = 1; b <= run.max_depth - 1; ++b) {
         for (int w = 0; w < waves; ++w) {
-            PM_CHECK(cudaMemsetAsync(Q.fill, 0, 4 * (size_t)nb, s));
             k_scatter<<<scatter_blocks, 256, 0, s>>>(a);
             PM_CHECK(cudaGetLastError());
-            PM_CHECK(cudaMemsetAsync(Q.ctl, 0, ctl_bytes, s));
+            Q.flip();
             a.last_wave = w == waves - 1;
             a.g.continue_cells = ddm_wave_continues(run.g, w, waves);
             k_trace_wave<false><<<trace_blocks, 128, 0, s>>>(a);

@@ -140,6 +140,8 @@ __global__ void __launch_bounds__(128, SDDM_TRACE_MIN_BLOCKS) k_trace_wave(KArgs
     // (the groups of cells resident together in the subdomain cache)
     const int q0 = a.q_end > 0 ? (int)a.q_begin : 0;
     const int total = (a.q_end > 0 ? (int)a.q_end : Q.off[g.n_bins]) - q0;
+    if (Q.ctl_next && blockIdx.x == 0)   // the cursors of the next wave's sort
+        for (int i = threadIdx.x; i < g.n_bins; i += blockDim.x) Q.fill[i] = 0;
     if (total <= 0) return;
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;

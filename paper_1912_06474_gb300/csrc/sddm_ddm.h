@@ -80,7 +80,33 @@ struct Queues {
     int *fill;            // [n_bins] scatter cursors
     int *off;             // [n_bins + 1] offsets of the sorted `in`
     unsigned long long *ctl;   // [4]: stage count, claim cursor, -, -
+    // The counts a wave's sort reads (cnt, ctl) and those its trace writes are two
+    // sets that take turns: the sort empties the set of the trace after it, the
+    // trace the sort's cursors, so that no memset stands between the kernels.
+    // NULL: the caller empties the one set itself.
+    int *cnt_next;
+    unsigned long long *ctl_next;
+    void flip() {
+        int *c = cnt;
+        cnt = cnt_next;
+        cnt_next = c;
+        unsigned long long *t = ctl;
+        ctl = ctl_next;
+        ctl_next = t;
+    }
 };
+
+// Memory of a Queues' counters (two sets and the sort's cursors, 16-byte aligned,
+// all of it zero at the start) and the pointers into it.
+inline size_t queue_counter_bytes(int n_bins) { return 2 * (32 + 4 * (size_t)((n_bins + 7) & ~7)) + 4 * (size_t)n_bins; }
+inline void queue_counters(Queues &q, char *m, int n_bins) {
+    const size_t set = 32 + 4 * (size_t)((n_bins + 7) & ~7);
+    q.ctl = (unsigned long long *)m;
+    q.cnt = (int *)(m + 32);
+    q.ctl_next = (unsigned long long *)(m + set);
+    q.cnt_next = (int *)(m + set + 32);
+    q.fill = (int *)(m + 2 * set);
+}
 
 struct DDMBuffers {
     void *mem = nullptr;
