@@ -107,8 +107,52 @@ struct DevBuf {
     T *as() const { return reinterpret_cast<T *>(p); }
 };
 
+// Page-locked host memory: copies to and from it are queued without the driver's
+// own staging.
+struct PinnedBuf {
+    void *p = nullptr;
+    size_t bytes = 0;
+    PinnedBuf() = default;
+    PinnedBuf(const PinnedBuf &) = delete;
+    PinnedBuf &operator=(const PinnedBuf &) = delete;
+    ~PinnedBuf() {
+        if (p) cudaFreeHost(p);
+    }
+    cudaError_t ensure(size_t n) {
+        if (n <= bytes) return cudaSuccess;
+        if (p) cudaFreeHost(p);
+        p = nullptr;
+        bytes = 0;
+        const cudaError_t e = cudaHostAlloc(&p, n, cudaHostAllocDefault);
+        if (e != cudaSuccess) {
+            p = nullptr;
+            return e;
+        }
+        bytes = n;
+        return cudaSuccess;
+    }
+};
+
 // Device error word [4] and, behind it, the surrogate's batch counts [4].
 constexpr size_t kErrBytes = 32;
+
+// Layout of a render's table for n renders and M materials: statistics counters
+// and the error word (zero before the call, read back after it), then the render
+// records, coloration states and output pointers.
+struct RenderTable {
+    static constexpr size_t counters = 0, err = kNumCounters * sizeof(unsigned long long), results = err + 16;
+    static constexpr size_t info = 256;
+    size_t state, outs, aov_x, aov_p, bytes;
+    RenderTable(size_t n, size_t M) {
+        auto up = [](size_t x) { return (x + 15) & ~(size_t)15; };
+        state = up(info + n * sizeof(RenderInfo));
+        outs = up(state + n * M * sizeof(float));
+        aov_x = outs + n * sizeof(void *);
+        aov_p = aov_x + n * sizeof(void *);
+        bytes = aov_p + n * sizeof(void *);
+    }
+};
+static_assert(RenderTable::results <= RenderTable::info, "results fit before the render records");
 
 }  // namespace sddm
 
@@ -140,7 +184,11 @@ struct sddm_ctx {
     HostBuf h_cell_nodes, h_cell_tris;   // the same, in host memory (bvh_in_host_memory, cell_cache_bytes)
     CellCache cache;                     // device cache of subdomain BVHs (cell_cache_bytes > 0)
     // per-render scratch
-    DevBuf d_info, d_state, d_out_tab, d_aov_xyz_tab, d_aov_prim_tab, d_samples, d_first, d_counters, d_err;
+    DevBuf d_table;      // a render's counters, error word and tables (RenderTable), one copy each way
+    PinnedBuf h_table;   // its host side; stage_busy: a copy from it may still be under way
+    bool stage_busy = false;
+    DevBuf d_samples, d_first, d_err;
+    DevBuf d_host_out;   // device side of sddm_render_host's outputs
     DDMBuffers ddm_buf;
     // photon map (sddm_render_photon_map): slots, grid, and the view the
     // megakernel reads while pm_view.on
@@ -163,8 +211,7 @@ struct sddm_ctx {
     // CUDA graphs of the render launch sequence, keyed by everything that is
     // baked into kernel parameters (sizes, buffer addresses, build)
     int64_t build_id = 0;
-    cudaStream_t gstream = nullptr;
-    cudaEvent_t hand0 = nullptr, hand1 = nullptr;
+    cudaStream_t gstream = nullptr;   // captures only; a graph is launched on the context's stream
     struct Graph {
         cudaGraphExec_t exec;
         int64_t launches;   // kernels in the captured sequence
@@ -176,8 +223,6 @@ struct sddm_ctx {
     ~sddm_ctx() {
         for (auto &kv : graphs) cudaGraphExecDestroy(kv.second.exec);
         if (gstream) cudaStreamDestroy(gstream);
-        if (hand0) cudaEventDestroy(hand0);
-        if (hand1) cudaEventDestroy(hand1);
     }
 };
 
@@ -206,10 +251,9 @@ int sddm_create(sddm_ctx **out, int device, void *stream) {
     c->stream = reinterpret_cast<cudaStream_t>(stream);
     c->sm_count = prop.multiProcessorCount;
     if ((e = cudaEventCreate(&c->ev0)) != cudaSuccess || (e = cudaEventCreate(&c->ev1)) != cudaSuccess ||
-        (e = cudaEventCreateWithFlags(&c->hand0, cudaEventDisableTiming)) != cudaSuccess ||
-        (e = cudaEventCreateWithFlags(&c->hand1, cudaEventDisableTiming)) != cudaSuccess ||
-        (e = cudaStreamCreateWithFlags(&c->gstream, cudaStreamNonBlocking)) != cudaSuccess)
-        return cuda_fail(e, "sddm_create: events and graph stream");
+        (e = cudaStreamCreateWithFlags(&c->gstream, cudaStreamNonBlocking)) != cudaSuccess ||
+        (e = c->h_table.ensure(4096)) != cudaSuccess || (e = c->d_table.ensure(4096)) != cudaSuccess)
+        return cuda_fail(e, "sddm_create: events, graph stream and render table");
     *out = c.release();
     return SDDM_OK;
 }
@@ -815,10 +859,23 @@ int sddm_render(sddm_ctx *ctx, const sddm_render_desc *d, int n, sddm_stats *st)
     cudaError_t e = cudaSetDevice(ctx->device);
     if (e != cudaSuccess) return cuda_fail(e, "sddm_render: cudaSetDevice");
     const int M = (int)ctx->mats.size();
-    std::vector<RenderInfo> info(n);
-    std::vector<float> state((size_t)n * M);
-    std::vector<float *> outs(n), aov_x(n);
-    std::vector<int32_t *> aov_p(n);
+    cudaStream_t s = ctx->stream;
+    const RenderTable tab((size_t)n, (size_t)M);
+    if (ctx->stage_busy) {   // a call that failed left its copy unwaited for
+        if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(e, "sddm_render: synchronize");
+        ctx->stage_busy = false;
+    }
+    if ((e = ctx->h_table.ensure(std::max<size_t>(tab.bytes, 4096))) || (e = ctx->d_table.ensure(std::max<size_t>(tab.bytes, 4096))))
+        return e == cudaErrorMemoryAllocation ? fail(SDDM_ERR_OOM, "sddm_render: render table allocation failed")
+                                              : cuda_fail(e, "sddm_render: render table");
+    char *const host = static_cast<char *>(ctx->h_table.p), *const devt = ctx->d_table.as<char>();
+    std::memset(host, 0, RenderTable::info);
+    RenderInfo *const info = reinterpret_cast<RenderInfo *>(host + RenderTable::info);
+    float *const state = reinterpret_cast<float *>(host + tab.state);
+    float **const outs = reinterpret_cast<float **>(host + tab.outs), **const aov_x = reinterpret_cast<float **>(host + tab.aov_x);
+    int32_t **const aov_p = reinterpret_cast<int32_t **>(host + tab.aov_p);
+    unsigned long long *const d_counters = reinterpret_cast<unsigned long long *>(devt + RenderTable::counters);
+    int *const d_err = reinterpret_cast<int *>(devt + RenderTable::err);
     int64_t paths = 0, pixels = 0;
     bool any_aov = false;
     for (int r = 0; r < n; ++r) {
@@ -845,18 +902,13 @@ int sddm_render(sddm_ctx *ctx, const sddm_render_desc *d, int n, sddm_stats *st)
         paths += (int64_t)x.width * x.height * x.spp;
         pixels += (int64_t)x.width * x.height;
     }
-    cudaStream_t s = ctx->stream;
-    if ((e = ctx->d_info.upload(info, s)) || (e = ctx->d_state.upload(state, s)) || (e = ctx->d_out_tab.upload(outs, s)) ||
-        (e = ctx->d_aov_xyz_tab.upload(aov_x, s)) || (e = ctx->d_aov_prim_tab.upload(aov_p, s)) ||
-        (e = ctx->d_counters.ensure(kNumCounters * sizeof(unsigned long long))) || (e = ctx->d_err.ensure(kErrBytes)))
+    if ((e = cudaMemcpyAsync(devt, host, tab.bytes, cudaMemcpyHostToDevice, s)) != cudaSuccess)
         return cuda_fail(e, "sddm_render: upload of the render table");
-    if ((e = cudaMemsetAsync(ctx->d_counters.p, 0, kNumCounters * sizeof(unsigned long long), s)) ||
-        (e = cudaMemsetAsync(ctx->d_err.p, 0, 16, s)))
-        return cuda_fail(e, "sddm_render: memset");
+    ctx->stage_busy = true;
     RenderBatch rb;
-    rb.info = ctx->d_info.as<RenderInfo>();
+    rb.info = reinterpret_cast<const RenderInfo *>(devt + RenderTable::info);
     rb.n = n;
-    rb.state_s = ctx->d_state.as<float>();
+    rb.state_s = reinterpret_cast<const float *>(devt + tab.state);
 
     // chunks of whole pixels, at most `cap` paths each
     int64_t cap = ctx->opts.paths_in_flight > 0 ? ctx->opts.paths_in_flight : (int64_t)1 << 22;
@@ -902,8 +954,8 @@ int sddm_render(sddm_ctx *ctx, const sddm_render_desc *d, int n, sddm_stats *st)
                 a.path_count = np;
                 a.sample_xyz = ctx->d_samples.as<float>();
                 a.first_prim = any_aov ? ctx->d_first.as<int32_t>() : nullptr;
-                a.counters = ctx->d_counters.as<unsigned long long>();
-                a.error_flag = ctx->d_err.as<int>();
+                a.counters = d_counters;
+                a.error_flag = d_err;
                 a.cursor = a.counters + kNumCounters - 1;
                 a.sm_count = ctx->sm_count;
                 a.count_traversal = count_trav;
@@ -928,8 +980,8 @@ int sddm_render(sddm_ctx *ctx, const sddm_render_desc *d, int n, sddm_stats *st)
                 for (int q = 0; q < n; ++q) run.max_depth = std::max(run.max_depth, d[q].max_depth);
                 run.sample_xyz = ctx->d_samples.as<float>();
                 run.first_prim = any_aov ? ctx->d_first.as<int32_t>() : nullptr;
-                run.counters = ctx->d_counters.as<unsigned long long>();
-                run.error_flag = ctx->d_err.as<int>();
+                run.counters = d_counters;
+                run.error_flag = d_err;
                 run.sm_count = ctx->sm_count;
                 run.blocks_per_sm = ctx->opts.blocks_per_sm;
                 run.queue_capacity = ctx->opts.queue_capacity;
@@ -950,9 +1002,9 @@ int sddm_render(sddm_ctx *ctx, const sddm_render_desc *d, int n, sddm_stats *st)
             ra.rb = rb;
             ra.path_begin = path0;
             ra.sample_xyz = ctx->d_samples.as<float>();
-            ra.xyz_out = ctx->d_out_tab.as<float *>();
-            ra.aov_xyz = ctx->d_aov_xyz_tab.as<float *>();
-            ra.aov_prim = ctx->d_aov_prim_tab.as<int32_t *>();
+            ra.xyz_out = reinterpret_cast<float *const *>(devt + tab.outs);
+            ra.aov_xyz = reinterpret_cast<float *const *>(devt + tab.aov_x);
+            ra.aov_prim = reinterpret_cast<int32_t *const *>(devt + tab.aov_p);
             ra.first_prim = any_aov ? ctx->d_first.as<int32_t>() : nullptr;
             if ((e = launch_reduce_pixels(ra, pix0, pix1 - pix0, s)) != cudaSuccess)
                 return cuda_fail(e, "sddm_render: reduce launch");
@@ -971,10 +1023,11 @@ int sddm_render(sddm_ctx *ctx, const sddm_render_desc *d, int n, sddm_stats *st)
     std::string key;
     if (graphable) {
         char buf[256];
-        std::snprintf(buf, sizeof buf, "%lld|%d|%d|%d|%d|%lld|%d|%u|%d|%p|%p|%p|%p|%p|%p", (long long)ctx->build_id,
+        std::snprintf(buf, sizeof buf, "%lld|%d|%d|%d|%d|%lld|%d|%u|%d|%p|%p|%p|%p|%p", (long long)ctx->build_id,
                       n, d[0].method, d[0].bsdf_mode, (int)any_aov, (long long)ctx->opts.paths_in_flight,
-                      ctx->opts.blocks_per_sm, d[0].seed, time_trace, ctx->d_samples.p, ctx->d_first.p,
-                      ctx->ddm_buf.mem, ctx->d_info.p, (const void *)mlp_params, ctx->d_counters.p);
+                      ctx->opts.blocks_per_sm, mlp_params ? d[0].seed : 0u /* the probes' key */, time_trace,
+                      ctx->d_samples.p, ctx->d_first.p,
+                      ctx->ddm_buf.mem, ctx->d_table.p, (const void *)mlp_params);
         key = buf;
         for (int r = 0; r < n; ++r) {
             std::snprintf(buf, sizeof buf, "|%d,%d,%d,%d", d[r].width, d[r].height, d[r].spp, d[r].max_depth);
@@ -983,8 +1036,6 @@ int sddm_render(sddm_ctx *ctx, const sddm_render_desc *d, int n, sddm_stats *st)
     }
     auto it = graphable ? ctx->graphs.find(key) : ctx->graphs.end();
     if (graphable && (it != ctx->graphs.end() || ctx->seen[key] > 0)) {
-        if ((e = cudaEventRecord(ctx->hand0, s)) || (e = cudaStreamWaitEvent(ctx->gstream, ctx->hand0, 0)))
-            return cuda_fail(e, "sddm_render: stream hand-off");
         if (it == ctx->graphs.end()) {
             if (ctx->graphs.size() >= 8) {
                 for (auto &kv : ctx->graphs) cudaGraphExecDestroy(kv.second.exec);
@@ -1008,8 +1059,7 @@ int sddm_render(sddm_ctx *ctx, const sddm_render_desc *d, int n, sddm_stats *st)
         }
         launches = it->second.launches;
         ctx->ddm_buf.events_used = it->second.events_used;
-        if ((e = cudaGraphLaunch(it->second.exec, ctx->gstream)) || (e = cudaEventRecord(ctx->hand1, ctx->gstream)) ||
-            (e = cudaStreamWaitEvent(s, ctx->hand1, 0)))
+        if ((e = cudaGraphLaunch(it->second.exec, s)) != cudaSuccess)
             return cuda_fail(e, "sddm_render: graph launch");
     } else {
         int rc2 = launch_all(s);
@@ -1017,12 +1067,12 @@ int sddm_render(sddm_ctx *ctx, const sddm_render_desc *d, int n, sddm_stats *st)
         if (graphable) ctx->seen[key] = 1;
     }
     if ((e = cudaEventRecord(ctx->ev1, s)) != cudaSuccess) return cuda_fail(e, "sddm_render: event");
-    unsigned long long cnt[kNumCounters];
-    int err[4];
-    if ((e = cudaMemcpyAsync(cnt, ctx->d_counters.p, sizeof(cnt), cudaMemcpyDeviceToHost, s)) ||
-        (e = cudaMemcpyAsync(err, ctx->d_err.p, sizeof(err), cudaMemcpyDeviceToHost, s)) ||
+    if ((e = cudaMemcpyAsync(host, devt, RenderTable::results, cudaMemcpyDeviceToHost, s)) ||
         (e = cudaStreamSynchronize(s)))
         return cuda_fail(e, "sddm_render: kernel execution");
+    ctx->stage_busy = false;
+    const unsigned long long *cnt = reinterpret_cast<const unsigned long long *>(host + RenderTable::counters);
+    const int *err = reinterpret_cast<const int *>(host + RenderTable::err);
     if (err[0] != 0) {
         char msg[160];
         std::snprintf(msg, sizeof msg, "sddm_render: device reported error %d (detail %d, %d)", err[0], err[1], err[2]);
@@ -1298,43 +1348,36 @@ int sddm_render_progressive_photon_map(sddm_ctx *ctx, const sddm_render_desc *d,
     return SDDM_OK;
 }
 
+// Outputs of sddm_render_host up to this size keep their device memory for the next call.
+static constexpr size_t kHostOutKeep = (size_t)256 << 20;
+
 int sddm_render_host(sddm_ctx *ctx, const sddm_render_desc *d, int n, sddm_stats *st) {
     int rc = validate_desc(ctx, d, n);
     if (rc != SDDM_OK) return rc;
     cudaError_t e = cudaSetDevice(ctx->device);
     if (e != cudaSuccess) return cuda_fail(e, "sddm_render_host: cudaSetDevice");
     std::vector<sddm_render_desc> dd(d, d + n);
-    std::vector<void *> bufs;
-    auto cleanup = [&]() {
-        for (void *p : bufs) cudaFree(p);
+    // device side of every output in one buffer that the context keeps
+    size_t need = 0;
+    auto take = [&](size_t bytes) {
+        const size_t at = need;
+        need += (bytes + 255) & ~(size_t)255;
+        return at;
     };
+    std::vector<size_t> at(3 * (size_t)n, 0);
     for (int r = 0; r < n; ++r) {
-        size_t px = (size_t)d[r].width * d[r].height;
-        void *p = nullptr;
-        if ((e = cudaMalloc(&p, px * 3 * sizeof(float))) != cudaSuccess) {
-            cleanup();
-            return fail(SDDM_ERR_OOM, "sddm_render_host: device allocation failed");
-        }
-        bufs.push_back(p);
-        dd[r].xyz_out = (float *)p;
-        dd[r].aov_sample_xyz = nullptr;
-        dd[r].aov_first_prim = nullptr;
-        if (d[r].aov_sample_xyz) {
-            if ((e = cudaMalloc(&p, px * d[r].spp * 3 * sizeof(float))) != cudaSuccess) {
-                cleanup();
-                return fail(SDDM_ERR_OOM, "sddm_render_host: device allocation failed");
-            }
-            bufs.push_back(p);
-            dd[r].aov_sample_xyz = (float *)p;
-        }
-        if (d[r].aov_first_prim) {
-            if ((e = cudaMalloc(&p, px * d[r].spp * sizeof(int32_t))) != cudaSuccess) {
-                cleanup();
-                return fail(SDDM_ERR_OOM, "sddm_render_host: device allocation failed");
-            }
-            bufs.push_back(p);
-            dd[r].aov_first_prim = (int32_t *)p;
-        }
+        const size_t px = (size_t)d[r].width * d[r].height;
+        at[3 * r] = take(px * 3 * sizeof(float));
+        if (d[r].aov_sample_xyz) at[3 * r + 1] = take(px * d[r].spp * 3 * sizeof(float));
+        if (d[r].aov_first_prim) at[3 * r + 2] = take(px * d[r].spp * sizeof(int32_t));
+    }
+    if ((e = ctx->d_host_out.ensure(need)) != cudaSuccess)
+        return fail(SDDM_ERR_OOM, "sddm_render_host: device allocation failed");
+    for (int r = 0; r < n; ++r) {
+        char *const base = ctx->d_host_out.as<char>();
+        dd[r].xyz_out = reinterpret_cast<float *>(base + at[3 * r]);
+        dd[r].aov_sample_xyz = d[r].aov_sample_xyz ? reinterpret_cast<float *>(base + at[3 * r + 1]) : nullptr;
+        dd[r].aov_first_prim = d[r].aov_first_prim ? reinterpret_cast<int32_t *>(base + at[3 * r + 2]) : nullptr;
     }
     rc = sddm_render(ctx, dd.data(), n, st);
     for (int r = 0; r < n && rc == SDDM_OK; ++r) {
@@ -1351,7 +1394,7 @@ int sddm_render_host(sddm_ctx *ctx, const sddm_render_desc *d, int n, sddm_stats
     }
     if (rc == SDDM_OK && (e = cudaStreamSynchronize(ctx->stream)) != cudaSuccess)
         rc = cuda_fail(e, "sddm_render_host: synchronize");
-    cleanup();
+    if (ctx->d_host_out.bytes > kHostOutKeep) ctx->d_host_out.release();
     return rc;
 }
 
@@ -1457,7 +1500,7 @@ static int mlp_net_for(sddm_ctx *ctx, uint32_t mat, bool create, sddm_ctx::MlpNe
         cudaError_t e;
         sddm_ctx::MlpNet &n = *ctx->nets.back();
         if ((e = n.params.ensure(mlp_param_buffer_bytes())) || (e = n.m.ensure(kMlpParams * 4)) ||
-            (e = n.v.ensure(kMlpParams * 4)))
+            (e = n.v.ensure(kMlpParams * 4)) || (e = ctx->mlp_lists.ensure((size_t)1 << 20)))   // lists of 2^22 rows
             return cuda_fail(e, "surrogate: allocation");
         for (size_t m = 0; m < ctx->mats.size(); ++m)
             if (same_curves(ctx->mats[m], ctx->mats[mat]) && ctx->net_of_mat[m] < 0) ctx->net_of_mat[m] = id;
@@ -1718,8 +1761,10 @@ int sddm_glass_eval(sddm_ctx *ctx, uint32_t mat, int n, const float *cos_theta, 
         a.raw = mode == SDDM_BSDF_MLP_RAW;
         a.fallbacks = nullptr;
         a.test_timeout = (ctx->profile & SDDM_PROFILE_TEST_MLP_TIMEOUT) != 0;
-        int derr[4] = {0, 0, 0, 0};
+        int *const derr = static_cast<int *>(ctx->h_table.p);   // page-locked; no render is under way
         cudaError_t e = cudaSetDevice(ctx->device);
+        if (e == cudaSuccess && ctx->stage_busy) e = cudaStreamSynchronize(ctx->stream);
+        ctx->stage_busy = false;
         // the batch counts lie behind the error word, the two lists in scratch kept for the next call
         const size_t n_batch = ((size_t)n + 31) / 32;
         if (e == cudaSuccess) e = ctx->d_err.ensure(kErrBytes);
@@ -1731,7 +1776,7 @@ int sddm_glass_eval(sddm_ctx *ctx, uint32_t mat, int n, const float *cos_theta, 
         a.list_fail = a.list_pass + n_batch;
         a.list_cap = (uint32_t)n_batch;
         if (e == cudaSuccess) e = launch_mlp_rows(a, ctx->sm_count, ctx->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(derr, ctx->d_err.p, sizeof derr, cudaMemcpyDeviceToHost, ctx->stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(derr, ctx->d_err.p, 4 * sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
         if (e != cudaSuccess) return cuda_fail(e, "sddm_glass_eval (surrogate)");
         if (derr[0] != 0)
