@@ -103,8 +103,8 @@ constexpr int kTraceBatch = SDDM_TRACE_BATCH;
 #define SDDM_TRACE_QUORUM 6
 #endif
 constexpr int kTraceQuorum = SDDM_TRACE_QUORUM;
-// Queue slots a warp reserves per refill atomic (>= 32, so one run always covers a refill).
-constexpr int kRefillChunk = 32;
+// Narrow warps of small waves: lanes at least, and the nodes a cell has on average from which.
+constexpr int kTraceMinLanes = 4, kTraceDeepCell = 64;
 // Rays a warp buffers in shared memory before appending them to the staging area.
 constexpr int kPushBuf = 32;
 
@@ -145,6 +145,15 @@ __global__ void __launch_bounds__(128, SDDM_TRACE_MIN_BLOCKS) k_trace_wave(KArgs
     if (total <= 0) return;
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
+    // A wave with fewer rays than lanes there are spreads over more warps of fewer
+    // lanes: a warp's rounds last as long as its longest lane's, so narrow warps
+    // answer sooner. At least 32 / 8 / 4 / 2 lanes: photon-mapped hotel room 6.36 /
+    // 6.07 / 5.96 / 5.87 ms, hotel room 100 x 100 x 4 spp 1.47 / 1.37 / 1.35 / 1.37.
+    // In cells of a few nodes the claims cost more than the rounds (coated tiny room
+    // 926 / 943 / 943 us): these keep whole warps.
+    const int n_warps = (int)(gridDim.x * (blockDim.x >> 5)), per_warp = (total + n_warps - 1) / n_warps;
+    const bool deep = g.node_cap >= (int64_t)kTraceDeepCell * g.n_cells;
+    const int lanes = deep ? min(32, max(kTraceMinLanes, per_warp)) : 32, batch = max(1, lanes * kTraceBatch / 32);
     const unsigned lt_mask = (1u << lane) - 1u;
     const int64_t np = a.ps.np;
     unsigned n_cross = 0, n_vis = 0, n_cont = 0;   // n_cont: crossings carried on by the lane
@@ -154,7 +163,7 @@ __global__ void __launch_bounds__(128, SDDM_TRACE_MIN_BLOCKS) k_trace_wave(KArgs
     float4 *pbuf = s_push[threadIdx.x >> 5];
     int nbuf = 0;              // rays in the warp's buffer (uniform)
     int idx = -1;              // queue index of this lane's ray, -1 = none
-    bool exhausted = false;    // no ray left for this lane
+    bool exhausted = lane >= lanes;   // no ray left for this lane
     __shared__ unsigned long long s_run[128 / 32][2];    // per warp: reserved run [begin, end) of queue slots
     unsigned long long *run = s_run[threadIdx.x >> 5];
     if (lane == 0) run[0] = run[1] = 0;
@@ -177,7 +186,7 @@ __global__ void __launch_bounds__(128, SDDM_TRACE_MIN_BLOCKS) k_trace_wave(KArgs
         const unsigned m_fin = __ballot_sync(full, t.fin);
         const unsigned m_need = __ballot_sync(full, idx < 0 && !exhausted);
         const unsigned m_busy = __ballot_sync(full, idx >= 0 && !t.fin);
-        if (m_busy == 0 || __popc(m_fin | m_need) >= kTraceBatch) {
+        if (m_busy == 0 || __popc(m_fin | m_need) >= batch) {
             if ((m_fin | m_need) == 0) break;
             // 1a. finished lanes: final result, or hand-off to the neighbouring cell
             bool want = false;
@@ -276,8 +285,8 @@ __global__ void __launch_bounds__(128, SDDM_TRACE_MIN_BLOCKS) k_trace_wave(KArgs
                 __syncwarp();
             }
             // 1b. idle lanes take the next rays of the queue, from a run of
-            //     kRefillChunk queue slots the warp reserves at a time (one
-            //     atomic per run instead of one per refill)
+            //     queue slots the warp reserves at a time, one for each of its
+            //     lanes (one atomic per run instead of one per refill)
             const bool need = idx < 0 && !exhausted;
             const unsigned m = __ballot_sync(full, need);
             if (m) {
@@ -286,7 +295,7 @@ __global__ void __launch_bounds__(128, SDDM_TRACE_MIN_BLOCKS) k_trace_wave(KArgs
                 const unsigned long long avail = cend - cbeg;
                 unsigned long long nb = 0;
                 if (avail < want_n) {
-                    if (lane == 0) nb = atomicAdd(Q.ctl + 1, (unsigned long long)kRefillChunk);
+                    if (lane == 0) nb = atomicAdd(Q.ctl + 1, (unsigned long long)lanes);
                     nb = __shfl_sync(full, nb, 0);
                 }
                 const unsigned rank = __popc(m & lt_mask);
@@ -297,7 +306,7 @@ __global__ void __launch_bounds__(128, SDDM_TRACE_MIN_BLOCKS) k_trace_wave(KArgs
                         run[0] = cbeg + want_n;
                     } else {
                         run[0] = nb + (want_n - avail);
-                        run[1] = nb + kRefillChunk;
+                        run[1] = nb + lanes;
                     }
                 }
                 __syncwarp();

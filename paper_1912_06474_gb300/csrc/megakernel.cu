@@ -258,6 +258,7 @@ constexpr int kMrEmit = 1, kMrResolve = 2, kMrDiffuse = 4, kMrConductor = 8, kMr
 #define SDDM_MEGA_MIN_BLOCKS 8
 #endif
 constexpr int kMegaBatch = SDDM_MEGA_BATCH;
+constexpr int kMegaMinLanes = 2;   // lanes of a warp that take paths, at least
 constexpr int kMegaWarps = 2;      // warps of a block: small images spread over more SMs
 constexpr int kMegaItems = 96;     // chunks worked through between two sums
 static_assert(4 * kMegaItems >= kBranchTerms, "the two share their place");
@@ -354,7 +355,8 @@ __device__ __forceinline__ float3 mega_chunk(const MegaArgs &a, const MegaRec &m
 }
 
 template <bool COUNT, bool FILMS>
-__global__ void __launch_bounds__(32 * kMegaWarps, SDDM_MEGA_MIN_BLOCKS) k_megakernel(const __grid_constant__ MegaArgs a) {
+__global__ void __launch_bounds__(32 * kMegaWarps, SDDM_MEGA_MIN_BLOCKS) k_megakernel(const __grid_constant__ MegaArgs a,
+                                                                                           int lanes, int batch) {
     extern __shared__ __align__(16) unsigned char s_mega[];
     const DevScene &sc = a.sc;
     const int L = sc.L, Lp = sc.Lp, n_chunk = Lp >> 2, M = sc.n_mat;
@@ -370,7 +372,7 @@ __global__ void __launch_bounds__(32 * kMegaWarps, SDDM_MEGA_MIN_BLOCKS) k_megak
     enum { kIdle, kExt, kShadow };
     int mode = kIdle, b = 0;
     int64_t g = 0;                // the lane's path
-    bool dry = false;             // no path left for this lane
+    bool dry = lane >= lanes;     // no path left for this lane
     bool prev_specular = true, t_set = false;   // t_set: the lane's row holds the throughput (1 until a weight)
     V3 rd = v3(0.f, 0.f, 0.f);    // direction of the query under way
     V3 ro = rd;
@@ -388,7 +390,7 @@ __global__ void __launch_bounds__(32 * kMegaWarps, SDDM_MEGA_MIN_BLOCKS) k_megak
     for (;;) {
         const unsigned m_wait = __ballot_sync(full, t.fin || (mode == kIdle && !dry));
         const unsigned m_busy = __ballot_sync(full, mode != kIdle && !t.fin);
-        if (m_busy == 0 || __popc(m_wait) >= kMegaBatch) {
+        if (m_busy == 0 || __popc(m_wait) >= batch) {
             if (m_wait == 0) break;
             int next_mode = kIdle;        // the lane's next query, where it has one
             V3 no = ro, nd = rd;
@@ -684,15 +686,24 @@ static cudaError_t launch_plain(const MegaArgs &a, cudaStream_t stream) {
         e = cudaFuncSetAttribute(k_megakernel<COUNT, FILMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) e = cudaMemsetAsync(a.cursor, 0, sizeof(unsigned long long), stream);
     if (e != cudaSuccess) return e;
-    // one wave of resident blocks, fewer when there are not the paths for them
-    const int64_t want = (a.path_count + 32 * kMegaWarps - 1) / (32 * kMegaWarps);
-    int per_sm = 1;
-    if (want > a.sm_count) {
+    // One wave of resident blocks. An image with fewer paths than lanes there are
+    // spreads over more warps of fewer lanes: a warp's rounds last as long as its
+    // longest lane's, so narrow warps answer sooner (at least 32 / 8 / 4 / 2 lanes:
+    // tiny room 64 x 64 x 1 spp 70 / 56 / 50 / 49 us, hotel room 654 / 465 / 386 /
+    // 330 us, 128 x 128 x 2 spp 759 / 677 / 683 / 692 us).
+    constexpr int kWarpsPerSm = kMegaWarps * SDDM_MEGA_MIN_BLOCKS;
+    const int64_t warps = (int64_t)a.sm_count * kWarpsPerSm, per_warp = (a.path_count + warps - 1) / warps;
+    const int lanes = (int)(per_warp < kMegaMinLanes ? kMegaMinLanes : per_warp < 32 ? per_warp : 32);
+    const int batch = lanes * kMegaBatch / 32 > 1 ? lanes * kMegaBatch / 32 : 1;
+    const int64_t want = (a.path_count + lanes * kMegaWarps - 1) / (lanes * kMegaWarps);
+    int64_t most = want;
+    if (lanes == 32) {
+        int per_sm = 1;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_megakernel<COUNT, FILMS>, 32 * kMegaWarps, smem);
         if (e != cudaSuccess) return e;
+        most = (int64_t)a.sm_count * (per_sm > 0 ? per_sm : 1);
     }
-    const int64_t most = (int64_t)a.sm_count * (per_sm > 0 ? per_sm : 1);
-    k_megakernel<COUNT, FILMS><<<(unsigned)(want < most ? want : most), 32 * kMegaWarps, smem, stream>>>(a);
+    k_megakernel<COUNT, FILMS><<<(unsigned)(want < most ? want : most), 32 * kMegaWarps, smem, stream>>>(a, lanes, batch);
     return cudaGetLastError();
 }
 
