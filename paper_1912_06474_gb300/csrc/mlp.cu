@@ -82,11 +82,10 @@ __device__ __forceinline__ void features(float c, float lam, float s, float alph
 }
 
 // ------------------------------------------------------------- inference
-// The network runs on the fifth-generation tensor cores (tcgen05): a CTA of
-// four warps carries a tile of 128 rows through the hidden layers, one row
-// per thread. For each layer one thread issues the MMAs (M = 128, N = 64,
+// The network runs on the fifth-generation tensor cores (tcgen05): four warps, a
+// group, carry a tile of 128 rows through the hidden layers, one row per thread. For each layer one thread issues the MMAs (M = 128, N = 64,
 // K = 16 each, BF16 operands from shared memory, FP32 accumulators in tensor
-// memory), the CTA waits on an mbarrier that the tensor core arrives on when
+// memory), the group waits on an mbarrier that the tensor core arrives on when
 // they are done, and every warp reads back its 32 rows of accumulators
 // (tensor-memory lanes 32w .. 32w + 31 belong to warp w), applies SiLU and
 // writes the BF16 activations into the A operand of the next layer.
@@ -110,7 +109,12 @@ __device__ __forceinline__ void features(float c, float lam, float s, float alph
 // swizzle: 8-row x 16-byte core matrices, the core matrices of one 8-row group
 // side by side along K (128 B apart, the leading-dimension offset) and the
 // 8-row groups one after the other (the stride offset).
-constexpr int kTcRows = 128;          // rows per tile = threads per CTA = TMEM lanes
+#ifndef SDDM_MLP_GROUPS
+#define SDDM_MLP_GROUPS 4
+#endif
+constexpr int kTcRows = 128;          // rows per tile = threads of a group = TMEM lanes
+constexpr int kTcGroups = SDDM_MLP_GROUPS;   // tiles a CTA has under way, a group of four warps each
+constexpr int kTcThreads = kTcRows * kTcGroups;
 constexpr int kTcCols = 64;           // TMEM columns: one 128 x 64 FP32 accumulator
 constexpr int kChA = 10;              // A chunks per 8-row group: 8 activations + bias ones + zero
 constexpr int kChB1 = 2;              // layer-1 B: K = 16
@@ -130,8 +134,8 @@ struct __align__(128) TcWeights {
 static_assert(sizeof(TcWeights) % 16 == 0, "bulk copies move multiples of 16 bytes");
 struct __align__(128) TcSmem {
     TcWeights w;
-    __nv_bfloat16 a[kTcRows * kChA * 8];    // activations / inputs, K-major core matrices
-    unsigned long long mbar, mbar_w;        // MMA completion; weights arrived
+    __nv_bfloat16 a[kTcGroups][kTcRows * kChA * 8];   // per tile: activations / inputs, K-major core matrices
+    unsigned long long mbar[kTcGroups], mbar_w;       // MMA completion per tile; weights arrived
     uint32_t tmem;
 };
 
@@ -191,29 +195,35 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, uint32
     return false;
 }
 
-// 64 consecutive FP32 accumulator columns of this thread's TMEM lane; the
+// 32 consecutive FP32 accumulator columns of this thread's TMEM lane; the
 // wait is in the same statement, so no use of the registers can precede it.
-__device__ __forceinline__ void tmem_ld64(uint32_t taddr, float v[64]) {
-    uint32_t r[64];
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float v[32]) {
+    uint32_t r[32];
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x64.b32 "
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
         "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,"
-        "%32,%33,%34,%35,%36,%37,%38,%39,%40,%41,%42,%43,%44,%45,%46,%47,"
-        "%48,%49,%50,%51,%52,%53,%54,%55,%56,%57,%58,%59,%60,%61,%62,%63}, [%64];\n\t"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n\t"
         "tcgen05.wait::ld.sync.aligned;\n"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
           "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
           "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]),
-          "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]), "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39]),
-          "=r"(r[40]), "=r"(r[41]), "=r"(r[42]), "=r"(r[43]), "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47]),
-          "=r"(r[48]), "=r"(r[49]), "=r"(r[50]), "=r"(r[51]), "=r"(r[52]), "=r"(r[53]), "=r"(r[54]), "=r"(r[55]),
-          "=r"(r[56]), "=r"(r[57]), "=r"(r[58]), "=r"(r[59]), "=r"(r[60]), "=r"(r[61]), "=r"(r[62]), "=r"(r[63])
+          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
         : "r"(taddr)
         : "memory");
 #pragma unroll
-    for (int i = 0; i < 64; ++i) v[i] = __uint_as_float(r[i]);
+    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// Barrier of a tile's four warps; whether any of their threads passes `flag`.
+__device__ __forceinline__ bool group_sync_or(int group, bool flag) {
+    uint32_t any;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\t"
+        "barrier.cta.red.or.pred q, %2, %3, p;\n\tselp.u32 %0, 1, 0, q;\n\t}\n"
+        : "=r"(any)
+        : "r"((uint32_t)flag), "r"(group + 1), "n"(kTcRows)
+        : "memory");
+    return any != 0;
 }
 
 // SiLU of z given h = z / 2.
@@ -252,12 +262,10 @@ __global__ void __launch_bounds__(256) k_mlp_pack(const float *__restrict__ p, T
     if (threadIdx.x < 2) s.b4[threadIdx.x] = p[OFF_B4 + threadIdx.x];
 }
 
-// A columns 64..79 of every row: [1, 1, 0, ...] against the biases' two parts.
-__device__ void tc_put_bias_columns(TcSmem &s) {
-    for (int i = threadIdx.x; i < kTcRows * 16; i += blockDim.x) {
-        const int r = i >> 4, k = 64 + (i & 15);
-        s.a[kmaj(r, k, kChA)] = __float2bfloat16_rn(k < 66 ? 1.0f : 0.0f);
-    }
+// A columns 64..79 of this thread's row: [1, 1, 0, ...] against the biases' two parts.
+__device__ __forceinline__ void tc_put_bias_columns(__nv_bfloat16 *a, int row) {
+    *reinterpret_cast<uint4 *>(a + kmaj(row, 64, kChA)) = make_uint4(pack_bf16x2(1.0f, 1.0f), 0u, 0u, 0u);
+    *reinterpret_cast<uint4 *>(a + kmaj(row, 72, kChA)) = make_uint4(0u, 0u, 0u, 0u);
 }
 
 // Byte offset of the packed image behind the FP32 parameters in one buffer.
@@ -267,7 +275,7 @@ __device__ __forceinline__ const TcWeights *weight_image(const float *params) {
 }
 
 // This thread's row of layer-1 A: [x_hi | x_lo], then [1, 1, 0 ...].
-__device__ __forceinline__ void tc_put_inputs(TcSmem &s, int row, const float x[4]) {
+__device__ __forceinline__ void tc_put_inputs(__nv_bfloat16 *a, int row, const float x[4]) {
     float hi[4], lo[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -277,20 +285,26 @@ __device__ __forceinline__ void tc_put_inputs(TcSmem &s, int row, const float x[
     const uint4 c0 = make_uint4(pack_bf16x2(hi[0], hi[1]), pack_bf16x2(hi[2], hi[3]), pack_bf16x2(lo[0], lo[1]),
                                 pack_bf16x2(lo[2], lo[3]));
     const uint4 c1 = make_uint4(pack_bf16x2(1.0f, 1.0f), 0u, 0u, 0u);
-    *reinterpret_cast<uint4 *>(s.a + kmaj(row, 0, kChA)) = c0;
-    *reinterpret_cast<uint4 *>(s.a + kmaj(row, 8, kChA)) = c1;
+    *reinterpret_cast<uint4 *>(a + kmaj(row, 0, kChA)) = c0;
+    *reinterpret_cast<uint4 *>(a + kmaj(row, 8, kChA)) = c1;
 }
 
-// SiLU of this thread's 64 accumulators (h = z / 2), as BF16 into its A row.
-__device__ __forceinline__ void tc_put_hidden(TcSmem &s, int row, const float v[64]) {
+// SiLU of this thread's 64 accumulators (h = z / 2), as BF16 into its A row, half
+// of them in registers at a time.
+__device__ __forceinline__ void tc_put_hidden(__nv_bfloat16 *a, int row, uint32_t taddr) {
 #pragma unroll
-    for (int c = 0; c < 8; ++c) {
-        uint4 u;
-        u.x = pack_bf16x2(silu_h(v[8 * c + 0]), silu_h(v[8 * c + 1]));
-        u.y = pack_bf16x2(silu_h(v[8 * c + 2]), silu_h(v[8 * c + 3]));
-        u.z = pack_bf16x2(silu_h(v[8 * c + 4]), silu_h(v[8 * c + 5]));
-        u.w = pack_bf16x2(silu_h(v[8 * c + 6]), silu_h(v[8 * c + 7]));
-        *reinterpret_cast<uint4 *>(s.a + kmaj(row, 8 * c, kChA)) = u;
+    for (int half = 0; half < 2; ++half) {
+        float v[32];
+        tmem_ld32(taddr + 32 * half, v);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            uint4 u;
+            u.x = pack_bf16x2(silu_h(v[8 * c + 0]), silu_h(v[8 * c + 1]));
+            u.y = pack_bf16x2(silu_h(v[8 * c + 2]), silu_h(v[8 * c + 3]));
+            u.z = pack_bf16x2(silu_h(v[8 * c + 4]), silu_h(v[8 * c + 5]));
+            u.w = pack_bf16x2(silu_h(v[8 * c + 6]), silu_h(v[8 * c + 7]));
+            *reinterpret_cast<uint4 *>(a + kmaj(row, 32 * half + 8 * c, kChA)) = u;
+        }
     }
 }
 
@@ -471,14 +485,14 @@ __device__ __forceinline__ int64_t batch_row(const MlpRows &a, const BatchShape 
     row_input(a, r, a.n, in);
     return r;
 }
-// Rows of a list, and row i of it (false past its end).
+// Rows of a list, and row i of it (false past its end) given its full batches' rows
+// and its short batches.
 __device__ __forceinline__ int64_t list_rows(const MlpRows &a, const BatchShape &s, int full) {
     return 32 * (int64_t)a.list_cnt[full] + (int64_t)s.tail * a.list_cnt[full + 1];
 }
-__device__ __forceinline__ bool list_row(const MlpRows &a, const BatchShape &s, int full, int64_t i, uint32_t &b,
-                                         int &k) {
+__device__ __forceinline__ bool list_row(const MlpRows &a, const BatchShape &s, int full, int64_t n_full, uint32_t n_short,
+                                         int64_t i, uint32_t &b, int &k) {
     const uint32_t *list = full == kPassFull ? a.list_pass : a.list_fail;
-    const int64_t n_full = 32 * (int64_t)a.list_cnt[full];
     if (i < n_full) {
         b = list[i >> 5];
         k = (int)(i & 31);
@@ -487,7 +501,7 @@ __device__ __forceinline__ bool list_row(const MlpRows &a, const BatchShape &s, 
     if (s.tail == 0) return false;
     const uint64_t j = (uint64_t)(i - n_full);
     const uint32_t e = (j >> 32) == 0 ? (uint32_t)j / (uint32_t)s.tail : (uint32_t)(j / (uint32_t)s.tail);
-    if (e >= a.list_cnt[full + 1]) return false;
+    if (e >= n_short) return false;
     b = list[a.list_cap - 1 - e];
     k = (int)((uint32_t)j - e * (uint32_t)s.tail);
     return true;
@@ -517,28 +531,40 @@ __device__ __forceinline__ void list_push(const MlpRows &a, int full, bool is_sh
 // stops.
 constexpr int kNetAll = 0, kNetProbe = 1, kNetList = 2;
 #ifndef SDDM_MLP_MINB
-#define SDDM_MLP_MINB 5   // resident 128-thread tile CTAs per SM (96 registers; shared memory admits 5)
+#define SDDM_MLP_MINB 2   // resident CTAs per SM
 #endif
+// Several tiles per CTA share one copy of the weights: four groups and two CTAs
+// are eight tiles on an SM (64 registers a thread, 105 KB per CTA, 512 TMEM
+// columns), which overlap one another's barriers, MMAs and tensor-memory loads
+// with the SiLU's tanh, the bound (192 a row at 16 a cycle and SM: 161 us per 2^22
+// rows). A CTA per tile with a copy each fits five times, of which four ran.
+// Groups x CTAs 1 x 5 / 2 x 3 / 4 x 2: 747 M rows of a facade render in 45.2 / 44.1 /
+// 42.1 ms, 2^24 explicit rows 1007 / 1020 / 983 us.
 template <bool FILMS, int ROWS>
-__global__ void __launch_bounds__(kTcRows, SDDM_MLP_MINB) k_mlp_net(const __grid_constant__ MlpRows a) {
-    __shared__ TcSmem s;
-    const int tid = threadIdx.x, warp = tid >> 5;
+__global__ void __launch_bounds__(kTcThreads, SDDM_MLP_MINB) k_mlp_net(const __grid_constant__ MlpRows a) {
+    extern __shared__ __align__(128) unsigned char s_mlp[];
+    TcSmem &s = *reinterpret_cast<TcSmem *>(s_mlp);
+    const int tid = threadIdx.x, warp = tid >> 5, group = tid / kTcRows, row = tid % kTcRows;
     BatchShape shape{};
     if (ROWS != kNetAll) shape = batch_shape(a);
     const int64_t total = ROWS == kNetAll ? mlp_total_rows(a) : ROWS == kNetProbe ? shape.n : list_rows(a, shape, kPassFull);
     const int64_t n_tiles = (total + kTcRows - 1) / kTcRows;
     if (blockIdx.x >= n_tiles) return;   // nothing set up yet
-    const uint32_t mbar = smem_addr(&s.mbar), mbar_w = smem_addr(&s.mbar_w);
+    int64_t n_full = 0;
+    uint32_t n_short = 0;
+    if (ROWS == kNetList) {
+        n_full = 32 * (int64_t)a.list_cnt[kPassFull];
+        n_short = a.list_cnt[kPassFull + 1];
+    }
+    const uint32_t mbar = smem_addr(&s.mbar[group]), mbar_w = smem_addr(&s.mbar_w);
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&s.tmem)),
-                     "r"((uint32_t)kTcCols)
+                     "r"((uint32_t)(kTcCols * kTcGroups))
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    if (tid == 0) {
-        mbar_init(mbar);
-        mbar_init(mbar_w);
-    }
+    if (row == 0) mbar_init(mbar);
+    if (tid == 0) mbar_init(mbar_w);
     __syncthreads();
     // the packed weights by one bulk copy (the TMA engine), completion on mbar_w
     if (tid == 0) {
@@ -550,15 +576,16 @@ __global__ void __launch_bounds__(kTcRows, SDDM_MLP_MINB) k_mlp_net(const __grid
                      "l"(weight_image(a.params)), "r"((uint32_t)sizeof(TcWeights)), "r"(mbar_w)
                      : "memory");
     }
-    tc_put_bias_columns(s);
+    __nv_bfloat16 *const act = s.a[group];
+    tc_put_bias_columns(act, row);
     const bool w_ok = mbar_wait(mbar_w, 0u, kMbarTries);
     fence_async_smem();
     tc_fence_before();
     const bool w_failed = __syncthreads_or(!w_ok) != 0;
     tc_fence_after();
-    const uint32_t tmem = s.tmem;
-    const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16);   // this warp's 32 lanes
-    const uint32_t sa = smem_addr(s.a), sb1 = smem_addr(s.w.b1), sb2 = smem_addr(s.w.b2), sb3 = smem_addr(s.w.b3);
+    const uint32_t tmem = s.tmem, acc = tmem + (uint32_t)(kTcCols * group);   // this group's accumulators
+    const uint32_t taddr = acc + ((uint32_t)((warp & 3) * 32) << 16);         // this warp's 32 lanes of them
+    const uint32_t sa = smem_addr(act), sb1 = smem_addr(s.w.b1), sb2 = smem_addr(s.w.b2), sb3 = smem_addr(s.w.b3);
     constexpr uint32_t kSboA = kChA * 128, kSboB1 = kChB1 * 128, kSboB = kChB * 128;
     if (a.rows && blockIdx.x == 0 && tid == 0) atomicAdd(a.rows, (unsigned long long)total);
     uint32_t phase = 0;
@@ -566,25 +593,25 @@ __global__ void __launch_bounds__(kTcRows, SDDM_MLP_MINB) k_mlp_net(const __grid
     // failure-path test: CTA 0 issues nothing, so its first wait runs out
     const bool skip = a.test_timeout && blockIdx.x == 0;
     const uint32_t tries = skip ? kMbarTriesTest : kMbarTries;
-    // One layer: the A rows written by every thread are made visible to the
-    // tensor core, the CTA synchronises (and learns whether any thread's
+    // One layer: the A rows written by the group's threads are made visible to
+    // the tensor core, the group synchronises (and learns whether any thread's
     // previous wait ran out: then it stops, false), one thread issues the
     // MMAs, and every thread waits on the mbarrier for their completion.
     auto layer = [&](int l) -> bool {
         fence_async_smem();
         tc_fence_before();
-        if (__syncthreads_or(failed)) return false;
-        if (tid == 0 && !skip) {
+        if (group_sync_or(group, failed)) return false;
+        if (row == 0 && !skip) {
             tc_fence_after();
             if (l == 1) {
-                tc_mma(tmem, tc_desc(sa, 128, kSboA), tc_desc(sb1, 128, kSboB1), kIdescHidden, 0u);
+                tc_mma(acc, tc_desc(sa, 128, kSboA), tc_desc(sb1, 128, kSboB1), kIdescHidden, 0u);
             } else {
                 const uint32_t sb = l == 2 ? sb2 : sb3;
 #pragma unroll
                 for (int ks = 0; ks < 4; ++ks)
-                    tc_mma(tmem, tc_desc(sa + 256 * ks, 128, kSboA), tc_desc(sb + 256 * ks, 128, kSboB), kIdescHidden,
+                    tc_mma(acc, tc_desc(sa + 256 * ks, 128, kSboA), tc_desc(sb + 256 * ks, 128, kSboB), kIdescHidden,
                            ks > 0 ? 1u : 0u);
-                tc_mma(tmem, tc_desc(sa + 1024, 128, kSboA), tc_desc(sb + 1024, 128, kSboB), kIdescHidden, 1u);
+                tc_mma(acc, tc_desc(sa + 1024, 128, kSboA), tc_desc(sb + 1024, 128, kSboB), kIdescHidden, 1u);
             }
             tc_commit(mbar);
         }
@@ -593,8 +620,9 @@ __global__ void __launch_bounds__(kTcRows, SDDM_MLP_MINB) k_mlp_net(const __grid
         tc_fence_after();
         return true;
     };
-    for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-        int64_t r = tile * kTcRows + tid;
+    // a CTA's groups take tiles a grid apart, so that few tiles spread over the SMs
+    for (int64_t tile = blockIdx.x + (int64_t)group * gridDim.x; tile < n_tiles; tile += (int64_t)kTcGroups * gridDim.x) {
+        int64_t r = tile * kTcRows + row;
         RowIn in;
         bool valid;
         uint32_t batch = 0;
@@ -612,7 +640,7 @@ __global__ void __launch_bounds__(kTcRows, SDDM_MLP_MINB) k_mlp_net(const __grid
                     k = (int)(pr.x % (uint32_t)(is_short ? shape.tail : 32));
                 }
             } else {
-                valid = list_row(a, shape, kPassFull, r, batch, k);
+                valid = list_row(a, shape, kPassFull, n_full, n_short, r, batch, k);
             }
             if (valid)
                 r = batch_row(a, shape, batch, k, in);
@@ -621,7 +649,7 @@ __global__ void __launch_bounds__(kTcRows, SDDM_MLP_MINB) k_mlp_net(const __grid
         }
         float x[4];
         features(in.c, in.lam, in.s, row_alpha_d<FILMS>(a.sc, in), x);
-        tc_put_inputs(s, tid, x);
+        tc_put_inputs(act, row, x);
         if (ROWS == kNetList && a.mode == 0) {
             // explicit rows are looked at one by one: a warp holds the rows of
             // one batch (full batches start at multiples of 32, one short batch
@@ -629,21 +657,22 @@ __global__ void __launch_bounds__(kTcRows, SDDM_MLP_MINB) k_mlp_net(const __grid
             const unsigned out = __ballot_sync(kFull, valid && !row_in_box(a, in));
             if (out) list_push(a, kFailFull, batch_short(a, shape, batch), batch, (tid & 31) == 0);
         }
-        float v[64];
         if (!layer(1)) break;
-        tmem_ld64(taddr, v);
-        tc_put_hidden(s, tid, v);
+        tc_put_hidden(act, row, taddr);
         if (!layer(2)) break;
-        tmem_ld64(taddr, v);
-        tc_put_hidden(s, tid, v);
+        tc_put_hidden(act, row, taddr);
         if (!layer(3)) break;
-        tmem_ld64(taddr, v);
         float y0 = s.w.b4[0], y1 = s.w.b4[1];
 #pragma unroll
-        for (int j = 0; j < H; ++j) {
-            const float h = silu_h(v[j]);
-            y0 = fmaf(s.w.w4[0][j], h, y0);
-            y1 = fmaf(s.w.w4[1][j], h, y1);
+        for (int half = 0; half < 2; ++half) {
+            float v[32];
+            tmem_ld32(taddr + 32 * half, v);
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+                const float h = silu_h(v[j]);
+                y0 = fmaf(s.w.w4[0][32 * half + j], h, y0);
+                y1 = fmaf(s.w.w4[1][32 * half + j], h, y1);
+            }
         }
         const float2 y = make_float2(out_to_rt(y0), out_to_rt(y1));
         if (ROWS == kNetProbe) {
@@ -681,7 +710,8 @@ __global__ void __launch_bounds__(kTcRows, SDDM_MLP_MINB) k_mlp_net(const __grid
     __syncthreads();
     if (warp == 0) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)kTcCols)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                     "r"((uint32_t)(kTcCols * kTcGroups))
                      : "memory");
     }
 }
@@ -690,12 +720,13 @@ __global__ void __launch_bounds__(kTcRows, SDDM_MLP_MINB) k_mlp_net(const __grid
 template <bool FILMS>
 __global__ void __launch_bounds__(256) k_mlp_fallback(MlpRows a) {
     const BatchShape shape = batch_shape(a);
-    const int64_t total = list_rows(a, shape, kFailFull);
+    const int64_t total = list_rows(a, shape, kFailFull), n_full = 32 * (int64_t)a.list_cnt[kFailFull];
+    const uint32_t n_short = a.list_cnt[kFailFull + 1];
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
         uint32_t b;
         int k;
-        if (!list_row(a, shape, kFailFull, i, b, k)) break;
+        if (!list_row(a, shape, kFailFull, n_full, n_short, i, b, k)) break;
         RowIn in;
         const int64_t r = batch_row(a, shape, b, k, in);
         store_row(a, r, in, exact_row<FILMS>(a, in));
@@ -1159,21 +1190,24 @@ static int resident_per_sm(K kernel, int threads, int cap) {
     return n < cap ? n : cap;
 }
 
-// Tile CTAs per SM: as many as the registers and shared memory allow
+// CTAs per SM: as many as the registers and shared memory allow
 // (__launch_bounds__ asks for SDDM_MLP_MINB). Tensor memory has 512 columns
-// per SM and each CTA holds kTcCols of them, so up to 512 / kTcCols resident
-// CTAs never wait on one another's allocation.
-static_assert(SDDM_MLP_MINB * kTcCols <= 512, "tensor-memory columns of the resident tile CTAs");
+// per SM and each CTA holds kTcCols for each of its tiles, so resident CTAs never
+// wait on one another's allocation.
+static_assert(SDDM_MLP_MINB * kTcCols * kTcGroups <= 512, "tensor-memory columns of the resident tile CTAs");
 template <bool FILMS, int ROWS>
 static cudaError_t launch_mlp_net(const MlpRows &a, int sm_count, cudaStream_t stream) {
     static bool attr_set = false;
     if (!attr_set) {
         cudaError_t e = cudaFuncSetAttribute(k_mlp_net<FILMS, ROWS>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                              (int)cudaSharedmemCarveoutMaxShared);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_mlp_net<FILMS, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)sizeof(TcSmem));
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
-    k_mlp_net<FILMS, ROWS><<<sm_count * SDDM_MLP_MINB, kTcRows, 0, stream>>>(a);
+    k_mlp_net<FILMS, ROWS><<<sm_count * SDDM_MLP_MINB, kTcThreads, sizeof(TcSmem), stream>>>(a);
     return cudaGetLastError();
 }
 
