@@ -477,13 +477,11 @@ int ddm_photon_pass(const DDMPhotonRun &run, DDMBuffers &buf, cudaStream_t s) {
     *run.launches += 1;
     for (int b = 1; b <= run.max_depth - 1; ++b) {
         for (int w = 0; w < waves; ++w) {
-            k_scatter<<<scatter_blocks, 256, 0, s>>>(a);
-            PM_CHECK(cudaGetLastError());
+            PM_CHECK(launch_after(true, k_scatter, scatter_blocks, 256, 0, s, a));
             Q.flip();
             a.last_wave = w == waves - 1;
             a.g.continue_cells = ddm_wave_continues(run.g, w, waves);
-            k_trace_wave<false><<<trace_blocks, 128, 0, s>>>(a);
-            PM_CHECK(cudaGetLastError());
+            PM_CHECK(launch_after(true, k_trace_wave<false>, trace_blocks, 128, 0, s, a));
             *run.launches += 2;
         }
         a.b = b;

@@ -134,6 +134,7 @@ __device__ __forceinline__ void flush_push_buf(const Queues &Q, const float4 *bu
 // it is read; a bad one is recorded (codes 8-10) and the ray is dropped.
 template <bool COUNT, bool CHECKED = false>
 __global__ void __launch_bounds__(128, SDDM_TRACE_MIN_BLOCKS) k_trace_wave(KArgs a) {
+    grid_entry();
     const Queues &Q = a.Q;
     const DDMScene &g = a.g;
     // the rays of this launch: the whole wave, or one group's range of it

@@ -9,6 +9,33 @@
 
 namespace sddm {
 
+// ------------------------------------------------- overlapped kernel launches
+// First statement of a kernel launched by launch_after: let the kernel after it be
+// launched, and wait until the kernel before it is done and its writes are seen.
+__device__ __forceinline__ void grid_entry() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+// Launch a kernel that may be brought in while the stream's kernel before it
+// drains: its blocks wait for that kernel themselves (grid_entry, before they read
+// anything it wrote), so that launch latency and start-up overlap. After anything
+// but a kernel (a memset, an event), or with early = false, it is an ordinary launch.
+template <typename... P, typename... A>
+inline cudaError_t launch_after(bool early, void (*kernel)(P...), unsigned blocks, unsigned threads, size_t smem,
+                                cudaStream_t stream, A &&...args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // ----------------------------------------------------------- vector helpers
 struct V3 {
     float x, y, z;

@@ -814,8 +814,7 @@ __global__ void __launch_bounds__(kTrainThreads) k_mlp_train_tile(const __grid_c
     const int w = (tid >> 5) & 3, cg = tid >> 7, j0 = cg * kColJ;   // row block, column group, its first MMA tile
     const int cta = blockIdx.x;
     const int cta_row0 = cta * kMlpRowsPerCta;
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");   // samples, and the parameters of the step before
+    grid_entry();   // samples, and the parameters of the step before
     for (int i = tid; i < kMlpRowsPerCta; i += kTrainThreads) {
         const bool ok = cta_row0 + i < a.n_rows;
         const int64_t gr = (a.row0 + cta_row0 + i) % a.n_samples;
@@ -1103,8 +1102,7 @@ __global__ void __launch_bounds__(kAdamThreads) k_mlp_adam(float *params, float 
                                                            float bc2, float *grad_out, float *loss_out,
                                                            float loss_scale) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");   // the gradients of the tile pass
+    grid_entry();   // the gradients of the tile pass
     if (i == kMlpParams && loss_out) *loss_out = ordered_sum(loss_cta, 1, n_cta) * loss_scale;
     if (i >= kMlpParams) return;
     const float gsum = ordered_sum(grad_cta + i, kMlpParams, n_cta);
@@ -1244,26 +1242,6 @@ cudaError_t launch_slab_rows(const MlpRows &a, int sm_count, cudaStream_t stream
     return cudaGetLastError();
 }
 
-// Launch a kernel that may start while the stream's kernel before it drains: it
-// waits for that kernel's results itself (griddepcontrol.wait, before its first
-// read of them), so the launch latency overlaps. Training alternates two kernels
-// of some microseconds each.
-template <typename... KArgs, typename... Args>
-static cudaError_t launch_after(void (*kernel)(KArgs...), int blocks, int threads, size_t smem, cudaStream_t stream,
-                                Args... args) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)blocks);
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr{};
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
 cudaError_t launch_mlp_train_tile(const MlpTrainArgs &a, cudaStream_t stream) {
     static bool attr_set = false;
     const size_t bytes = sizeof(TrainSmem);
@@ -1273,14 +1251,14 @@ cudaError_t launch_mlp_train_tile(const MlpTrainArgs &a, cudaStream_t stream) {
         attr_set = true;
     }
     const int n_cta = (a.n_rows + kMlpRowsPerCta - 1) / kMlpRowsPerCta;
-    return launch_after(k_mlp_train_tile, n_cta, kTrainThreads, bytes, stream, a);
+    return launch_after(true, k_mlp_train_tile, n_cta, kTrainThreads, bytes, stream, a);
 }
 
 cudaError_t launch_mlp_adam(float *params, float *m, float *v, const float *grad_cta, const float *loss_cta, int n_cta,
                             float lr, float bc1, float bc2, float *grad_out, float *loss_out, float loss_scale,
                             cudaStream_t stream) {
     // one thread more than there are parameters: the loss
-    return launch_after(k_mlp_adam, (kMlpParams + kAdamThreads) / kAdamThreads, kAdamThreads, 0, stream, params, m, v,
+    return launch_after(true, k_mlp_adam, (kMlpParams + kAdamThreads) / kAdamThreads, kAdamThreads, 0, stream, params, m, v,
                         grad_cta, loss_cta, n_cta, lr, bc1, bc2, grad_out, loss_out, loss_scale);
 }
 
