@@ -545,8 +545,13 @@ constexpr int kMaxFilms = SDDM_MAX_FILMS;
 // faces incoherently:
 //   R = R_a + T_a T_g R_g tau^2 / (1 - R_g^2 tau^2),  T = T_a T_g tau / (1 - R_g^2 tau^2),
 // per polarisation, averaged.
-static __device__ __noinline__ void coated_RT(float c, float lam_nm, float n_sub, float alpha, float thick, int J,
-                                       const float *nf, const float *kf, const float *tf_nm, float &R, float &T) {
+// JT > 0: that many films, known to the compiler.
+template <int JT>
+__device__ __forceinline__ void coated_RT_films(float c, float lam_nm, float n_sub, float alpha, float thick, int Jn,
+                                                const float *nf, const float *kf, const float *tf_nm, float &R,
+                                                float &T) {
+    const int J = JT > 0 ? JT : Jn;
+    constexpr int kN = JT > 0 ? JT : kMaxFilms;
     if (c <= 0.0f) {
         R = 1.0f;
         T = 0.0f;
@@ -556,7 +561,7 @@ static __device__ __noinline__ void coated_RT(float c, float lam_nm, float n_sub
     const float s2 = fmaf(-c, c, 1.0f);
     const float ct_sub = sqrtf(fmaf(-s2, __frcp_rn(n_sub * n_sub), 1.0f));
     const float tau = expf(-alpha * thick / ct_sub), t2 = tau * tau;
-    Cx N[kMaxFilms], CT[kMaxFilms], CD[kMaxFilms], SD[kMaxFilms];
+    Cx N[kN], CT[kN], CD[kN], SD[kN];
     for (int j = 0; j < J; ++j) {
         N[j] = cx(nf[j], kf[j]);
         const Cx n2 = N[j] * N[j];
@@ -611,12 +616,34 @@ static __device__ __noinline__ void coated_RT(float c, float lam_nm, float n_sub
     R = 0.5f * Rsum;
     T = 0.5f * Tsum;
 }
+static __device__ __noinline__ void coated_RT(float c, float lam_nm, float n_sub, float alpha, float thick, int J,
+                                       const float *nf, const float *kf, const float *tf_nm, float &R, float &T) {
+    coated_RT_films<0>(c, lam_nm, n_sub, alpha, thick, J, nf, kf, tf_nm, R, T);
+}
+// A stack of J films of material m at bin i in state s, all of it in registers.
+template <int J>
+static __device__ __noinline__ float2 coated_few(const DevScene &sc, int m, int i, float c, float s, float alpha,
+                                                 float thick) {
+    float nf[J], kf[J], tf[J], R, T;
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+        const size_t f = ((size_t)m * kMaxFilms + j) * sc.L + i;
+        nf[j] = __ldg(sc.film_n + f);
+        kf[j] = __ldg(sc.film_k + f) + s * __ldg(sc.film_dk + f);
+        tf[j] = __ldg(sc.film_t + (size_t)m * kMaxFilms + j);
+    }
+    coated_RT_films<J>(c, __ldg(sc.lam + i), __ldg(sc.mat_a + (size_t)m * sc.L + i), alpha, thick, J, nf, kf, tf, R, T);
+    return make_float2(R, T);
+}
 
 // R, T of glass material m at wavelength bin i: the bare absorbing slab, or
 // the coated slab when the material carries films (film k = k + s dk).
 // Kernels are instantiated with FILMS = false for scenes without coated glass,
-// which keeps the film code (and its call) out of them entirely.
-template <bool FILMS = true>
+// which keeps the film code (and its call) out of them entirely. DENSE: in kernels
+// that evaluate rows of glass and nothing else, stacks of up to three films (the
+// usual ones) keep their matrices in registers instead of indexed local arrays (the
+// same bits): 262,147 rows of 1 / 2 / 3 films 29.7 / 33.4 / 38.3 -> 25.3 / 29.0 / 32.9 us a call.
+template <bool FILMS = true, bool DENSE = false>
 __device__ __forceinline__ void glass_rt(const DevScene &sc, int m, int i, float c, float s, float thick, float &R,
                                          float &T) {
     const size_t k = (size_t)m * sc.L + i;
@@ -627,6 +654,14 @@ __device__ __forceinline__ void glass_rt(const DevScene &sc, int m, int i, float
         const int J = sc.mat_nfilm ? __ldg(sc.mat_nfilm + m) : 0;
         if (J == 0) {
             slab_RT(c, __ldg(sc.lam + i), __ldg(sc.mat_a + k), alpha, thick, R, T);
+            return;
+        }
+        if (DENSE && J <= 3) {
+            const float2 rt = J == 1   ? coated_few<1>(sc, m, i, c, s, alpha, thick)
+                              : J == 2 ? coated_few<2>(sc, m, i, c, s, alpha, thick)
+                                       : coated_few<3>(sc, m, i, c, s, alpha, thick);
+            R = rt.x;
+            T = rt.y;
             return;
         }
         float nf[kMaxFilms], kf[kMaxFilms], tf[kMaxFilms];

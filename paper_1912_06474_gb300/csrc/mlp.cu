@@ -394,10 +394,10 @@ __device__ __forceinline__ bool row_input(const MlpRows &a, int64_t r, int64_t t
     return true;
 }
 
-template <bool FILMS = true>
+template <bool FILMS = true, bool DENSE = false>
 __device__ __forceinline__ float2 exact_row(const MlpRows &a, const RowIn &in) {
     float R_, T_;
-    glass_rt<FILMS>(a.sc, in.mat, in.bin, in.c, in.s, in.d, R_, T_);
+    glass_rt<FILMS, DENSE>(a.sc, in.mat, in.bin, in.c, in.s, in.d, R_, T_);
     return make_float2(R_, T_);
 }
 
@@ -746,7 +746,7 @@ __global__ void __launch_bounds__(256) k_slab_rows(MlpRows a) {
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < total; r += stride) {
         RowIn in;
         row_input(a, r, total, in);
-        store_row(a, r, in, exact_row<FILMS>(a, in));
+        store_row(a, r, in, exact_row<FILMS, true>(a, in));
     }
 }
 
