@@ -1,4 +1,4 @@
-// Plain baseline: one thread per camera path over the global BVH -- the
+// Plain baseline: a lane per camera path over the global BVH -- the
 // classical parallelisation of Sec. 5 (split the pixels, every worker sees
 // the whole scene) -- computing the same estimator as the DDM path.
 //
@@ -682,8 +682,9 @@ template <bool COUNT, bool FILMS>
 static cudaError_t launch_plain(const MegaArgs &a, cudaStream_t stream) {
     const size_t smem = mega_warp_bytes(a.sc.Lp) * kMegaWarps;
     cudaError_t e = cudaSuccess;
-    if (smem > 48 * 1024)   // more than a block has without asking: over 104 bins
-        e = cudaFuncSetAttribute(k_megakernel<COUNT, FILMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (smem > 48 * 1024)   // more than a block has without asking (over 104 bins); the same for every caller
+        e = cudaFuncSetAttribute(k_megakernel<COUNT, FILMS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(mega_warp_bytes(kMaxL) * kMegaWarps));
     if (e == cudaSuccess) e = cudaMemsetAsync(a.cursor, 0, sizeof(unsigned long long), stream);
     if (e != cudaSuccess) return e;
     // One wave of resident blocks. An image with fewer paths than lanes there are
