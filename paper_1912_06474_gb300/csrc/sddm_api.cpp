@@ -1023,9 +1023,16 @@ int sddm_render(sddm_ctx *ctx, const sddm_render_desc *d, int n, sddm_stats *st)
     std::string key;
     if (graphable) {
         char buf[256];
-        std::snprintf(buf, sizeof buf, "%lld|%d|%d|%d|%d|%lld|%d|%u|%d|%p|%p|%p|%p|%p", (long long)ctx->build_id,
+        // the trained box goes into the kernels' arguments by value, and training again or
+        // setting other weights changes it without moving the parameters
+        uint32_t box[2] = {0, 0};
+        if (mlp_params) {
+            std::memcpy(&box[0], &mlp_dmin, 4);
+            std::memcpy(&box[1], &mlp_dmax, 4);
+        }
+        std::snprintf(buf, sizeof buf, "%lld|%d|%d|%d|%d|%lld|%d|%u|%x|%x|%d|%p|%p|%p|%p|%p", (long long)ctx->build_id,
                       n, d[0].method, d[0].bsdf_mode, (int)any_aov, (long long)ctx->opts.paths_in_flight,
-                      ctx->opts.blocks_per_sm, mlp_params ? d[0].seed : 0u /* the probes' key */, time_trace,
+                      ctx->opts.blocks_per_sm, mlp_params ? d[0].seed : 0u /* the probes' key */, box[0], box[1], time_trace,
                       ctx->d_samples.p, ctx->d_first.p,
                       ctx->ddm_buf.mem, ctx->d_table.p, (const void *)mlp_params);
         key = buf;
