@@ -1194,17 +1194,25 @@ static int resident_per_sm(K kernel, int threads, int cap) {
 // wait on one another's allocation.
 static_assert(SDDM_MLP_MINB * kTcCols * kTcGroups <= 512, "tensor-memory columns of the resident tile CTAs");
 template <bool FILMS, int ROWS>
+static cudaError_t prepare_mlp_net() {
+    const cudaError_t e = cudaFuncSetAttribute(k_mlp_net<FILMS, ROWS>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                               (int)cudaSharedmemCarveoutMaxShared);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(k_mlp_net<FILMS, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TcSmem));
+}
+cudaError_t mlp_prepare_device() {
+    cudaError_t e = cudaFuncSetAttribute(k_mlp_train_tile, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sizeof(TrainSmem));
+    if (e == cudaSuccess) e = prepare_mlp_net<false, kNetAll>();
+    if (e == cudaSuccess) e = prepare_mlp_net<false, kNetProbe>();
+    if (e == cudaSuccess) e = prepare_mlp_net<false, kNetList>();
+    if (e == cudaSuccess) e = prepare_mlp_net<true, kNetAll>();
+    if (e == cudaSuccess) e = prepare_mlp_net<true, kNetProbe>();
+    if (e == cudaSuccess) e = prepare_mlp_net<true, kNetList>();
+    return e;
+}
+template <bool FILMS, int ROWS>
 static cudaError_t launch_mlp_net(const MlpRows &a, int sm_count, cudaStream_t stream) {
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k_mlp_net<FILMS, ROWS>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                             (int)cudaSharedmemCarveoutMaxShared);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_mlp_net<FILMS, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)sizeof(TcSmem));
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
     k_mlp_net<FILMS, ROWS><<<sm_count * SDDM_MLP_MINB, kTcThreads, sizeof(TcSmem), stream>>>(a);
     return cudaGetLastError();
 }
@@ -1243,15 +1251,8 @@ cudaError_t launch_slab_rows(const MlpRows &a, int sm_count, cudaStream_t stream
 }
 
 cudaError_t launch_mlp_train_tile(const MlpTrainArgs &a, cudaStream_t stream) {
-    static bool attr_set = false;
-    const size_t bytes = sizeof(TrainSmem);
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k_mlp_train_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
     const int n_cta = (a.n_rows + kMlpRowsPerCta - 1) / kMlpRowsPerCta;
-    return launch_after(true, k_mlp_train_tile, n_cta, kTrainThreads, bytes, stream, a);
+    return launch_after(true, k_mlp_train_tile, n_cta, kTrainThreads, sizeof(TrainSmem), stream, a);
 }
 
 cudaError_t launch_mlp_adam(float *params, float *m, float *v, const float *grad_cta, const float *loss_cta, int n_cta,

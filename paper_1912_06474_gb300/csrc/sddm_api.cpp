@@ -207,6 +207,7 @@ struct sddm_ctx {
     };
     std::vector<std::unique_ptr<MlpNet>> nets;
     std::vector<int> net_of_mat;     // per material, -1 = none
+    bool mlp_ready = false;          // the surrogate's kernels are prepared on this context's device
     DevBuf mlp_grad_cta, mlp_loss_cta, mlp_scalar, mlp_X, mlp_Y, mlp_lists;
     // CUDA graphs of the render launch sequence, keyed by everything that is
     // baked into kernel parameters (sizes, buffer addresses, build)
@@ -1495,16 +1496,26 @@ static bool same_curves(const Material &a, const Material &b) {
     return true;
 }
 
+// The context's device current and the surrogate's kernels prepared on it.
+static cudaError_t mlp_device(sddm_ctx *ctx) {
+    cudaError_t e = cudaSetDevice(ctx->device);
+    if (e == cudaSuccess && !ctx->mlp_ready && (e = mlp_prepare_device()) == cudaSuccess) ctx->mlp_ready = true;
+    return e;
+}
+
+// The network of a glass material (with `create`, a new one where there is none),
+// its device current.
 static int mlp_net_for(sddm_ctx *ctx, uint32_t mat, bool create, sddm_ctx::MlpNet **out) {
     if (mat >= ctx->mats.size() || ctx->mats[mat].kind != kGlass)
         return fail(SDDM_ERR_INVALID_ARG, "surrogate: material is not a glass slab");
     ctx->net_of_mat.resize(ctx->mats.size(), -1);
     int id = ctx->net_of_mat[mat];
+    if (id < 0 && !create) return fail(SDDM_ERR_MLP_UNTRAINED, "surrogate: no weights for this material");
+    cudaError_t e = mlp_device(ctx);
+    if (e != cudaSuccess) return cuda_fail(e, "surrogate: device");
     if (id < 0) {
-        if (!create) return fail(SDDM_ERR_MLP_UNTRAINED, "surrogate: no weights for this material");
         ctx->nets.emplace_back(new sddm_ctx::MlpNet());
         id = (int)ctx->nets.size() - 1;
-        cudaError_t e;
         sddm_ctx::MlpNet &n = *ctx->nets.back();
         if ((e = n.params.ensure(mlp_param_buffer_bytes())) || (e = n.m.ensure(kMlpParams * 4)) ||
             (e = n.v.ensure(kMlpParams * 4)) || (e = ctx->mlp_lists.ensure((size_t)1 << 20)))   // lists of 2^22 rows
@@ -1536,7 +1547,7 @@ int sddm_mlp_train(sddm_ctx *ctx, uint32_t mat, const sddm_mlp_train_opts *opts,
     sddm_ctx::MlpNet *net = nullptr;
     int rc = mlp_net_for(ctx, mat, true, &net);
     if (rc != SDDM_OK) return rc;
-    cudaError_t e = cudaSetDevice(ctx->device);
+    cudaError_t e;
     cudaStream_t s = ctx->stream;
     const int n_cta = o.batch / kMlpRowsPerCta;
     if ((e = ctx->mlp_grad_cta.ensure((size_t)n_cta * kMlpParams * 4)) || (e = ctx->mlp_loss_cta.ensure(n_cta * 4)) ||
@@ -1706,7 +1717,8 @@ int sddm_mlp_grad(sddm_ctx *ctx, int n, const float *X, const float *Y, const fl
                   float *loss) {
     if (!ctx || n <= 0 || n > (1 << 20) || !X || !Y || !params || !grad || !loss)
         return fail(SDDM_ERR_INVALID_ARG, "sddm_mlp_grad: bad arguments");
-    cudaError_t e = cudaSetDevice(ctx->device);
+    cudaError_t e = mlp_device(ctx);
+    if (e != cudaSuccess) return cuda_fail(e, "sddm_mlp_grad: device");
     cudaStream_t s = ctx->stream;
     const int n_cta = (n + kMlpRowsPerCta - 1) / kMlpRowsPerCta;
     if ((e = ctx->mlp_grad_cta.ensure((size_t)n_cta * kMlpParams * 4)) || (e = ctx->mlp_loss_cta.ensure(n_cta * 4)))
@@ -1769,8 +1781,7 @@ int sddm_glass_eval(sddm_ctx *ctx, uint32_t mat, int n, const float *cos_theta, 
         a.fallbacks = nullptr;
         a.test_timeout = (ctx->profile & SDDM_PROFILE_TEST_MLP_TIMEOUT) != 0;
         int *const derr = static_cast<int *>(ctx->h_table.p);   // page-locked; no render is under way
-        cudaError_t e = cudaSetDevice(ctx->device);
-        if (e == cudaSuccess && ctx->stage_busy) e = cudaStreamSynchronize(ctx->stream);
+        cudaError_t e = ctx->stage_busy ? cudaStreamSynchronize(ctx->stream) : cudaSuccess;
         ctx->stage_busy = false;
         // the batch counts lie behind the error word, the two lists in scratch kept for the next call
         const size_t n_batch = ((size_t)n + 31) / 32;

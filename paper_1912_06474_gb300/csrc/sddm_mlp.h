@@ -45,6 +45,10 @@ struct MlpRows {
     uint32_t list_cap;                // at least the call's batches
     int test_timeout;                 // 1: CTA 0 issues no layer-1 MMA and waits 2^10 tries (failure-path test)
 };
+// The attributes the network and training kernels are launched with, set on the
+// current device, where they hold (a device keeps its own). Every context calls it
+// before its first such launch.
+cudaError_t mlp_prepare_device();
 // raw: the network over every row (tensor cores). Otherwise the network over
 // one probe row per batch, then over the batches that passed, and the exact slab
 // over the others: three kernels on `stream`. With ev0 / ev1 given, they are
