@@ -486,13 +486,13 @@ int ddm_photon_pass(const DDMPhotonRun &run, DDMBuffers &buf, cudaStream_t s) {
         }
         a.b = b;
         const size_t shade_smem = sizeof(int) * (size_t)((nb + 3) & ~3) + photon_stage_bytes(L);
+        // the same limit from every caller: contexts on several threads cannot lower one another's
+        constexpr int kMostSmem = (int)(sizeof(int) * (size_t)kMaxBins + photon_stage_bytes(kStageMaxL));
         if (run.sc.mat_nfilm) {
-            PM_CHECK(cudaFuncSetAttribute(k_photon_shade<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)shade_smem));
+            PM_CHECK(cudaFuncSetAttribute(k_photon_shade<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostSmem));
             k_photon_shade<true><<<path_blocks, 256, shade_smem, s>>>(a, pp);
         } else {
-            PM_CHECK(cudaFuncSetAttribute(k_photon_shade<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)shade_smem));
+            PM_CHECK(cudaFuncSetAttribute(k_photon_shade<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostSmem));
             k_photon_shade<false><<<path_blocks, 256, shade_smem, s>>>(a, pp);
         }
         PM_CHECK(cudaGetLastError());

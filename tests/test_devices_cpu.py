@@ -61,7 +61,7 @@ if what == "renders":
         render(sc, ctx, method="megakernel")
         render(sc, ctx, method="ddm")
 elif what == "photons":
-    for sc, ctx in both + (context(0, 8), first):
+    for sc, ctx in both + (context(0, 64), context(0, 8), first):
         photons(sc, ctx)
         photons(sc, ctx, "megakernel")
 elif what == "weights":
@@ -107,7 +107,7 @@ def fake_library(tmp_path_factory):
     return lib
 
 
-@pytest.mark.parametrize("what", ["renders", "weights", "training"])
+@pytest.mark.parametrize("what", ["renders", "photons", "weights", "training"])
 def test_second_device(fake_library, what):
     r = subprocess.run([sys.executable, "-c", CALLS, fake_library, what], cwd=ROOT, capture_output=True, text=True,
                        timeout=300)
