@@ -520,8 +520,9 @@ __global__ void __launch_bounds__(256) k_glass_gather(KArgs a) {
 // 16-byte accesses of neighbouring lanes, and lanes side by side mostly share a
 // record's branch; the rows of a pass are all fetched at once (cp.async) before
 // the first is used, and a chunk's XYZ takes its row chunk's place in shared
-// memory. (3) A lane per path adds its chunks in bin order with compensation and
-// updates the path's accumulator.
+// memory. (3) A lane per path and colour component adds the path's chunks in bin
+// order and updates its accumulator. Every addition, within a chunk (chunk_xyz) and
+// between chunks, keeps what it rounds off.
 // The bound is the row traffic (2 x 176 B per live path at L = 41). A row is not
 // read before a weight has been applied to it (up to the second vertex the
 // throughput is 1) nor written once the path has ended.
@@ -544,23 +545,16 @@ static_assert(sizeof(SpecRec) == 64, "four 16-byte loads");
 constexpr int kSrResolve = 1, kSrEmit = 2, kSrLoad = 4, kSrStore = 8, kSrRow = 16, kSrConductor = 32, kSrGlass = 64,
               kSrDirect = 128;   // a glass evaluation the query list had no room for
 constexpr int kSpecThreads = 128;
-constexpr int kSpecItems = 192;  // chunks a warp works through between two sums (at least 3 records at L = 256)
-
-struct Float4 {
-    float v[4];
-};
-__device__ __forceinline__ Float4 ld4(const float4 *p) {
-    const float4 x = __ldg(p);
-    return Float4{{x.x, x.y, x.z, x.w}};
-}
+constexpr int kSpecItems = 128;  // chunks a warp works through between two sums (two records of 256 bins; 24 bytes each)
 
 // One chunk of a record: the XYZ it adds (bins past L have a zero colour
-// matching function), the row's four bins updated. DIRECT also evaluates the
+// matching function) to *s and *c, the row's four bins updated. DIRECT also evaluates the
 // glass that has no query; that variant stays out of line: with it in the loop
 // every warp runs, instruction cache misses cost three times the pass (518
 // against 163 us, hotel room 256 x 256 x 16 spp, bounce 3).
 template <bool FILMS, bool DIRECT>
-__device__ __forceinline__ float3 spec_chunk(const KArgs &a, const SpecRec &rec, int ch, const float4 &tin) {
+__device__ __forceinline__ void spec_chunk(const KArgs &a, const SpecRec &rec, int ch, const float4 &tin, float4 *s,
+                                           float2 *c) {
     const DevScene &sc = a.sc;
     const PathState &ps = a.ps;
     const int L = sc.L, n_chunk = sc.Lp >> 2, xf = rec.flags, q = rec.q;
@@ -623,26 +617,19 @@ __device__ __forceinline__ float3 spec_chunk(const KArgs &a, const SpecRec &rec,
 #pragma unroll
         for (int u = 0; u < 4; ++u) e.v[u] = t.v[u] * le.v[u];
     }
-    float3 s = make_float3(0.f, 0.f, 0.f);
     if (xf & (kSrResolve | kSrEmit)) {
-        const float4 *const w = tab + 2 * sc.n_mat * n_chunk;
-        const Float4 wx = ld4(w), wy = ld4(w + n_chunk), wz = ld4(w + 2 * n_chunk);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            s.x = fmaf(e.v[u], wx.v[u], s.x);
-            s.y = fmaf(e.v[u], wy.v[u], s.y);
-            s.z = fmaf(e.v[u], wz.v[u], s.z);
-        }
+        const ChunkXyz v = chunk_xyz(e, tab + 2 * sc.n_mat * n_chunk, n_chunk);
+        *s = v.s;
+        *c = v.c;
     }
     if (xf & kSrStore)
         reinterpret_cast<float4 *>(ps.T)[(size_t)q * n_chunk + ch] = make_float4(t.v[0], t.v[1], t.v[2], t.v[3]);
-    return s;
 }
 
 // The chunks of a warp's records, dealt to its lanes.
 template <bool FILMS, bool DIRECT>
-__device__ __forceinline__ void spec_items(const KArgs &a, const SpecRec *rec, float4 *part, int n_item, int n_chunk,
-                                           unsigned inv_chunk) {
+__device__ __forceinline__ void spec_items(const KArgs &a, const SpecRec *rec, float4 *part, float2 *lost, int n_item,
+                                           int n_chunk, unsigned inv_chunk) {
     const int lane = threadIdx.x & 31;
     for (int i = lane; i < n_item; i += 32) {
         const int j = (int)((unsigned)i * inv_chunk >> 16);
@@ -655,22 +642,14 @@ __device__ __forceinline__ void spec_items(const KArgs &a, const SpecRec *rec, f
 #pragma unroll 1
     for (int i = lane; i < n_item; i += 32) {
         const int j = (int)((unsigned)i * inv_chunk >> 16);
-        const float3 s = spec_chunk<FILMS, DIRECT>(a, rec[j], i - j * n_chunk, part[i]);
-        part[i] = make_float4(s.x, s.y, s.z, 0.0f);
+        spec_chunk<FILMS, DIRECT>(a, rec[j], i - j * n_chunk, part[i], part + i, lost + i);
     }
-}
-// k + (s2 - c2), the rounding error of the addition kept in k.c (true sum k.s - k.c).
-__device__ __forceinline__ void two_sum(Kahan &k, float s2, float c2) {
-    const float t = k.s + s2, b = t - k.s;
-    const float e = (k.s - (t - b)) + (s2 - b);
-    k.c = (k.c + c2) - e;
-    k.s = t;
 }
 
 template <bool FILMS>
-static __device__ __noinline__ void spec_items_direct(const KArgs &a, const SpecRec *rec, float4 *part, int n_item,
-                                                      int n_chunk, unsigned inv_chunk) {
-    spec_items<FILMS, true>(a, rec, part, n_item, n_chunk, inv_chunk);
+static __device__ __noinline__ void spec_items_direct(const KArgs &a, const SpecRec *rec, float4 *part, float2 *lost,
+                                                      int n_item, int n_chunk, unsigned inv_chunk) {
+    spec_items<FILMS, true>(a, rec, part, lost, n_item, n_chunk, inv_chunk);
 }
 
 #ifndef SDDM_SHS_MINB
@@ -680,6 +659,7 @@ template <bool FILMS>
 __global__ void __launch_bounds__(kSpecThreads, SDDM_SHS_MINB) k_shade_spectral(const __grid_constant__ KArgs a) {
     __shared__ __align__(16) SpecRec s_rec[kSpecThreads];
     __shared__ __align__(16) float4 s_part[kSpecThreads / 32][kSpecItems];
+    __shared__ __align__(8) float2 s_lost[kSpecThreads / 32][kSpecItems];
     const int64_t np = a.ps.np;
     const DevScene &sc = a.sc;
     const int n_chunk = sc.Lp >> 2, M = sc.n_mat;
@@ -689,7 +669,8 @@ __global__ void __launch_bounds__(kSpecThreads, SDDM_SHS_MINB) k_shade_spectral(
     const int lane = threadIdx.x & 31;
     SpecRec *const rec = s_rec + (threadIdx.x & ~31);
     float4 *const part = s_part[threadIdx.x >> 5];
-    const int per_pass = min(32, kSpecItems / n_chunk);        // records summed at a time
+    float2 *const lost = s_lost[threadIdx.x >> 5];
+    const int per_pass = records_per_pass(kSpecItems, n_chunk);
     const unsigned inv_chunk = 65536u / (unsigned)n_chunk + 1u;   // i / n_chunk = i inv >> 16 for i < kSpecItems
     unsigned long long n_glass = 0;
     const PathState &ps = a.ps;
@@ -781,34 +762,21 @@ __global__ void __launch_bounds__(kSpecThreads, SDDM_SHS_MINB) k_shade_spectral(
         for (int r0 = 0; r0 < n_rec; r0 += per_pass) {
             const int nr = min(per_pass, n_rec - r0), n_item = nr * n_chunk;
             if (!any_direct)
-                spec_items<FILMS, false>(a, rec + r0, part, n_item, n_chunk, inv_chunk);
+                spec_items<FILMS, false>(a, rec + r0, part, lost, n_item, n_chunk, inv_chunk);
             else
-                spec_items_direct<FILMS>(a, rec + r0, part, n_item, n_chunk, inv_chunk);
+                spec_items_direct<FILMS>(a, rec + r0, part, lost, n_item, n_chunk, inv_chunk);
             __syncwarp();
-            const int j = mine - r0;
-            if ((me.flags & (kSrResolve | kSrEmit)) && j >= 0 && j < nr) {
-                Kahan3 sum, acc;
-                const float4 *p = part + j * n_chunk;
-                for (int c = 0; c < n_chunk; ++c) {
-                    const float4 v = p[c];
-                    sum.add(v.x, v.y, v.z);
-                }
-                acc.x.s = ps.acc[0 * np + q];
-                acc.y.s = ps.acc[1 * np + q];
-                acc.z.s = ps.acc[2 * np + q];
-                acc.x.c = ps.acc[3 * np + q];
-                acc.y.c = ps.acc[4 * np + q];
-                acc.z.c = ps.acc[5 * np + q];
-                acc.x.c += sum.x.c;   // what the chunk sums lost goes on to the path's sum
-                acc.y.c += sum.y.c;
-                acc.z.c += sum.z.c;
-                acc.add(sum.x.s, sum.y.s, sum.z.s);
-                ps.acc[0 * np + q] = acc.x.s;
-                ps.acc[1 * np + q] = acc.y.s;
-                ps.acc[2 * np + q] = acc.z.s;
-                ps.acc[3 * np + q] = acc.x.c;
-                ps.acc[4 * np + q] = acc.y.c;
-                ps.acc[5 * np + q] = acc.z.c;
+            for (int i = lane; i < 3 * nr; i += 32) {
+                const int j = i / 3, k = i - 3 * j;
+                if (!(rec[r0 + j].flags & (kSrResolve | kSrEmit))) continue;
+                const Kahan sum = sum_chunks<4>(part + j * n_chunk, lost + j * n_chunk, n_chunk, k);
+                float *const acc = ps.acc + k * np + rec[r0 + j].q;
+                Kahan to;
+                to.s = acc[0];
+                to.c = acc[3 * np] + sum.c;   // what the chunk sums lost goes on to the path's sum
+                to.add(sum.s);
+                acc[0] = to.s;
+                acc[3 * np] = to.c;
             }
             __syncwarp();   // the next pass rewrites the partial sums, the next trip the records
         }

@@ -260,7 +260,7 @@ constexpr int kMrEmit = 1, kMrResolve = 2, kMrDiffuse = 4, kMrConductor = 8, kMr
 constexpr int kMegaBatch = SDDM_MEGA_BATCH;
 constexpr int kMegaMinLanes = 2;   // lanes of a warp that take paths, at least
 constexpr int kMegaWarps = 2;      // warps of a block: small images spread over more SMs
-constexpr int kMegaItems = 96;     // chunks worked through between two sums
+constexpr int kMegaItems = 64;     // chunks worked through between two sums (a record of 256 bins)
 static_assert(4 * kMegaItems >= kBranchTerms, "the two share their place");
 // What a lane needs only when the warp shades: the path's sums, and the
 // continuation ray while its vertex's shadow ray is under way.
@@ -270,39 +270,32 @@ struct MegaWarp {
     int xprim[32], xobj[32];
     MegaRec rec[32];
     float4 part[kMegaItems];   // also the glass branch's terms
+    float2 lost[kMegaItems];
     int order[32];
 };
 __host__ __device__ constexpr size_t mega_warp_bytes(int Lp) { return sizeof(MegaWarp) + sizeof(float) * 32 * (size_t)Lp; }
 
-struct Quad {
-    float v[4];
-};
-__device__ __forceinline__ Quad ld_quad(const float4 *p) {
-    const float4 x = __ldg(p);
-    return Quad{{x.x, x.y, x.z, x.w}};
-}
-
-// One chunk of a lane's record: the XYZ it adds; its four throughput bins updated.
+// One chunk of a lane's record: the XYZ it adds, to *s and *c; its four throughput bins updated.
 template <bool FILMS>
-__device__ __forceinline__ float3 mega_chunk(const MegaArgs &a, const MegaRec &m, float4 *row, int ch) {
+__device__ __forceinline__ void mega_chunk(const MegaArgs &a, const MegaRec &m, float4 *row, int ch, float4 *s, float2 *c) {
     const DevScene &sc = a.sc;
     const int n_chunk = sc.Lp >> 2, xf = m.flags;
     const float4 *const tab = reinterpret_cast<const float4 *>(sc.tab) + ch;
-    Quad t{{1.f, 1.f, 1.f, 1.f}}, e{{0.f, 0.f, 0.f, 0.f}};
+    Float4 t{{1.f, 1.f, 1.f, 1.f}}, e{{0.f, 0.f, 0.f, 0.f}};
     if (!(xf & kMrFirst)) {
         const float4 v = row[ch];
-        t = Quad{{v.x, v.y, v.z, v.w}};
+        t = Float4{{v.x, v.y, v.z, v.w}};
     }
     if (xf & kMrEmit) {
-        const Quad le = ld_quad(tab + m.r_emit * n_chunk);
+        const Float4 le = ld4(tab + m.r_emit * n_chunk);
 #pragma unroll
         for (int u = 0; u < 4; ++u) e.v[u] = t.v[u] * le.v[u];
     }
     if (xf & (kMrResolve | kMrDiffuse)) {
-        const Quad rho = ld_quad(tab + m.r_rho * n_chunk);
+        const Float4 rho = ld4(tab + m.r_rho * n_chunk);
         if (xf & kMrResolve) {
-            const Quad le = ld_quad(tab + m.r_le * n_chunk);
-            Quad tr{{1.f, 1.f, 1.f, 1.f}};
+            const Float4 le = ld4(tab + m.r_le * n_chunk);
+            Float4 tr{{1.f, 1.f, 1.f, 1.f}};
 #pragma unroll 1
             for (int k = 0; k < m.ncr; ++k) {
                 const int cm = m.cmat[k];
@@ -324,7 +317,7 @@ __device__ __forceinline__ float3 mega_chunk(const MegaArgs &a, const MegaRec &m
         }
     }
     if (xf & kMrConductor) {
-        const Quad n = ld_quad(tab + m.r_w * n_chunk), k = ld_quad(tab + m.r_w2 * n_chunk);
+        const Float4 n = ld4(tab + m.r_w * n_chunk), k = ld4(tab + m.r_w2 * n_chunk);
 #pragma unroll
         for (int u = 0; u < 4; ++u) t.v[u] *= conductor_F(m.pcos, n.v[u], k.v[u]);
     } else if (xf & kMrGlass) {
@@ -340,18 +333,11 @@ __device__ __forceinline__ float3 mega_chunk(const MegaArgs &a, const MegaRec &m
         }
     }
     if (xf & (kMrDiffuse | kMrConductor | kMrGlass)) row[ch] = make_float4(t.v[0], t.v[1], t.v[2], t.v[3]);
-    float3 s = make_float3(0.f, 0.f, 0.f);
     if (xf & (kMrEmit | kMrResolve)) {
-        const float4 *const w = tab + 2 * sc.n_mat * n_chunk;
-        const Quad wx = ld_quad(w), wy = ld_quad(w + n_chunk), wz = ld_quad(w + 2 * n_chunk);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            s.x = fmaf(e.v[u], wx.v[u], s.x);
-            s.y = fmaf(e.v[u], wy.v[u], s.y);
-            s.z = fmaf(e.v[u], wz.v[u], s.z);
-        }
+        const ChunkXyz v = chunk_xyz(e, tab + 2 * sc.n_mat * n_chunk, n_chunk);
+        *s = v.s;
+        *c = v.c;
     }
-    return s;
 }
 
 template <bool COUNT, bool FILMS>
@@ -366,7 +352,7 @@ __global__ void __launch_bounds__(32 * kMegaWarps, SDDM_MEGA_MIN_BLOCKS) k_megak
     unsigned char *const mem = s_mega + mega_warp_bytes(Lp) * (threadIdx.x >> 5);
     float4 *const rows = reinterpret_cast<float4 *>(mem);
     MegaWarp &w = *reinterpret_cast<MegaWarp *>(mem + sizeof(float) * 32 * (size_t)Lp);
-    const int per_pass = kMegaItems / n_chunk;                    // records summed at a time (n_chunk <= 64)
+    const int per_pass = records_per_pass(kMegaItems, n_chunk);   // n_chunk <= 64
     const unsigned inv_chunk = 65536u / (unsigned)n_chunk + 1u;   // i / n_chunk = i inv >> 16 for i < kMegaItems
 
     enum { kIdle, kExt, kShadow };
@@ -561,32 +547,20 @@ __global__ void __launch_bounds__(32 * kMegaWarps, SDDM_MEGA_MIN_BLOCKS) k_megak
 #pragma unroll 1
                 for (int i = lane; i < n_item; i += 32) {
                     const int jr = (int)((unsigned)i * inv_chunk >> 16), from = w.order[r0 + jr];
-                    const float3 s = mega_chunk<FILMS>(a, w.rec[from], rows + from * n_chunk, i - jr * n_chunk);
-                    w.part[i] = make_float4(s.x, s.y, s.z, 0.0f);
+                    mega_chunk<FILMS>(a, w.rec[from], rows + from * n_chunk, i - jr * n_chunk, w.part + i, w.lost + i);
                 }
                 __syncwarp();
-                const int jr = mine - r0;
-                if ((flags & (kMrEmit | kMrResolve)) && jr >= 0 && jr < nr) {
-                    Kahan3 sum, acc;
-                    const float4 *pp = w.part + jr * n_chunk;
 #pragma unroll 1
-                    for (int c = 0; c < n_chunk; ++c) {
-                        const float4 v = pp[c];
-                        sum.add(v.x, v.y, v.z);
-                    }
-                    acc.x.s = w.acc[0][lane];
-                    acc.y.s = w.acc[1][lane];
-                    acc.z.s = w.acc[2][lane];
-                    acc.x.c = w.acc[3][lane] + sum.x.c;   // what the chunk sums lost goes on to the path's sum
-                    acc.y.c = w.acc[4][lane] + sum.y.c;
-                    acc.z.c = w.acc[5][lane] + sum.z.c;
-                    acc.add(sum.x.s, sum.y.s, sum.z.s);
-                    w.acc[0][lane] = acc.x.s;
-                    w.acc[1][lane] = acc.y.s;
-                    w.acc[2][lane] = acc.z.s;
-                    w.acc[3][lane] = acc.x.c;
-                    w.acc[4][lane] = acc.y.c;
-                    w.acc[5][lane] = acc.z.c;
+                for (int i = lane; i < 3 * nr; i += 32) {
+                    const int jr = i / 3, k = i - 3 * jr, from = w.order[r0 + jr];
+                    if (!(w.rec[from].flags & (kMrEmit | kMrResolve))) continue;
+                    const Kahan sum = sum_chunks<1>(w.part + jr * n_chunk, w.lost + jr * n_chunk, n_chunk, k);
+                    Kahan to;
+                    to.s = w.acc[k][from];
+                    to.c = w.acc[3 + k][from] + sum.c;   // what the chunk sums lost goes on to the path's sum
+                    to.add(sum.s);
+                    w.acc[k][from] = to.s;
+                    w.acc[3 + k][from] = to.c;
                 }
                 __syncwarp();
             }
