@@ -670,7 +670,7 @@ __global__ void __launch_bounds__(kSpecThreads, SDDM_SHS_MINB) k_shade_spectral(
     SpecRec *const rec = s_rec + (threadIdx.x & ~31);
     float4 *const part = s_part[threadIdx.x >> 5];
     float2 *const lost = s_lost[threadIdx.x >> 5];
-    const int per_pass = records_per_pass(kSpecItems, n_chunk);
+    const int per_pass = min(32, kSpecItems / n_chunk);        // records summed at a time
     const unsigned inv_chunk = 65536u / (unsigned)n_chunk + 1u;   // i / n_chunk = i inv >> 16 for i < kSpecItems
     unsigned long long n_glass = 0;
     const PathState &ps = a.ps;

@@ -812,7 +812,8 @@ __device__ __forceinline__ Float4 ld4(const float4 *p) {
 // square error against 64 bits, 8 / 16 / 41 / 81 bins, of sums that differ in this alone:
 // 4.28 / 3.62 / 3.18 / 2.70e-8 with plain sums inside the chunk and compensated ones
 // between chunks, 3.11 / 2.58 / 2.20 / 2.17e-8 so (3.09 / 2.57 / 2.23 / 2.14e-8 is what
-// one rounding of products and result makes). It costs 1 to 2 % of a render.
+// one rounding of products and result makes). It costs 1 % of a hotel room render and 2 to
+// 9 % of a tiny room's, whose time is mostly this pass.
 struct ChunkXyz {
     float4 s;    // sums of x, y, z; what x lost (true sum s - c)
     float2 c;    // what y and z lost
@@ -843,12 +844,6 @@ __device__ __forceinline__ Kahan sum_chunks(const float4 *s, const float2 *c, in
 #pragma unroll UNROLL
     for (int i = 0; i < n; ++i) two_sum(sum, ps[4 * i], pc[step * i]);
     return sum;
-}
-// Records summed in one pass when `items` chunks fit: as many as fill the last
-// round of lanes, three to a record.
-__host__ __device__ __forceinline__ int records_per_pass(int items, int n_chunk) {
-    const int n = items / n_chunk < 32 ? items / n_chunk : 32, rounds = 3 * n / 32;
-    return rounds > 0 ? 32 * rounds / 3 : n;
 }
 
 // ------------------------------------------------------------------ camera

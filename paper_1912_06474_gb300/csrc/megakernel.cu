@@ -352,7 +352,7 @@ __global__ void __launch_bounds__(32 * kMegaWarps, SDDM_MEGA_MIN_BLOCKS) k_megak
     unsigned char *const mem = s_mega + mega_warp_bytes(Lp) * (threadIdx.x >> 5);
     float4 *const rows = reinterpret_cast<float4 *>(mem);
     MegaWarp &w = *reinterpret_cast<MegaWarp *>(mem + sizeof(float) * 32 * (size_t)Lp);
-    const int per_pass = records_per_pass(kMegaItems, n_chunk);   // n_chunk <= 64
+    const int per_pass = min(32, kMegaItems / n_chunk);           // records summed at a time (n_chunk <= 64)
     const unsigned inv_chunk = 65536u / (unsigned)n_chunk + 1u;   // i / n_chunk = i inv >> 16 for i < kMegaItems
 
     enum { kIdle, kExt, kShadow };
