@@ -16,6 +16,8 @@
 // of the photons within radius r that arrived on the visible side, over pi r^2.
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "device_common.cuh"
 #include "photon.cuh"
 
@@ -229,7 +231,7 @@ __global__ void __launch_bounds__(128) k_megakernel_pm(MegaArgs a) {
 //  * the spectral part of shading is done by the whole warp: each waiting lane
 //    leaves a record (emission, resolved shadow ray, weight), the rows of bins
 //    are dealt out to the lanes in chunks of four, as in the DDM's spectral pass,
-//    with the throughput rows in shared memory, a row per lane.
+//    with a throughput row per lane, in shared memory while there are few bins.
 // Hotel room, 512 x 512 x 4 spp, 41 bins: 10.2 -> 6.1 ms; tiny room, 400 x 400 x 6
 // spp, depth 6: 4.4 -> 3.4 ms; with a coated pane, 200 x 200 x 3 spp: 2.1 -> 0.96.
 // The loop holds all that a path meets, some 4000 instructions, and the
@@ -273,7 +275,20 @@ struct MegaWarp {
     float2 lost[kMegaItems];
     int order[32];
 };
+// Shared memory of a warp whose throughput rows are there, too.
 __host__ __device__ constexpr size_t mega_warp_bytes(int Lp) { return sizeof(MegaWarp) + sizeof(float) * 32 * (size_t)Lp; }
+// Padded bins up to which the rows lie in shared memory. Above them they lie in global
+// memory (a.rows): a warp's rows push eight blocks out of an SM from some 56 bins on (at
+// 256 there are two), and take the L1 from the nodes and stacks before that. Rows in
+// shared / global memory, hotel room 512 x 512 x 4 spp at 41 / 48 / 64 / 81 / 128 / 256 bins:
+// 6.03 / 6.36 / 7.12 / 8.40 / 10.1 / 24.0 against 5.95 / 5.88 / 5.93 / 6.32 / 6.41 / 7.74 ms;
+// tiny room, 400 x 400 x 4 spp: 2.23 / 2.25 / 2.48 / 3.00 / 4.03 / 17.3 against 2.24 / 2.25 /
+// 2.35 / 2.75 / 3.14 / 5.93, coated, 16 bins: 0.85 against 0.89. (A thread per path with its
+// row in local memory, before this kernel: 21.5 and 12.2 ms at 256 bins.)
+constexpr int kMegaRowBins = 44;
+size_t mega_row_bytes(int sm_count, int Lp) {
+    return Lp > kMegaRowBins ? (size_t)sm_count * SDDM_MEGA_MIN_BLOCKS * kMegaWarps * 32 * Lp * sizeof(float) : 0;
+}
 
 // One chunk of a lane's record: the XYZ it adds, to *s and *c; its four throughput bins updated.
 template <bool FILMS>
@@ -340,7 +355,7 @@ __device__ __forceinline__ void mega_chunk(const MegaArgs &a, const MegaRec &m, 
     }
 }
 
-template <bool COUNT, bool FILMS>
+template <bool COUNT, bool FILMS, bool ROWS>
 __global__ void __launch_bounds__(32 * kMegaWarps, SDDM_MEGA_MIN_BLOCKS) k_megakernel(const __grid_constant__ MegaArgs a,
                                                                                            int lanes, int batch) {
     extern __shared__ __align__(16) unsigned char s_mega[];
@@ -349,9 +364,10 @@ __global__ void __launch_bounds__(32 * kMegaWarps, SDDM_MEGA_MIN_BLOCKS) k_megak
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const unsigned lt_mask = (1u << lane) - 1u;
-    unsigned char *const mem = s_mega + mega_warp_bytes(Lp) * (threadIdx.x >> 5);
-    float4 *const rows = reinterpret_cast<float4 *>(mem);
-    MegaWarp &w = *reinterpret_cast<MegaWarp *>(mem + sizeof(float) * 32 * (size_t)Lp);
+    const int warp = threadIdx.x >> 5;
+    unsigned char *const mem = s_mega + (ROWS ? sizeof(MegaWarp) : mega_warp_bytes(Lp)) * warp;
+    float4 *const rows = ROWS ? a.rows + ((size_t)blockIdx.x * kMegaWarps + warp) * 32 * n_chunk : reinterpret_cast<float4 *>(mem);
+    MegaWarp &w = *reinterpret_cast<MegaWarp *>(ROWS ? mem : mem + sizeof(float) * 32 * (size_t)Lp);
     const int per_pass = min(32, kMegaItems / n_chunk);           // records summed at a time (n_chunk <= 64)
     const unsigned inv_chunk = 65536u / (unsigned)n_chunk + 1u;   // i / n_chunk = i inv >> 16 for i < kMegaItems
 
@@ -652,12 +668,12 @@ static void launch_pm(const MegaArgs &a, cudaStream_t stream) {
     }
 }
 
-template <bool COUNT, bool FILMS>
+template <bool COUNT, bool FILMS, bool ROWS>
 static cudaError_t launch_plain(const MegaArgs &a, cudaStream_t stream) {
-    const size_t smem = mega_warp_bytes(a.sc.Lp) * kMegaWarps;
+    const size_t smem = (ROWS ? sizeof(MegaWarp) : mega_warp_bytes(a.sc.Lp)) * kMegaWarps;
     cudaError_t e = cudaSuccess;
     if (smem > 48 * 1024)   // more than a block has without asking (over 104 bins); the same for every caller
-        e = cudaFuncSetAttribute(k_megakernel<COUNT, FILMS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(k_megakernel<COUNT, FILMS, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)(mega_warp_bytes(kMaxL) * kMegaWarps));
     if (e == cudaSuccess) e = cudaMemsetAsync(a.cursor, 0, sizeof(unsigned long long), stream);
     if (e != cudaSuccess) return e;
@@ -674,11 +690,12 @@ static cudaError_t launch_plain(const MegaArgs &a, cudaStream_t stream) {
     int64_t most = want;
     if (lanes == 32) {
         int per_sm = 1;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_megakernel<COUNT, FILMS>, 32 * kMegaWarps, smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_megakernel<COUNT, FILMS, ROWS>, 32 * kMegaWarps, smem);
         if (e != cudaSuccess) return e;
+        if (ROWS && per_sm > SDDM_MEGA_MIN_BLOCKS) per_sm = SDDM_MEGA_MIN_BLOCKS;   // as many rows as there are
         most = (int64_t)a.sm_count * (per_sm > 0 ? per_sm : 1);
     }
-    k_megakernel<COUNT, FILMS><<<(unsigned)(want < most ? want : most), 32 * kMegaWarps, smem, stream>>>(a, lanes, batch);
+    k_megakernel<COUNT, FILMS, ROWS><<<(unsigned)(want < most ? want : most), 32 * kMegaWarps, smem, stream>>>(a, lanes, batch);
     return cudaGetLastError();
 }
 
@@ -689,8 +706,13 @@ cudaError_t launch_megakernel(const MegaArgs &a, cudaStream_t stream) {
         films ? launch_pm<true>(a, stream) : launch_pm<false>(a, stream);
         return cudaGetLastError();
     }
-    if (a.count_traversal) return films ? launch_plain<true, true>(a, stream) : launch_plain<true, false>(a, stream);
-    return films ? launch_plain<false, true>(a, stream) : launch_plain<false, false>(a, stream);
+    const bool rows = a.rows && a.sc.Lp > kMegaRowBins;
+    auto launch = [&](auto count) {
+        constexpr bool C = decltype(count)::value;
+        if (rows) return films ? launch_plain<C, true, true>(a, stream) : launch_plain<C, false, true>(a, stream);
+        return films ? launch_plain<C, true, false>(a, stream) : launch_plain<C, false, false>(a, stream);
+    };
+    return a.count_traversal ? launch(std::true_type()) : launch(std::false_type());
 }
 
 }  // namespace sddm

@@ -147,6 +147,7 @@ extern "C" int sddm_render_noalloc(sddm_ctx *ctx, const sddm_render_desc *d, sdd
     a.error_flag = reinterpret_cast<int *>(scratch + kOffErr);
     a.cursor = reinterpret_cast<unsigned long long *>(scratch + kOffCursor);
     a.sm_count = v.sm_count;
+    a.rows = v.mega_rows;
     a.count_traversal = 0;
     if ((e = launch_megakernel(a, s)) != cudaSuccess) return cuda_fail(e, "sddm_render_noalloc: megakernel");
     ReduceArgs ra;

@@ -188,6 +188,7 @@ struct sddm_ctx {
     PinnedBuf h_table;   // its host side; stage_busy: a copy from it may still be under way
     bool stage_busy = false;
     DevBuf d_samples, d_first, d_err;
+    DevBuf d_mega_rows;  // throughput rows of the plain method at many bins (with the build)
     DevBuf d_host_out;   // device side of sddm_render_host's outputs
     DDMBuffers ddm_buf;
     // photon map (sddm_render_photon_map): slots, grid, and the view the
@@ -662,6 +663,13 @@ int sddm_build(sddm_ctx *ctx, const sddm_build_opts *opts) {
     d.g_nodes = ctx->d_gnodes.as<float4>();
     d.g_tris = ctx->d_gtris.as<float4>();
 
+    // the plain method's throughput rows; where there is no memory for them it keeps them on chip
+    const size_t row_bytes = mega_row_bytes(ctx->sm_count, Lp);
+    if (row_bytes == 0)
+        ctx->d_mega_rows.release();
+    else if (ctx->d_mega_rows.ensure(row_bytes) != cudaSuccess)
+        cudaGetLastError();
+
     DDMScene &g = ctx->ddm;
     for (int a = 0; a < 3; ++a) {
         g.dims[a] = o.grid[a];
@@ -812,6 +820,7 @@ int ctx_view(sddm_ctx *ctx, CtxView *v) {
     v->ev0 = ctx->ev0;
     v->ev1 = ctx->ev1;
     v->sm_count = ctx->sm_count;
+    v->mega_rows = ctx->d_mega_rows.as<float4>();
     return SDDM_OK;
 }
 int check_render_desc(const sddm_ctx *ctx, const sddm_render_desc *d, int n) { return validate_desc(ctx, d, n); }
@@ -959,6 +968,7 @@ int sddm_render(sddm_ctx *ctx, const sddm_render_desc *d, int n, sddm_stats *st)
                 a.error_flag = d_err;
                 a.cursor = a.counters + kNumCounters - 1;
                 a.sm_count = ctx->sm_count;
+                a.rows = ctx->d_mega_rows.as<float4>();
                 a.count_traversal = count_trav;
                 a.pm = ctx->pm_view;
                 a.pmc = ctx->pmc_view;

@@ -138,6 +138,7 @@ struct CtxView {
     int n_mat;
     cudaEvent_t ev0, ev1;
     int sm_count;
+    float4 *mega_rows;
 };
 int ctx_view(sddm_ctx *ctx, CtxView *v);
 int check_render_desc(const sddm_ctx *ctx, const sddm_render_desc *d, int n);
@@ -171,6 +172,7 @@ struct MegaArgs {
     unsigned long long *counters;      // [16]: ext, shadow, glass, crossings, fallbacks, nodes, tris, visits,
                                        // surrogate batches, spare
     int *error_flag;
+    float4 *rows = nullptr;            // throughput rows of the lanes, mega_row_bytes (NULL: in shared memory)
     unsigned long long *cursor;        // next path to hand to a lane (set to 0 by the launch)
     int sm_count;
     int count_traversal;
@@ -178,6 +180,8 @@ struct MegaArgs {
     PhotonGridView pmc = {};           // caustic map gathered there too (pmc.on)
 };
 cudaError_t launch_megakernel(const MegaArgs &a, cudaStream_t stream);
+// Global memory for the plain method's throughput rows at Lp padded bins (0: in shared memory).
+size_t mega_row_bytes(int sm_count, int Lp);
 
 struct ReduceArgs {
     RenderBatch rb;

@@ -24,6 +24,7 @@ struct Call {
     cudaStream_t stream;
 } g_call;
 long g_launches = 0, g_optin = 0;
+size_t g_most = (size_t)-1;   // larger device allocations fail
 
 bool wrong_device(const void *p) {
     auto it = g_mem.upper_bound(static_cast<const char *>(p));
@@ -49,6 +50,7 @@ cudaError_t alloc(void **p, size_t n) {
 extern "C" {
 long fake_launches() { return g_launches; }
 long fake_optin_launches() { return g_optin; }
+void fake_limit_alloc(size_t bytes) { g_most = bytes; }
 
 void **__cudaRegisterFatBinary(void *) {
     static void *h;
@@ -122,7 +124,7 @@ cudaError_t cudaGetDeviceProperties(cudaDeviceProp *p, int) {
 }
 
 cudaError_t cudaMalloc(void **p, size_t n) {
-    const cudaError_t e = alloc(p, n);
+    const cudaError_t e = n > g_most ? (g_last = cudaErrorMemoryAllocation) : alloc(p, n);
     if (e == cudaSuccess) g_mem[static_cast<const char *>(*p)] = {n, g_device};
     return e;
 }

@@ -60,6 +60,10 @@ if what == "renders":
     for sc, ctx in both:
         render(sc, ctx, method="megakernel")
         render(sc, ctx, method="ddm")
+    # no memory for the throughput rows of 256 bins: they stay in shared memory
+    lib.fake_limit_alloc(ctypes.c_size_t(1 << 20))
+    for device in (0, 1):
+        render(*context(device, 256), method="megakernel")
 elif what == "photons":
     for sc, ctx in both + (context(0, 64), context(0, 8), first):
         photons(sc, ctx)
