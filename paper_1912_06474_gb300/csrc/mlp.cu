@@ -109,12 +109,7 @@ __device__ __forceinline__ void features(float c, float lam, float s, float alph
 // swizzle: 8-row x 16-byte core matrices, the core matrices of one 8-row group
 // side by side along K (128 B apart, the leading-dimension offset) and the
 // 8-row groups one after the other (the stride offset).
-#ifndef SDDM_MLP_GROUPS
-#define SDDM_MLP_GROUPS 4
-#endif
 constexpr int kTcRows = 128;          // rows per tile = threads of a group = TMEM lanes
-constexpr int kTcGroups = SDDM_MLP_GROUPS;   // tiles a CTA has under way, a group of four warps each
-constexpr int kTcThreads = kTcRows * kTcGroups;
 constexpr int kTcCols = 64;           // TMEM columns: one 128 x 64 FP32 accumulator
 constexpr int kChA = 10;              // A chunks per 8-row group: 8 activations + bias ones + zero
 constexpr int kChB1 = 2;              // layer-1 B: K = 16
@@ -132,10 +127,11 @@ struct __align__(128) TcWeights {
     float b4[2];
 };
 static_assert(sizeof(TcWeights) % 16 == 0, "bulk copies move multiples of 16 bytes");
+template <int GROUPS>   // tiles a CTA has under way, a group of four warps each
 struct __align__(128) TcSmem {
     TcWeights w;
-    __nv_bfloat16 a[kTcGroups][kTcRows * kChA * 8];   // per tile: activations / inputs, K-major core matrices
-    unsigned long long mbar[kTcGroups], mbar_w;       // MMA completion per tile; weights arrived
+    __nv_bfloat16 a[GROUPS][kTcRows * kChA * 8];   // per tile: activations / inputs, K-major core matrices
+    unsigned long long mbar[GROUPS], mbar_w;       // MMA completion per tile; weights arrived
     uint32_t tmem;
 };
 
@@ -530,20 +526,23 @@ __device__ __forceinline__ void list_push(const MlpRows &a, int full, bool is_sh
 // out (the tensor core never signalled completion) the CTA reports error 2 and
 // stops.
 constexpr int kNetAll = 0, kNetProbe = 1, kNetList = 2;
-#ifndef SDDM_MLP_MINB
-#define SDDM_MLP_MINB 2   // resident CTAs per SM
-#endif
+constexpr int kNetGroups = 4;                 // tiles of a CTA in the passes over probes and lists
+constexpr int kNetFewRows = 1 << 22;          // explicit rows up to which a CTA takes one tile
+__host__ __device__ constexpr int net_ctas(int groups) { return groups == 1 ? 5 : 2; }   // resident CTAs per SM
 // Several tiles per CTA share one copy of the weights: four groups and two CTAs
 // are eight tiles on an SM (64 registers a thread, 105 KB per CTA, 512 TMEM
 // columns), which overlap one another's barriers, MMAs and tensor-memory loads
 // with the SiLU's tanh, the bound (192 a row at 16 a cycle and SM: 161 us per 2^22
 // rows). A CTA per tile with a copy each fits five times, of which four ran.
 // Groups x CTAs 1 x 5 / 2 x 3 / 4 x 2: 747 M rows of a facade render in 45.2 / 44.1 /
-// 42.1 ms, 2^24 explicit rows 1007 / 1020 / 983 us.
-template <bool FILMS, int ROWS>
-__global__ void __launch_bounds__(kTcThreads, SDDM_MLP_MINB) k_mlp_net(const __grid_constant__ MlpRows a) {
+// 42.1 ms, 2^24 explicit rows 1007 / 1020 / 983 us. With a few tiles a group the last
+// round weighs more and the smaller CTAs win (a call of 0.5 / 1.05 / 1.3 / 3 / 4.2 M
+// explicit rows: 64 / 90 / 104 / 201 / 275 us with 1 x 5, 63 / 99 / 113 / 210 / 275 with
+// 4 x 2), so the pass over all explicit rows takes 1 x 5 up to 2^22 rows.
+template <bool FILMS, int ROWS, int GROUPS>
+__global__ void __launch_bounds__(kTcRows *GROUPS, net_ctas(GROUPS)) k_mlp_net(const __grid_constant__ MlpRows a) {
     extern __shared__ __align__(128) unsigned char s_mlp[];
-    TcSmem &s = *reinterpret_cast<TcSmem *>(s_mlp);
+    TcSmem<GROUPS> &s = *reinterpret_cast<TcSmem<GROUPS> *>(s_mlp);
     const int tid = threadIdx.x, warp = tid >> 5, group = tid / kTcRows, row = tid % kTcRows;
     BatchShape shape{};
     if (ROWS != kNetAll) shape = batch_shape(a);
@@ -559,7 +558,7 @@ __global__ void __launch_bounds__(kTcThreads, SDDM_MLP_MINB) k_mlp_net(const __g
     const uint32_t mbar = smem_addr(&s.mbar[group]), mbar_w = smem_addr(&s.mbar_w);
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&s.tmem)),
-                     "r"((uint32_t)(kTcCols * kTcGroups))
+                     "r"((uint32_t)(kTcCols * GROUPS))
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -621,7 +620,7 @@ __global__ void __launch_bounds__(kTcThreads, SDDM_MLP_MINB) k_mlp_net(const __g
         return true;
     };
     // a CTA's groups take tiles a grid apart, so that few tiles spread over the SMs
-    for (int64_t tile = blockIdx.x + (int64_t)group * gridDim.x; tile < n_tiles; tile += (int64_t)kTcGroups * gridDim.x) {
+    for (int64_t tile = blockIdx.x + (int64_t)group * gridDim.x; tile < n_tiles; tile += (int64_t)GROUPS * gridDim.x) {
         int64_t r = tile * kTcRows + row;
         RowIn in;
         bool valid;
@@ -711,7 +710,7 @@ __global__ void __launch_bounds__(kTcThreads, SDDM_MLP_MINB) k_mlp_net(const __g
     if (warp == 0) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
-                     "r"((uint32_t)(kTcCols * kTcGroups))
+                     "r"((uint32_t)(kTcCols * GROUPS))
                      : "memory");
     }
 }
@@ -1189,39 +1188,51 @@ static int resident_per_sm(K kernel, int threads, int cap) {
 }
 
 // CTAs per SM: as many as the registers and shared memory allow
-// (__launch_bounds__ asks for SDDM_MLP_MINB). Tensor memory has 512 columns
+// (__launch_bounds__ asks for net_ctas). Tensor memory has 512 columns
 // per SM and each CTA holds kTcCols for each of its tiles, so resident CTAs never
 // wait on one another's allocation.
-static_assert(SDDM_MLP_MINB * kTcCols * kTcGroups <= 512, "tensor-memory columns of the resident tile CTAs");
-template <bool FILMS, int ROWS>
+static_assert(net_ctas(1) * kTcCols <= 512 && net_ctas(kNetGroups) * kTcCols * kNetGroups <= 512,
+              "tensor-memory columns of the resident tile CTAs");
+template <bool FILMS, int ROWS, int GROUPS>
 static cudaError_t prepare_mlp_net() {
-    const cudaError_t e = cudaFuncSetAttribute(k_mlp_net<FILMS, ROWS>, cudaFuncAttributePreferredSharedMemoryCarveout,
+    const cudaError_t e = cudaFuncSetAttribute(k_mlp_net<FILMS, ROWS, GROUPS>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                                (int)cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_mlp_net<FILMS, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TcSmem));
+    return cudaFuncSetAttribute(k_mlp_net<FILMS, ROWS, GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)sizeof(TcSmem<GROUPS>));
+}
+template <bool FILMS>
+static cudaError_t prepare_mlp_nets() {
+    cudaError_t e = prepare_mlp_net<FILMS, kNetAll, 1>();
+    if (e == cudaSuccess) e = prepare_mlp_net<FILMS, kNetAll, kNetGroups>();
+    if (e == cudaSuccess) e = prepare_mlp_net<FILMS, kNetProbe, kNetGroups>();
+    if (e == cudaSuccess) e = prepare_mlp_net<FILMS, kNetList, kNetGroups>();
+    return e;
 }
 cudaError_t mlp_prepare_device() {
     cudaError_t e = cudaFuncSetAttribute(k_mlp_train_tile, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)sizeof(TrainSmem));
-    if (e == cudaSuccess) e = prepare_mlp_net<false, kNetAll>();
-    if (e == cudaSuccess) e = prepare_mlp_net<false, kNetProbe>();
-    if (e == cudaSuccess) e = prepare_mlp_net<false, kNetList>();
-    if (e == cudaSuccess) e = prepare_mlp_net<true, kNetAll>();
-    if (e == cudaSuccess) e = prepare_mlp_net<true, kNetProbe>();
-    if (e == cudaSuccess) e = prepare_mlp_net<true, kNetList>();
+    if (e == cudaSuccess) e = prepare_mlp_nets<false>();
+    if (e == cudaSuccess) e = prepare_mlp_nets<true>();
     return e;
 }
-template <bool FILMS, int ROWS>
+template <bool FILMS, int ROWS, int GROUPS = kNetGroups>
 static cudaError_t launch_mlp_net(const MlpRows &a, int sm_count, cudaStream_t stream) {
-    k_mlp_net<FILMS, ROWS><<<sm_count * SDDM_MLP_MINB, kTcThreads, sizeof(TcSmem), stream>>>(a);
+    k_mlp_net<FILMS, ROWS, GROUPS>
+        <<<sm_count * net_ctas(GROUPS), kTcRows * GROUPS, sizeof(TcSmem<GROUPS>), stream>>>(a);
     return cudaGetLastError();
+}
+template <bool FILMS>
+static cudaError_t launch_mlp_all(const MlpRows &a, int sm_count, cudaStream_t stream) {
+    return a.mode == 0 && a.n > kNetFewRows ? launch_mlp_net<FILMS, kNetAll>(a, sm_count, stream)
+                                            : launch_mlp_net<FILMS, kNetAll, 1>(a, sm_count, stream);
 }
 
 template <bool FILMS>
 static cudaError_t launch_mlp(const MlpRows &a, int sm_count, cudaStream_t stream, cudaEvent_t ev0, cudaEvent_t ev1) {
     cudaError_t e = ev0 ? cudaEventRecord(ev0, stream) : cudaSuccess;
     if (a.raw) {
-        if (e == cudaSuccess) e = launch_mlp_net<FILMS, kNetAll>(a, sm_count, stream);
+        if (e == cudaSuccess) e = launch_mlp_all<FILMS>(a, sm_count, stream);
         if (e == cudaSuccess && ev1) e = cudaEventRecord(ev1, stream);
         return e;
     }
