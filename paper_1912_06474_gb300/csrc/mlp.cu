@@ -715,6 +715,31 @@ __global__ void __launch_bounds__(kTcRows *GROUPS, net_ctas(GROUPS)) k_mlp_net(c
     }
 }
 
+// Explicit rows of a small call (kMlpCheckRows): the network has run over all of them, a
+// warp takes a batch. Its lanes evaluate the exact slab side by side, the probe's lane
+// compares, and the batch keeps the network's rows or takes the exact ones. Launches
+// bound such a call: 2^10 rows 56 us with the probes first, 48 so (51 with a thread per
+// batch that checks and a warp that falls back), coated glass 65, 49 (61).
+template <bool FILMS>
+__global__ void __launch_bounds__(128) k_mlp_check(const __grid_constant__ MlpRows a) {
+    const uint32_t batch = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t r = (int64_t)batch * 32 + (threadIdx.x & 31);
+    const int rows = (int)min((int64_t)32, a.n - (int64_t)batch * 32);
+    if (rows <= 0) return;   // the whole warp
+    RowIn in;
+    const bool valid = row_input(a, r, a.n, in);
+    const uint4 pr = philox4x32_10(make_uint4(batch, 0u, 0u, kSlotProbe), a.probe_key, 0x50524f42u);
+    float2 e = make_float2(0.0f, 0.0f);
+    bool bad = false;
+    if (valid) {
+        e = exact_row<FILMS>(a, in);
+        bad = !row_in_box(a, in);
+        if ((int)(threadIdx.x & 31) == (int)(pr.x % (uint32_t)rows))
+            bad |= fabsf(e.x - a.R[r]) > kMlpProbeTol || fabsf(e.y - a.T[r]) > kMlpProbeTol;
+    }
+    if (__any_sync(kFull, bad) && valid) store_row(a, r, in, e);
+}
+
 // The exact slab over the rows of the failed batches, one thread per row.
 template <bool FILMS>
 __global__ void __launch_bounds__(256) k_mlp_fallback(MlpRows a) {
@@ -1235,6 +1260,13 @@ static cudaError_t launch_mlp(const MlpRows &a, int sm_count, cudaStream_t strea
         if (e == cudaSuccess) e = launch_mlp_all<FILMS>(a, sm_count, stream);
         if (e == cudaSuccess && ev1) e = cudaEventRecord(ev1, stream);
         return e;
+    }
+    if (a.mode == 0 && a.n <= kMlpCheckRows) {
+        if (e == cudaSuccess) e = launch_mlp_all<FILMS>(a, sm_count, stream);
+        if (e == cudaSuccess && ev1) e = cudaEventRecord(ev1, stream);
+        if (e != cudaSuccess) return e;
+        k_mlp_check<FILMS><<<(a.n + 127) / 128, 128, 0, stream>>>(a);
+        return cudaGetLastError();
     }
     if (e == cudaSuccess) e = launch_mlp_net<FILMS, kNetProbe>(a, sm_count, stream);
     if (e == cudaSuccess) {

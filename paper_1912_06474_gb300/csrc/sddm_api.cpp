@@ -1796,7 +1796,7 @@ int sddm_glass_eval(sddm_ctx *ctx, uint32_t mat, int n, const float *cos_theta, 
         // the batch counts lie behind the error word, the two lists in scratch kept for the next call
         const size_t n_batch = ((size_t)n + 31) / 32;
         if (e == cudaSuccess) e = ctx->d_err.ensure(kErrBytes);
-        if (e == cudaSuccess && !a.raw) e = ctx->mlp_lists.ensure(8 * n_batch);
+        if (e == cudaSuccess && !a.raw && n > kMlpCheckRows) e = ctx->mlp_lists.ensure(8 * n_batch);
         if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_err.p, 0, kErrBytes, ctx->stream);
         a.err = ctx->d_err.as<int>();
         a.list_cnt = ctx->d_err.as<uint32_t>() + 4;

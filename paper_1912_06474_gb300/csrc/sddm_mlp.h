@@ -38,21 +38,28 @@ struct MlpRows {
     int *err;                         // device error word [4] (NULL: not reported); 2 = a wait ran out
     unsigned int *grid_err;           // mode 2: largest |dR|, |dT| as float bits [2]
     unsigned long long *rows;         // rows the network evaluated (NULL: not counted)
-    // unless raw: batches sorted by their probes, full ones from the front of
+    // where the probes come first: batches sorted by them, full ones from the front of
     // a list, short ones from its back; list_cnt[4] zero before the call
     uint32_t *list_pass, *list_fail;  // [list_cap]
     uint32_t *list_cnt;               // passed full, passed short, failed full, failed short
     uint32_t list_cap;                // at least the call's batches
     int test_timeout;                 // 1: CTA 0 issues no layer-1 MMA and waits 2^10 tries (failure-path test)
 };
+// Explicit rows up to which the network runs over every row and a warp per batch
+// checks it: two kernels instead of three, and no lists. A call of 2^10 / 2^17 / 2^18 /
+// 0.35 M / 0.5 M / 1 M rows takes 48 / 53 / 62 / 69 / 79 / 112 us so and 54 / 65 / 67 / 75 / 79 /
+// 103 with the probes first; coated glass 49 / 61 / 77 / 88 / 110 / 173 and 64 / 76 / 83 / 88 /
+// 100 / 137.
+constexpr int kMlpCheckRows = 1 << 18;
 // The attributes the network and training kernels are launched with, set on the
 // current device, where they hold (a device keeps its own). Every context calls it
 // before its first such launch.
 cudaError_t mlp_prepare_device();
-// raw: the network over every row (tensor cores). Otherwise the network over
-// one probe row per batch, then over the batches that passed, and the exact slab
-// over the others: three kernels on `stream`. With ev0 / ev1 given, they are
-// recorded around the network kernels.
+// raw: the network over every row (tensor cores). Up to kMlpCheckRows explicit rows
+// the check of their batches follows. Otherwise the network over one probe row per
+// batch, then over the batches that passed, and the exact slab over the others:
+// three kernels on `stream`. With ev0 / ev1 given, they are recorded around the
+// network kernels.
 cudaError_t launch_mlp_rows(const MlpRows &a, int sm_count, cudaStream_t stream, cudaEvent_t ev0 = nullptr,
                             cudaEvent_t ev1 = nullptr);
 // The exact slab over the same rows (no network).
