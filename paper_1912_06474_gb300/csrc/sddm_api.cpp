@@ -1528,7 +1528,7 @@ static int mlp_net_for(sddm_ctx *ctx, uint32_t mat, bool create, sddm_ctx::MlpNe
         id = (int)ctx->nets.size() - 1;
         sddm_ctx::MlpNet &n = *ctx->nets.back();
         if ((e = n.params.ensure(mlp_param_buffer_bytes())) || (e = n.m.ensure(kMlpParams * 4)) ||
-            (e = n.v.ensure(kMlpParams * 4)) || (e = ctx->mlp_lists.ensure((size_t)1 << 20)))   // lists of 2^22 rows
+            (e = n.v.ensure(kMlpParams * 4)))
             return cuda_fail(e, "surrogate: allocation");
         for (size_t m = 0; m < ctx->mats.size(); ++m)
             if (same_curves(ctx->mats[m], ctx->mats[mat]) && ctx->net_of_mat[m] < 0) ctx->net_of_mat[m] = id;
@@ -1760,6 +1760,9 @@ int sddm_set_profiling(sddm_ctx *ctx, int flags) {
     return SDDM_OK;
 }
 
+// Batch lists of sddm_glass_eval up to this size (2^28 rows) stay for the next call.
+static constexpr size_t kMlpListsKeep = (size_t)64 << 20;
+
 int sddm_glass_eval(sddm_ctx *ctx, uint32_t mat, int n, const float *cos_theta, const int32_t *bin, const float *s,
                     const float *thickness_m, float *R, float *T, int mode) {
     if (!ctx) return fail(SDDM_ERR_INVALID_ARG, "sddm_glass_eval: ctx is NULL");
@@ -1793,7 +1796,8 @@ int sddm_glass_eval(sddm_ctx *ctx, uint32_t mat, int n, const float *cos_theta, 
         int *const derr = static_cast<int *>(ctx->h_table.p);   // page-locked; no render is under way
         cudaError_t e = ctx->stage_busy ? cudaStreamSynchronize(ctx->stream) : cudaSuccess;
         ctx->stage_busy = false;
-        // the batch counts lie behind the error word, the two lists in scratch kept for the next call
+        // the batch counts lie behind the error word, the two lists in scratch that the next call
+        // finds again, unless it is large
         const size_t n_batch = ((size_t)n + 31) / 32;
         if (e == cudaSuccess) e = ctx->d_err.ensure(kErrBytes);
         if (e == cudaSuccess && !a.raw && n > kMlpCheckRows) e = ctx->mlp_lists.ensure(8 * n_batch);
@@ -1806,6 +1810,7 @@ int sddm_glass_eval(sddm_ctx *ctx, uint32_t mat, int n, const float *cos_theta, 
         if (e == cudaSuccess) e = launch_mlp_rows(a, ctx->sm_count, ctx->stream);
         if (e == cudaSuccess) e = cudaMemcpyAsync(derr, ctx->d_err.p, 4 * sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+        if (ctx->mlp_lists.bytes > kMlpListsKeep) ctx->mlp_lists.release();
         if (e != cudaSuccess) return cuda_fail(e, "sddm_glass_eval (surrogate)");
         if (derr[0] != 0)
             return fail(SDDM_ERR_TIMEOUT, "sddm_glass_eval: the surrogate's tensor-core evaluation did not complete");
