@@ -534,6 +534,7 @@ __device__ __forceinline__ Cx cx_sqrt(Cx z) {   // principal root
 
 // Up to kMaxFilms films per face.
 constexpr int kMaxFilms = SDDM_MAX_FILMS;
+constexpr int kDenseFilms = 3;   // films of a stack held in registers (glass_rt, DENSE)
 
 // Glass coated on both faces with the same stack of J thin films (outermost
 // first): each face is a coherent stack evaluated by its characteristic
@@ -639,10 +640,14 @@ static __device__ __noinline__ float2 coated_few(const DevScene &sc, int m, int 
 // R, T of glass material m at wavelength bin i: the bare absorbing slab, or
 // the coated slab when the material carries films (film k = k + s dk).
 // Kernels are instantiated with FILMS = false for scenes without coated glass,
-// which keeps the film code (and its call) out of them entirely. DENSE: in kernels
-// that evaluate rows of glass and nothing else, stacks of up to three films (the
-// usual ones) keep their matrices in registers instead of indexed local arrays (the
-// same bits): 262,147 rows of 1 / 2 / 3 films 29.7 / 33.4 / 38.3 -> 25.3 / 29.0 / 32.9 us a call.
+// which keeps the film code (and its call) out of them entirely. DENSE: for the dense
+// exact passes (k_glass_eval, k_slab_rows) over scenes whose stacks have at most
+// kDenseFilms films, which keep their matrices in registers instead of indexed local
+// arrays (the same bits). 2^22 rows of 1 / 2 / 3 films 140 / 197 / 257 -> 134 / 183 / 241 us;
+// a call of 262,147 rows, mostly launch and wait, 40 / 45 / 49 -> 37 / 41 / 45. Deeper
+// stacks have kernels of their own: sharing one with the register variants takes it
+// from 48 to 80 registers, 4 / 6 / 10 films 320 / 440 / 681 us but 356 / 496 / 789.
+// Three is what the electrochromic panes here have; more in registers was not tried.
 template <bool FILMS = true, bool DENSE = false>
 __device__ __forceinline__ void glass_rt(const DevScene &sc, int m, int i, float c, float s, float thick, float &R,
                                          float &T) {
@@ -656,22 +661,22 @@ __device__ __forceinline__ void glass_rt(const DevScene &sc, int m, int i, float
             slab_RT(c, __ldg(sc.lam + i), __ldg(sc.mat_a + k), alpha, thick, R, T);
             return;
         }
-        if (DENSE && J <= 3) {
+        if constexpr (DENSE) {
             const float2 rt = J == 1   ? coated_few<1>(sc, m, i, c, s, alpha, thick)
                               : J == 2 ? coated_few<2>(sc, m, i, c, s, alpha, thick)
-                                       : coated_few<3>(sc, m, i, c, s, alpha, thick);
+                                       : coated_few<kDenseFilms>(sc, m, i, c, s, alpha, thick);
             R = rt.x;
             T = rt.y;
-            return;
+        } else {
+            float nf[kMaxFilms], kf[kMaxFilms], tf[kMaxFilms];
+            for (int j = 0; j < J; ++j) {
+                const size_t f = ((size_t)m * kMaxFilms + j) * sc.L + i;
+                nf[j] = __ldg(sc.film_n + f);
+                kf[j] = __ldg(sc.film_k + f) + s * __ldg(sc.film_dk + f);
+                tf[j] = __ldg(sc.film_t + (size_t)m * kMaxFilms + j);
+            }
+            coated_RT(c, __ldg(sc.lam + i), __ldg(sc.mat_a + k), alpha, thick, J, nf, kf, tf, R, T);
         }
-        float nf[kMaxFilms], kf[kMaxFilms], tf[kMaxFilms];
-        for (int j = 0; j < J; ++j) {
-            const size_t f = ((size_t)m * kMaxFilms + j) * sc.L + i;
-            nf[j] = __ldg(sc.film_n + f);
-            kf[j] = __ldg(sc.film_k + f) + s * __ldg(sc.film_dk + f);
-            tf[j] = __ldg(sc.film_t + (size_t)m * kMaxFilms + j);
-        }
-        coated_RT(c, __ldg(sc.lam + i), __ldg(sc.mat_a + k), alpha, thick, J, nf, kf, tf, R, T);
     }
 }
 

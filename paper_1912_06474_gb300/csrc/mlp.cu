@@ -763,14 +763,14 @@ __global__ void __launch_bounds__(256) k_mlp_fallback(MlpRows a) {
 
 // The exact slab for the same query rows, one thread per (query, bin): the
 // glass evaluations of a bounce as one dense, divergence-free pass.
-template <bool FILMS>
-__global__ void __launch_bounds__(256) k_slab_rows(MlpRows a) {
+template <bool FILMS, bool DENSE>
+__global__ void __launch_bounds__(256, 3) k_slab_rows(MlpRows a) {
     const int64_t total = mlp_total_rows(a);
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < total; r += stride) {
         RowIn in;
         row_input(a, r, total, in);
-        store_row(a, r, in, exact_row<FILMS, true>(a, in));
+        store_row(a, r, in, exact_row<FILMS, DENSE>(a, in));
     }
 }
 
@@ -1286,11 +1286,12 @@ cudaError_t launch_mlp_rows(const MlpRows &a, int sm_count, cudaStream_t stream,
 }
 
 cudaError_t launch_slab_rows(const MlpRows &a, int sm_count, cudaStream_t stream) {
-    if (a.sc.mat_nfilm)
-        k_slab_rows<true><<<sm_count * resident_per_sm(k_slab_rows<true>, 256, 8), 256, 0, stream>>>(a);
-    else
-        k_slab_rows<false><<<sm_count * resident_per_sm(k_slab_rows<false>, 256, 8), 256, 0, stream>>>(a);
-    return cudaGetLastError();
+    auto launch = [&](auto kernel) {
+        kernel<<<sm_count * resident_per_sm(kernel, 256, 8), 256, 0, stream>>>(a);
+        return cudaGetLastError();
+    };
+    if (!a.sc.mat_nfilm) return launch(k_slab_rows<false, false>);
+    return a.sc.max_films <= kDenseFilms ? launch(k_slab_rows<true, true>) : launch(k_slab_rows<true, false>);
 }
 
 cudaError_t launch_mlp_train_tile(const MlpTrainArgs &a, cudaStream_t stream) {

@@ -62,7 +62,7 @@ cudaError_t launch_philox(int n, const uint32_t *ctr, uint32_t k0, uint32_t k1, 
     return cudaGetLastError();
 }
 
-template <bool FILMS>
+template <bool FILMS, bool DENSE>
 __global__ void __launch_bounds__(128) k_glass_eval(const __grid_constant__ DevScene sc, uint32_t mat, int n, const float *cos_t, const int32_t *bin,
                              const float *s, const float *thick, float *R, float *T) {
     int q = blockIdx.x * blockDim.x + threadIdx.x;
@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(128) k_glass_eval(const __grid_constant__ DevS
     int i = bin[q];
     i = i < 0 ? 0 : (i >= L ? L - 1 : i);
     float r_, t_;
-    glass_rt<FILMS, true>(sc, (int)mat, i, cos_t[q], s[q], thick[q], r_, t_);
+    glass_rt<FILMS, DENSE>(sc, (int)mat, i, cos_t[q], s[q], thick[q], r_, t_);
     R[q] = r_;
     T[q] = t_;
 }
@@ -114,10 +114,12 @@ cudaError_t launch_blend(int64_t n, float a, float b, const float *in, float *ou
 cudaError_t launch_glass_eval(const DevScene &sc, uint32_t mat, int n, const float *cos_t, const int32_t *bin,
                               const float *s, const float *thick, float *R, float *T, cudaStream_t stream) {
     if (n <= 0) return cudaSuccess;
-    if (sc.mat_nfilm)
-        k_glass_eval<true><<<(n + 127) / 128, 128, 0, stream>>>(sc, mat, n, cos_t, bin, s, thick, R, T);
+    if (!sc.mat_nfilm)
+        k_glass_eval<false, false><<<(n + 127) / 128, 128, 0, stream>>>(sc, mat, n, cos_t, bin, s, thick, R, T);
+    else if (sc.max_films <= kDenseFilms)
+        k_glass_eval<true, true><<<(n + 127) / 128, 128, 0, stream>>>(sc, mat, n, cos_t, bin, s, thick, R, T);
     else
-        k_glass_eval<false><<<(n + 127) / 128, 128, 0, stream>>>(sc, mat, n, cos_t, bin, s, thick, R, T);
+        k_glass_eval<true, false><<<(n + 127) / 128, 128, 0, stream>>>(sc, mat, n, cos_t, bin, s, thick, R, T);
     return cudaGetLastError();
 }
 

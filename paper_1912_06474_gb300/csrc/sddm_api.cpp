@@ -650,6 +650,8 @@ int sddm_build(sddm_ctx *ctx, const sddm_build_opts *opts) {
     d.mat_c = ctx->d_c.as<float>();
     d.mat_thick = ctx->d_thick.as<float>();
     d.mat_nfilm = any_film ? ctx->d_nfilm.as<int>() : nullptr;
+    d.max_films = 0;
+    for (int m = 0; m < M; ++m) d.max_films = std::max(d.max_films, ctx->mats[m].n_film);
     d.film_n = any_film ? ctx->d_film_n.as<float>() : nullptr;
     d.film_k = any_film ? ctx->d_film_k.as<float>() : nullptr;
     d.film_dk = any_film ? ctx->d_film_dk.as<float>() : nullptr;

@@ -56,6 +56,7 @@ struct DevScene {
     const float *mat_thick;   // [n_mat]
     // thin-film coatings of glass materials (both faces; NULL when no material has one)
     const int *mat_nfilm;     // [n_mat] films per face, 0..SDDM_MAX_FILMS
+    int max_films;            // the most of them
     const float *film_n;      // [n_mat][SDDM_MAX_FILMS][L] real index
     const float *film_k;      // [n_mat][SDDM_MAX_FILMS][L] extinction at s = 0
     const float *film_dk;     // [n_mat][SDDM_MAX_FILMS][L] extinction added at s = 1
