@@ -816,7 +816,7 @@ __device__ __forceinline__ Float4 ld4(const float4 *p) {
 // a sum over bins rounds its products and its result and nothing between. Root mean
 // square error against 64 bits, 8 / 16 / 41 / 81 bins, of sums that differ in this alone:
 // 4.28 / 3.62 / 3.18 / 2.70e-8 with plain sums inside the chunk and compensated ones
-// between chunks, 3.11 / 2.58 / 2.20 / 2.17e-8 so (3.09 / 2.57 / 2.23 / 2.14e-8 is what
+// between chunks, 3.08 / 2.59 / 2.18 / 2.16e-8 so (3.09 / 2.57 / 2.23 / 2.14e-8 is what
 // one rounding of products and result makes). It costs 1 % of a hotel room render and 2 to
 // 9 % of a tiny room's, whose time is mostly this pass.
 struct ChunkXyz {
@@ -825,14 +825,15 @@ struct ChunkXyz {
 };
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }
 __device__ __forceinline__ Kahan weigh4(const Float4 &e, const Float4 &w) {
-    // bins 0, 1 and 2, 3 side by side (two operations an instruction), then the two sums
+    // bins 0, 2 and 1, 3 side by side (two operations an instruction); what adding the
+    // second pair rounds off, again with a fused product; then the two sums
+    const float2 e2 = make_float2(e.v[2], e.v[3]), w2 = make_float2(w.v[2], w.v[3]);
     const float2 p = __fmul2_rn(make_float2(e.v[0], e.v[1]), make_float2(w.v[0], w.v[1]));
-    const float2 q = __fmul2_rn(make_float2(e.v[2], e.v[3]), make_float2(w.v[2], w.v[3]));
-    const float2 t = __fadd2_rn(p, q), b = sub2(t, p), lost = __fadd2_rn(sub2(p, sub2(t, b)), sub2(q, b));
-    const float s = t.x + t.y, c = s - t.x;
+    const float2 t = __ffma2_rn(e2, w2, p), r = __ffma2_rn(e2, w2, sub2(p, t));
+    const float s = t.x + t.y, b = s - t.x;
     Kahan k;
     k.s = s;
-    k.c = -(((t.x - (s - c)) + (t.y - c)) + (lost.x + lost.y));
+    k.c = -(((t.x - (s - b)) + (t.y - b)) + (r.x + r.y));
     return k;
 }
 __device__ __forceinline__ ChunkXyz chunk_xyz(const Float4 &e, const float4 *w, int n_chunk) {
