@@ -120,14 +120,14 @@ struct PinnedBuf {
     }
     cudaError_t ensure(size_t n) {
         if (n <= bytes) return cudaSuccess;
-        if (p) cudaFreeHost(p);
-        p = nullptr;
-        bytes = 0;
-        const cudaError_t e = cudaHostAlloc(&p, n, cudaHostAllocDefault);
+        void *q = nullptr;
+        const cudaError_t e = cudaHostAlloc(&q, n, cudaHostAllocDefault);
         if (e != cudaSuccess) {
-            p = nullptr;
-            return e;
+            cudaGetLastError();
+            return e;   // what there was stays
         }
+        if (p) cudaFreeHost(p);
+        p = q;
         bytes = n;
         return cudaSuccess;
     }

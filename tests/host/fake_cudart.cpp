@@ -24,7 +24,7 @@ struct Call {
     cudaStream_t stream;
 } g_call;
 long g_launches = 0, g_optin = 0;
-size_t g_most = (size_t)-1;   // larger device allocations fail
+size_t g_most = (size_t)-1;   // larger device and page-locked allocations fail
 
 bool wrong_device(const void *p) {
     auto it = g_mem.upper_bound(static_cast<const char *>(p));
@@ -133,7 +133,9 @@ cudaError_t cudaFree(void *p) {
     std::free(p);
     return cudaSuccess;
 }
-cudaError_t cudaHostAlloc(void **p, size_t n, unsigned) { return alloc(p, n); }
+cudaError_t cudaHostAlloc(void **p, size_t n, unsigned) {
+    return n > g_most ? (g_last = cudaErrorMemoryAllocation) : alloc(p, n);
+}
 cudaError_t cudaFreeHost(void *p) {
     std::free(p);
     return cudaSuccess;

@@ -84,6 +84,23 @@ elif what == "weights":
             render(*both[1 - k % 2])
             ctx.mlp_get_weights(sc.glass_materials()[0])
             learned(sc, ctx)
+elif what == "no memory":
+    sc, ctx = context(0, 8)
+    ctx.mlp_set_weights(sc.glass_materials()[0], np.zeros(sddm.MLP_PARAMS, np.float32))
+    learned(sc, ctx)
+    spec = scenes.RenderSpec(2, 1, 1, 1, seed=1, camera=sc.camera)
+    lib.fake_limit_alloc(ctypes.c_size_t(1 << 16))
+    try:
+        out = np.zeros((1, 2, 3), np.float32)
+        arr, keep = ctx._descs([spec] * 2000, "megakernel", "exact", [out.ctypes.data] * 2000, None, None)
+        sddm._check(sddm.lib.sddm_render(ctx._h, arr, 2000, ctypes.byref(sddm.Stats())))
+        sys.exit("the table of 2000 renders fits?")
+    except sddm.SddmError:
+        pass
+    n = 100
+    rows = [torch.rand(n), torch.zeros(n, dtype=torch.int32), torch.rand(n), torch.full((n,), 0.004)]
+    ctx.glass_eval(sc.glass_materials()[0], *rows, mode="mlp")     # what fits still works
+    ctx.render_host([spec], [np.zeros((1, 2, 3), np.float32)], method="megakernel")
 elif what == "training":
     for sc, ctx in both:
         ctx.mlp_train(sc.glass_materials()[0], samples=256, steps=2, batch=64)
@@ -91,7 +108,7 @@ elif what == "training":
     for sc, ctx in (context(0, 16), context(1, 16)):   # a gradient is a context's first learned call
         ctx.mlp_grad(torch.zeros(100, 4), torch.zeros(100, 2), torch.zeros(sddm.MLP_PARAMS))
 assert lib.fake_launches() > 20
-assert lib.fake_optin_launches() > 0
+assert lib.fake_optin_launches() > 0, "no launch above 48 KiB"
 """
 
 
@@ -111,7 +128,7 @@ def fake_library(tmp_path_factory):
     return lib
 
 
-@pytest.mark.parametrize("what", ["renders", "photons", "weights", "training"])
+@pytest.mark.parametrize("what", ["renders", "photons", "weights", "no memory", "training"])
 def test_second_device(fake_library, what):
     r = subprocess.run([sys.executable, "-c", CALLS, fake_library, what], cwd=ROOT, capture_output=True, text=True,
                        timeout=300)
