@@ -545,7 +545,12 @@ static_assert(sizeof(SpecRec) == 64, "four 16-byte loads");
 constexpr int kSrResolve = 1, kSrEmit = 2, kSrLoad = 4, kSrStore = 8, kSrRow = 16, kSrConductor = 32, kSrGlass = 64,
               kSrDirect = 128;   // a glass evaluation the query list had no room for
 constexpr int kSpecThreads = 128;
-constexpr int kSpecItems = 128;  // chunks a warp works through between two sums (two records of 256 bins; 24 bytes each)
+// Chunks a warp works through between two sums (three records of 256 bins), 24 bytes of
+// shared memory each, and resident blocks: 128 and 8 / 192 and 8 / 192 and 7 / 192 and 6 take
+// 3780 / 3756 / 3746 / 3745 us for six tiny rooms (learned glass), 938 / 948 / 934 / 923 for the
+// coated one, 16.08 / 16.11 / 16.11 / 16.22 ms for the hotel room, 57.6 / 57.5 / 57.6 / 57.7 for
+// the facade room.
+constexpr int kSpecItems = 192;
 
 // One chunk of a record: the XYZ it adds (bins past L have a zero colour
 // matching function) to *s and *c, the row's four bins updated. DIRECT also evaluates the
@@ -653,7 +658,7 @@ static __device__ __noinline__ void spec_items_direct(const KArgs &a, const Spec
 }
 
 #ifndef SDDM_SHS_MINB
-#define SDDM_SHS_MINB 8      // resident 128-thread blocks per SM the spectral pass is compiled for
+#define SDDM_SHS_MINB 7      // resident 128-thread blocks per SM the spectral pass is compiled for
 #endif
 template <bool FILMS>
 __global__ void __launch_bounds__(kSpecThreads, SDDM_SHS_MINB) k_shade_spectral(const __grid_constant__ KArgs a) {
