@@ -1499,6 +1499,9 @@ int sddm_autotune(sddm_ctx *ctx, const sddm_render_desc *d, int n, sddm_build_op
 }
 
 // ---------------------------------------------------- learned glass surrogate
+// Batch lists of sddm_glass_eval up to this size (2^28 rows) stay for the next call.
+static constexpr size_t kMlpListsKeep = (size_t)64 << 20;
+
 static bool same_curves(const Material &a, const Material &b) {
     if (!(a.kind == kGlass && b.kind == kGlass && a.a == b.a && a.b == b.b && a.c == b.c && a.n_film == b.n_film &&
           a.film_n == b.film_n && a.film_k == b.film_k && a.film_dk == b.film_dk))
@@ -1562,8 +1565,10 @@ int sddm_mlp_train(sddm_ctx *ctx, uint32_t mat, const sddm_mlp_train_opts *opts,
     cudaError_t e;
     cudaStream_t s = ctx->stream;
     const int n_cta = o.batch / kMlpRowsPerCta;
+    // with the training's own buffers, the batch lists of a table of as many rows as there are samples
+    const size_t list_bytes = std::min<size_t>(8 * (((size_t)o.samples + 31) / 32), kMlpListsKeep);
     if ((e = ctx->mlp_grad_cta.ensure((size_t)n_cta * kMlpParams * 4)) || (e = ctx->mlp_loss_cta.ensure(n_cta * 4)) ||
-        (e = ctx->mlp_scalar.ensure(64)) || (e = ctx->mlp_X.ensure((size_t)o.samples * 16)) ||
+        (e = ctx->mlp_lists.ensure(list_bytes)) || (e = ctx->mlp_scalar.ensure(64)) || (e = ctx->mlp_X.ensure((size_t)o.samples * 16)) ||
         (e = ctx->mlp_Y.ensure((size_t)o.samples * 8)))
         return e == cudaErrorMemoryAllocation ? fail(SDDM_ERR_OOM, "sddm_mlp_train: allocation failed")
                                               : cuda_fail(e, "sddm_mlp_train: allocation");
@@ -1761,9 +1766,6 @@ int sddm_set_profiling(sddm_ctx *ctx, int flags) {
     ctx->graphs_enabled = flags == 0;   // events inside a replayed graph give no elapsed times
     return SDDM_OK;
 }
-
-// Batch lists of sddm_glass_eval up to this size (2^28 rows) stay for the next call.
-static constexpr size_t kMlpListsKeep = (size_t)64 << 20;
 
 int sddm_glass_eval(sddm_ctx *ctx, uint32_t mat, int n, const float *cos_theta, const int32_t *bin, const float *s,
                     const float *thickness_m, float *R, float *T, int mode) {
