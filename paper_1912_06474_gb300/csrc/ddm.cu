@@ -623,9 +623,7 @@ __device__ __forceinline__ void spec_chunk(const KArgs &a, const SpecRec &rec, i
         for (int u = 0; u < 4; ++u) e.v[u] = t.v[u] * le.v[u];
     }
     if (xf & (kSrResolve | kSrEmit)) {
-        const ChunkXyz v = chunk_xyz(e, tab + 2 * sc.n_mat * n_chunk, n_chunk);
-        *s = v.s;
-        *c = v.c;
+        chunk_xyz<3>(e, tab + 2 * sc.n_mat * n_chunk, n_chunk, s, c);
     }
     if (xf & kSrStore)
         reinterpret_cast<float4 *>(ps.T)[(size_t)q * n_chunk + ch] = make_float4(t.v[0], t.v[1], t.v[2], t.v[3]);
@@ -774,11 +772,12 @@ __global__ void __launch_bounds__(kSpecThreads, SDDM_SHS_MINB) k_shade_spectral(
             for (int i = lane; i < 3 * nr; i += 32) {
                 const int j = i / 3, k = i - 3 * j;
                 if (!(rec[r0 + j].flags & (kSrResolve | kSrEmit))) continue;
-                const Kahan sum = sum_chunks<4>(part + j * n_chunk, lost + j * n_chunk, n_chunk, k);
                 float *const acc = ps.acc + k * np + rec[r0 + j].q;
-                Kahan to;
+                Kahan to;   // under way while the chunks are added
                 to.s = acc[0];
-                to.c = acc[3 * np] + sum.c;   // what the chunk sums lost goes on to the path's sum
+                to.c = acc[3 * np];
+                const Kahan sum = sum_chunks<4>(part + j * n_chunk, lost + j * n_chunk, n_chunk, k);
+                to.c += sum.c;   // what the chunk sums lost goes on to the path's sum
                 to.add(sum.s);
                 acc[0] = to.s;
                 acc[3 * np] = to.c;

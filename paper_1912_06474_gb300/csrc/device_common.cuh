@@ -817,12 +817,9 @@ __device__ __forceinline__ Float4 ld4(const float4 *p) {
 // square error against 64 bits, 8 / 16 / 41 / 81 bins, of sums that differ in this alone:
 // 4.28 / 3.62 / 3.18 / 2.70e-8 with plain sums inside the chunk and compensated ones
 // between chunks, 3.08 / 2.59 / 2.18 / 2.16e-8 so (3.09 / 2.57 / 2.23 / 2.14e-8 is what
-// one rounding of products and result makes). It costs 1 % of a hotel room render and 2 to
-// 9 % of a tiny room's, whose time is mostly this pass.
-struct ChunkXyz {
-    float4 s;    // sums of x, y, z; what x lost (true sum s - c)
-    float2 c;    // what y and z lost
-};
+// one rounding of products and result makes). It costs 1 % of a hotel or facade room
+// render, up to 3 % of a tiny room's by the DDM and 7 % by the plain method, whose time is
+// mostly this.
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }
 __device__ __forceinline__ Kahan weigh4(const Float4 &e, const Float4 &w) {
     // bins 0, 2 and 1, 3 side by side (two operations an instruction); what adding the
@@ -836,9 +833,18 @@ __device__ __forceinline__ Kahan weigh4(const Float4 &e, const Float4 &w) {
     k.c = -(((t.x - (s - b)) + (t.y - b)) + (r.x + r.y));
     return k;
 }
-__device__ __forceinline__ ChunkXyz chunk_xyz(const Float4 &e, const float4 *w, int n_chunk) {
-    const Kahan x = weigh4(e, ld4(w)), y = weigh4(e, ld4(w + n_chunk)), z = weigh4(e, ld4(w + 2 * n_chunk));
-    return ChunkXyz{make_float4(x.s, y.s, z.s, x.c), make_float2(y.c, z.c)};
+// A chunk's sums of x, y, z and what x lost go to *s, what y and z lost to *c (true sums
+// s - c). UNROLL 1 keeps the code short where the instruction cache bounds the kernel.
+template <int UNROLL>
+__device__ __forceinline__ void chunk_xyz(const Float4 &e, const float4 *w, int n_chunk, float4 *s, float2 *c) {
+    float *ps = reinterpret_cast<float *>(s), *pc = ps + 3;
+#pragma unroll UNROLL
+    for (int k = 0; k < 3; ++k, w += n_chunk) {
+        const Kahan v = weigh4(e, ld4(w));
+        ps[k] = v.s;
+        *pc = v.c;
+        pc = reinterpret_cast<float *>(c) + k;
+    }
 }
 // Component k of the sum of n chunks, in bin order.
 template <int UNROLL>

@@ -349,9 +349,7 @@ __device__ __forceinline__ void mega_chunk(const MegaArgs &a, const MegaRec &m, 
     }
     if (xf & (kMrDiffuse | kMrConductor | kMrGlass)) row[ch] = make_float4(t.v[0], t.v[1], t.v[2], t.v[3]);
     if (xf & (kMrEmit | kMrResolve)) {
-        const ChunkXyz v = chunk_xyz(e, tab + 2 * sc.n_mat * n_chunk, n_chunk);
-        *s = v.s;
-        *c = v.c;
+        chunk_xyz<1>(e, tab + 2 * sc.n_mat * n_chunk, n_chunk, s, c);
     }
 }
 
