@@ -528,7 +528,7 @@ __global__ void __launch_bounds__(256) k_glass_gather(KArgs a) {
 // throughput is 1) nor written once the path has ended.
 // All bounces of the hotel room (512 x 512 x 16 spp, 41 bins): 1.9 ms, against
 // 4.5 ms with a thread walking its path's bins down a column of an [L][paths]
-// array; of a facade room (960 x 540 x 4 spp, 81 bins) 4.3 ms against 9.7. It is
+// array; of a facade room (960 x 540 x 4 spp, 81 bins) 4.5 ms against 9.7. It is
 // now bound by issue (60 % of the slots) and by the L1 it shares with the table rows.
 struct SpecRec {
     int q, flags;         // path slot; kSr* bits

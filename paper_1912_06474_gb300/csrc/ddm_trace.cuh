@@ -88,9 +88,10 @@ __device__ __forceinline__ void block_count3(unsigned long long *c0, unsigned lo
 //  * a lane carries only what the traversal itself uses, and triangle records are
 //    read in the ray's axis order (make_ray, load_tri) instead of permuted by
 //    selects: 12.7 -> 12.1 ms;
-//  * 7 resident blocks of 128 threads (72 registers, few spills): 11.4 ms, against
-//    12.1 with 8 (64 registers) and 12.1 with 6 (80).
-// 13.2 ms before all of it; facade room (480 x 270 x 4 spp, 81 bins) 7.4 -> 6.7 ms.
+//  * 7 resident blocks of 128 threads (72 registers, no spills): 11.4 ms, against
+//    12.1 with 8 (64 registers) and 12.1 with 6 (80);
+//  * one triangle test for both query kinds (trav_round): 11.0 ms.
+// 13.2 ms before all of it; facade room (480 x 270 x 4 spp, 81 bins) 7.4 -> 6.4 ms.
 #ifndef SDDM_TRACE_STEPS
 #define SDDM_TRACE_STEPS 64   // interior steps per round at most
 #endif

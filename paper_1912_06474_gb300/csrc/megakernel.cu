@@ -232,8 +232,8 @@ __global__ void __launch_bounds__(128) k_megakernel_pm(MegaArgs a) {
 //    leaves a record (emission, resolved shadow ray, weight), the rows of bins
 //    are dealt out to the lanes in chunks of four, as in the DDM's spectral pass,
 //    with a throughput row per lane, in shared memory while there are few bins.
-// Hotel room, 512 x 512 x 4 spp, 41 bins: 10.2 -> 6.1 ms; tiny room, 400 x 400 x 6
-// spp, depth 6: 4.4 -> 3.4 ms; with a coated pane, 200 x 200 x 3 spp: 2.1 -> 0.96.
+// Hotel room, 512 x 512 x 4 spp, 41 bins: 10.2 -> 5.9 ms; tiny room, 400 x 400 x 6
+// spp, depth 6: 4.4 -> 3.7 ms; with a coated pane, 200 x 200 x 3 spp: 2.1 -> 1.04.
 // The loop holds all that a path meets, some 4000 instructions, and the
 // instruction cache bounds it on small scenes (2.7 of 9 stall cycles per
 // instruction): not unrolling its loops took the tiny room from 4.4 to 3.5 ms,
@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(128) k_megakernel_pm(MegaArgs a) {
 // (warp_branch_proxy). Waiting lanes that stop the warp, 12 / 16 / 20 / 24 (hotel):
 // 8.0 (early version) / 6.04 / 6.06 / 6.25 ms, tiny room - / 3.54 / 3.41 / 3.35;
 // resident blocks 8 / 9 / 10 / 12: 6.0 / 6.3 / 5.9 / 6.4, tiny room 3.5 / 3.9 /
-// 3.9 / 4.7.
+// 3.9 / 4.7. (These choices were measured while the sums inside a chunk were plain ones.)
 struct __align__(16) MegaRec {
     float G, pcos, pw;             // shadow ray's geometry factor; |cos| and branch weight at this vertex
     int flags;                     // kMr* bits, 0 = nothing to do

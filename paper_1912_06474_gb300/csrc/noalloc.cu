@@ -9,7 +9,8 @@
 // sddm_render grows its scratch buffers (per-sample results, counters, render
 // tables) with cudaMalloc on demand; this entry point instead keeps all of
 // that scratch in one file-scope device array of fixed size, so a call
-// allocates nothing.
+// allocates nothing. (Above 44 bins the kernel's throughput rows lie in memory
+// that sddm_build allocated for the context, or in shared memory.)
 //
 // The array is 16 MiB and lives on every GPU that loads the library until the
 // process exits. Its first 8 KiB hold the counters, the error word, the render
