@@ -529,7 +529,8 @@ __global__ void __launch_bounds__(256) k_glass_gather(KArgs a) {
 // All bounces of the hotel room (512 x 512 x 16 spp, 41 bins): 1.9 ms, against
 // 4.5 ms with a thread walking its path's bins down a column of an [L][paths]
 // array; of a facade room (960 x 540 x 4 spp, 81 bins) 4.5 ms against 9.7. It is
-// now bound by issue (60 % of the slots) and by the L1 it shares with the table rows.
+// now bound by issue and load latency (51 % of the slots at seven blocks) and by the L1 it
+// shares with the table rows.
 struct SpecRec {
     int q, flags;         // path slot; kSr* bits
     float G;              // geometry factor of the shadow ray
